@@ -452,10 +452,20 @@ def bounds(w, esize, upd, hbm_bytes, seconds, peaks):
 
 
 def roofline(w, kern, peaks, esize, nvars):
-    """Roofline of the dominant swept kernel (the octahedron): its algorithmic
+    """Roofline of the dominant kernel (the octahedron, or the marching form's one
+    kernel, whose FP64 heat runs on the integer units and may pass the FP64
+    pipe's bound): its algorithmic
     work per launch over its CUDA-event launch time against the slowest of the
     HBM, FP64, FP32 and shared-memory bounds; the bridge's beside it."""
     n, N = w.tile, w.grid
+    launches, ms = kern.get("march", (0, 0.0))
+    if launches:                       # the marching form: every step in one launch
+        upd = N * N * w.nsteps // launches
+        hbm_bytes = 2 * N * N * nvars * esize // launches
+        out = {"kernel": "march", "avg_launch_ms": ms / launches, "updates_per_launch": upd,
+               "hbm_bytes_per_launch": hbm_bytes, "traffic": None, "traffic_source": None}
+        out.update(bounds(w, esize, upd, hbm_bytes, ms / launches * 1e-3, peaks))
+        return out
     tiles = (N // n) ** 2
     launches, ms = kern["octahedron"]
     avg_ms = ms / max(1, launches)
@@ -589,7 +599,8 @@ def main():
     with torch.cuda.stream(stream):
         sw.set_state(state_dev)
         sw.advance(w.nsteps, mode="swept")
-    kern = {k: sw.kernel_stats(k) for k in ("up", "bridge", "octahedron", "down", "naive")}
+    kern = {k: sw.kernel_stats(k) for k in ("up", "bridge", "octahedron", "down", "naive",
+                                               "march")}
     sw.set_timing(False)
     rf = roofline(w, kern, peaks, esize, nvars)
 

@@ -236,7 +236,8 @@ int swept2d_set_tuning(swept2d_t *h, int threads, int stage);
 #define SWEPT2D_K_OCTAHEDRON  3
 #define SWEPT2D_K_DOWN        4
 #define SWEPT2D_K_REDUCE      5
-#define SWEPT2D_K_COUNT       6
+#define SWEPT2D_K_MARCH       6   /* marching form: every step of an advance in one launch */
+#define SWEPT2D_K_COUNT       7
 int swept2d_set_timing(swept2d_t *h, int on);
 
 /* Per-item trace of the persistent form (a measurement aid; no counterpart in

@@ -13,13 +13,6 @@
 
 namespace swept {
 
-struct GridDesc {
-    Geom G;                 // the grid's geometry (tile side n of its class)
-    long long state_off;    // first element of the grid's state in the pooled state
-    long long panel_off;    // first element of the grid's panel slots in each pool
-    double c[8];            // the point update's constants for this grid (Euler's
-                            // depend on the grid's own state and spacing)
-};
 // Tile and block tables hold (grid index, tile or block index within the grid).
 
 // NC > 0: every grid of the launch's class has tile side NC (see fixed_tile).

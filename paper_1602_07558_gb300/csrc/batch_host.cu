@@ -18,6 +18,7 @@
 
 #include "../../include/swept2d.h"
 #include "batch.cuh"
+#include "march_table.cuh"
 
 using swept::BatchTable;
 using swept::GridDesc;
@@ -55,6 +56,13 @@ struct swept2d_batch {
     std::vector<GridDesc> grids;
     GridDesc *d_grids = nullptr;
     std::vector<BatchClass> classes;
+    // the update's marching form (nullptr: none), its shape, tile table (grid,
+    // tile) and counters (one per tile, the item counter)
+    const swept::MarchTable *mt = nullptr;
+    int mshape = 0;
+    std::vector<int2> mtiles;
+    int2 *d_mtiles = nullptr;
+    int *msched = nullptr;
     std::vector<int2> all_blocks;
     int2 *d_all_blocks = nullptr;
     void *state = nullptr, *state2 = nullptr, *up = nullptr, *br = nullptr;
@@ -95,6 +103,14 @@ const BatchTable *batch_table(int op, int dtype) {
     return nullptr;
 }
 
+const swept::MarchTable *batch_march(int op, int dtype) {
+    if (op == SWEPT2D_OP_HEAT) return swept::marchtable_heat();
+    if (op == SWEPT2D_OP_HEAT_KAHAN)
+        return dtype == SWEPT2D_F32 ? swept::marchtable_heat_kahan_f32()
+                                    : swept::marchtable_heat_kahan_bf16();
+    return nullptr;
+}
+
 void batch_free(swept2d_batch *b) {
     for (auto &c : b->classes) {
         if (c.d_tiles) cudaFree(c.d_tiles);
@@ -102,7 +118,7 @@ void batch_free(swept2d_batch *b) {
         if (c.d_sched) cudaFree(c.d_sched);
     }
     for (void *p : {(void *)b->d_grids, (void *)b->d_all_blocks, b->state, b->state2, b->up, b->br,
-                    (void *)b->errword, (void *)b->d_amax})
+                    (void *)b->errword, (void *)b->d_amax, (void *)b->d_mtiles, (void *)b->msched})
         if (p) cudaFree(p);
     for (auto &g : b->graphs) {
         cudaGraphExecDestroy(g.exec);
@@ -165,6 +181,21 @@ int batch_run(swept2d_batch *b, long long total, int mode) {
         if (rc) return rc;
         b->state = cur;
         b->state2 = other;
+        b->substeps += total;
+        return SWEPT2D_OK;
+    }
+    if (b->mt) {
+        if (total == 0) return SWEPT2D_OK;
+        void *out = b->state;
+        long long made = 0;
+        int rc = blaunch(b, "batched marching kernel", [&] {
+            return b->mt->many(b->mshape, b->d_grids, b->d_mtiles, (int)b->mtiles.size(),
+                               b->grids[0].c, b->state, b->state2, b->state, b->msched,
+                               total, b->errword, &out, &made, b->stream);
+        });
+        if (rc) return rc;
+        b->launches += made - 1;
+        if (out != b->state) std::swap(b->state, b->state2);
         b->substeps += total;
         return SWEPT2D_OK;
     }
@@ -365,6 +396,8 @@ int swept2d_batch_create(swept2d_batch_t **out, int count, const int *nx, const 
         b->wavespeed.assign(count, 0.0);
         b->dt.assign(count, 0.0);
     }
+    b->mt = batch_march(op, dtype);
+    if (b->mt) b->mshape = b->mt->shape(nx, ny, count);
     // grids, classes (by tile side), pooled offsets
     long long soff = 0, poff = 0;
     for (int i = 0; i < count; ++i) {
@@ -376,6 +409,10 @@ int swept2d_batch_create(swept2d_batch_t **out, int count, const int *nx, const 
         gd.G.T = n ? nx[i] / n : 0;
         gd.G.Q = n ? ny[i] / n : 0;
         gd.G.PS = n ? swept::panel_stride(n) : 0;
+        if (b->mt) {
+            gd.m = b->mt->cut(b->mshape, nx[i], ny[i]);
+            for (int t = 0; t < gd.m.bx * gd.m.by; ++t) b->mtiles.push_back(make_int2(i, t));
+        }
         gd.state_off = soff;
         gd.panel_off = poff;
         for (int k = 0; k < 8; ++k) gd.c[k] = b->consts[k];   // Euler's: at set_state
@@ -411,7 +448,10 @@ int swept2d_batch_create(swept2d_batch_t **out, int count, const int *nx, const 
         return cudaMemcpy(*dst, vec.data(), vec.size() * sizeof(T), cudaMemcpyHostToDevice);
     };
     if ((e = dev_copy(&b->d_grids, b->grids)) != cudaSuccess ||
-        (e = dev_copy(&b->d_all_blocks, b->all_blocks)) != cudaSuccess)
+        (e = dev_copy(&b->d_all_blocks, b->all_blocks)) != cudaSuccess ||
+        (e = dev_copy(&b->d_mtiles, b->mtiles)) != cudaSuccess ||
+        (b->mt && (e = cudaMalloc(&b->msched, (b->mtiles.size() + 1) * sizeof(int))) !=
+                      cudaSuccess))
         goto fail;
     for (auto &c : b->classes)
         if ((e = dev_copy(&c.d_tiles, c.tiles)) != cudaSuccess ||

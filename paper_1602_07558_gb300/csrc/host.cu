@@ -20,6 +20,7 @@
 
 #include "../../include/swept2d.h"
 #include "launch.cuh"
+#include "march_table.cuh"
 
 using swept::Geom;
 using swept::OpTable;
@@ -48,6 +49,12 @@ struct swept2d {
     int nx = 0, ny = 0, nv = 0, nst = 0, n = 0, op = 0, dtype = 0, esize = 0;
     Geom G{};
     const OpTable *ops = nullptr;
+    // the update's marching form (nullptr: none), the grid's shape and cut for
+    // it, and its counters (one per tile, the item counter)
+    const swept::MarchTable *mt = nullptr;
+    int mshape = 0;
+    swept::MarchGrid mgrid{};
+    int *msched = nullptr;
     cudaStream_t stream = nullptr;
     void *state = nullptr, *state2 = nullptr, *up = nullptr, *br = nullptr;
     unsigned long long *scratch8 = nullptr;
@@ -160,6 +167,16 @@ const OpTable *table_for(int op, int dtype) {
     }
 }
 
+const swept::MarchTable *march_for(int op, int dtype) {
+    switch (op) {
+        case SWEPT2D_OP_HEAT: return swept::marchtable_heat();
+        case SWEPT2D_OP_HEAT_KAHAN:
+            return dtype == SWEPT2D_F32 ? swept::marchtable_heat_kahan_f32()
+                                        : swept::marchtable_heat_kahan_bf16();
+        default: return nullptr;
+    }
+}
+
 bool dtype_ok(int op, int dtype) {
     if (op == SWEPT2D_OP_HASH || op == SWEPT2D_OP_WIDE2) return dtype == SWEPT2D_U64;
     if (op == SWEPT2D_OP_HEAT_KAHAN || op == SWEPT2D_OP_EULER_KAHAN)
@@ -175,6 +192,7 @@ void free_all(swept2d *h) {
     if (h->scratch8) cudaFree(h->scratch8);
     if (h->errword) cudaFree(h->errword);
     if (h->sched) cudaFree(h->sched);
+    if (h->msched) cudaFree(h->msched);
     for (auto &t : h->timed) {
         cudaEventDestroy(t.start);
         cudaEventDestroy(t.stop);
@@ -188,7 +206,7 @@ void free_all(swept2d *h) {
     h->state = h->state2 = h->up = h->br = nullptr;
     h->scratch8 = nullptr;
     h->errword = nullptr;
-    h->sched = nullptr;
+    h->sched = h->msched = nullptr;
 }
 
 int naive_substeps(swept2d *h, long long count) {
@@ -204,7 +222,29 @@ int naive_substeps(swept2d *h, long long count) {
     return SWEPT2D_OK;
 }
 
+// The whole advance (`total` sub-steps, whole steps) in the marching form;
+// `first` > 0 skips work items (the wait-timeout self-test).
+int march_substeps(swept2d *h, long long total, int first, long long spin_limit) {
+    if (total == 0) return SWEPT2D_OK;
+    void *out = h->state;
+    long long made = 0;
+    int rc = launch(h, SWEPT2D_K_MARCH, "marching kernel", [&] {
+        return h->mt->one(h->mshape, h->mgrid, h->consts, h->state, h->state2, h->state,
+                          h->msched, total, h->errword, first, spin_limit, &out, &made,
+                          h->stream);
+    });
+    if (rc) return rc;
+    h->launches += made - 1;
+    if (first > 0) return SWEPT2D_OK;
+    if (out != h->state) std::swap(h->state, h->state2);
+    h->substeps += total;
+    return SWEPT2D_OK;
+}
+
 int swept_substeps(swept2d *h, long long total, bool persistent) {
+    // (a trace records the items of the persistent swept form)
+    if (h->mt && !(persistent && h->trace))
+        return march_substeps(h, total, 0, swept::kPersistSpinLimit);
     const int half = h->n / 2;
     const long long H = total / half;
     const long long rem = total - H * half;
@@ -411,6 +451,16 @@ int swept2d_create(swept2d_t **out, int nx, int ny, int nvars, int nstages, int 
             return bail(e == cudaErrorMemoryAllocation ? SWEPT2D_ENOMEM : SWEPT2D_ECUDA);
         }
     }
+    h->mt = tile ? march_for(op, dtype) : nullptr;
+    if (h->mt) {
+        h->mshape = h->mt->shape(&nx, &ny, 1);
+        h->mgrid = h->mt->cut(h->mshape, nx, ny);
+        if ((e = cudaMalloc(&h->msched, ((size_t)h->mgrid.bx * h->mgrid.by + 1) * sizeof(int))) !=
+            cudaSuccess) {
+            cuda_fail(h, e, "schedule allocation");
+            return bail(e == cudaErrorMemoryAllocation ? SWEPT2D_ENOMEM : SWEPT2D_ECUDA);
+        }
+    }
     if ((e = cudaMalloc(&h->scratch8, sizeof(unsigned long long))) != cudaSuccess ||
         (e = cudaMalloc(&h->errword, sizeof(int))) != cudaSuccess ||
         (e = cudaMemset(h->errword, 0, sizeof(int))) != cudaSuccess) {
@@ -487,12 +537,15 @@ int swept2d_selftest_wait_timeout(swept2d_t *h, long long spin_limit) {
         return fail(h, SWEPT2D_EINVAL, "selftest: the persistent form takes at most 512 threads per block");
     int rc = persistent_prepare(h, 1);
     if (rc) return rc;
-    const int NT = h->G.T * h->G.Q;
-    cudaError_t e = cudaMemsetAsync(h->sched, 0, ((size_t)NT + 1) * sizeof(int), h->stream);
+    // the first phase's items skipped: every item taken waits for a counter that
+    // nothing releases
+    const int NT = h->mt ? h->mgrid.bx * h->mgrid.by : h->G.T * h->G.Q;
+    cudaError_t e = cudaMemsetAsync(h->sched, 0, ((size_t)h->G.T * h->G.Q + 1) * sizeof(int),
+                                    h->stream);
     if (e != cudaSuccess) return cuda_fail(h, e, "selftest schedule reset");
-    // one half cycle with the NT first-phase items skipped: every item taken
-    // waits for a phase-1 counter that nothing releases
-    rc = launch(h, SWEPT2D_K_OCTAHEDRON, "persistent kernel (wait-timeout self-test)", [&] {
+    if (h->mt)
+        rc = march_substeps(h, 2LL * h->nst * h->mt->steps(h->mshape), NT, spin_limit);
+    else rc = launch(h, SWEPT2D_K_OCTAHEDRON, "persistent kernel (wait-timeout self-test)", [&] {
         return h->ops->persistent(h->G, h->consts, h->state, h->up, h->br, h->sched, 1,
                                   (u64)h->substeps, h->errword, h->tune, NT, spin_limit,
                                   nullptr, h->stream);

@@ -51,6 +51,22 @@ struct Geom {
                   // multiple of 8 elements, so every panel starts on 16 bytes
 };
 
+// How the marching form (march.cuh) cuts a grid: bx x by tiles, tile i of a
+// side of n points covering [i n / b, (i + 1) n / b).
+struct MarchGrid {
+    int nx, ny, bx, by;
+};
+
+// One grid of a batch.
+struct GridDesc {
+    Geom G;                 // the grid's geometry (tile side n of its class)
+    MarchGrid m;            // its cut for the marching form
+    long long state_off;    // first element of the grid's state in the pooled state
+    long long panel_off;    // first element of the grid's panel slots in each pool
+    double c[8];            // the point update's constants for this grid (Euler's
+                            // depend on the grid's own state and spacing)
+};
+
 __host__ __device__ inline int panel_stride(int n) { return ((n * n / 2 + n) + 7) & ~7; }
 
 // The geometry a swept kernel works with: NC > 0 fixes the tile side at compile

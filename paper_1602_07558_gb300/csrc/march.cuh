@@ -1,0 +1,601 @@
+// The marching form of an advance: one launch runs every step of one or many
+// grids. The steps are cut into phases of up to K; in a phase each tile (a
+// rectangle of the grid, unrelated to the caller's tile side) is read with a
+// ring of K points around it, advanced K steps by one block with its values in
+// registers, and written to the other state buffer. The ring is computed
+// redundantly, which the swept rule avoids; in exchange a point's values stay
+// in registers for the whole phase and only the warps' edge rows and columns
+// pass through shared memory.
+//
+// Items (phase, tile) are taken in order from an atomic counter. An item of
+// phase j starts once its periodic 3 x 3 tile neighbourhood has finished phase
+// j - 1: those tiles hold every point its ring reads (a tile is at least K
+// points wide when the grid has more than one along that side), and they are
+// the only readers of the buffer it overwrites. A dependency has a smaller
+// index, so the lowest unfinished item can always run, whatever number of
+// blocks is resident. Waits are bounded, as in the persistent form.
+#pragma once
+#include <climits>
+#include <type_traits>
+
+#include "exact64.cuh"
+#include "kernels.cuh"
+#include "march_table.cuh"
+
+namespace swept {
+
+// One tile of a phase.
+struct MarchTile {
+    MarchGrid g;
+    int x0, y0, w, h;         // the tile
+    int I, J, base;           // its place, and its grid's first index among the counters
+    long long soff;           // first element of the grid's state in the pooled state
+    const double *c;          // the grid's own update constants (nullptr: the launch's)
+    // first column of tile i of a row of tiles: even, but for the grid's end
+    __device__ __forceinline__ int column(int i) const {
+        return i == g.bx ? g.nx : (int)((long long)i * g.nx / g.bx) & ~1;
+    }
+    __device__ __forceinline__ void place(int t) {
+        J = t / g.bx;
+        I = t - J * g.bx;
+        x0 = column(I);
+        y0 = (int)((long long)J * g.ny / g.by);
+        w = column(I + 1) - x0;
+        h = (int)((long long)(J + 1) * g.ny / g.by) - y0;
+    }
+};
+
+struct OneMarch {
+    MarchGrid g;
+    __device__ __forceinline__ MarchTile operator()(int t) const {
+        MarchTile m;
+        m.g = g;
+        m.base = 0;
+        m.soff = 0;
+        m.c = nullptr;
+        m.place(t);
+        return m;
+    }
+};
+
+// A launch's share of an advance: `phases` phases of K steps (the last one of
+// `last` steps), reading `src` in the first and then the buffer the phase
+// before wrote; phase j writes buf[j & 1].
+template <class S>
+struct MarchRun {
+    const S *src;
+    S *buf[2];
+    int *done, *queue, *err;   // per-tile phase counts, item counter (zeroed), error word
+    int NT, phases, K, last, first;
+    long long spin_limit;
+};
+
+// A ring of K columns, rounded up so that it starts at an even column.
+__host__ __device__ constexpr int even_ring(int k) { return (k + 1) & ~1; }
+
+__device__ __forceinline__ int wrap_index(int i, int n) {
+    i %= n;
+    return i < 0 ? i + n : i;
+}
+
+// Waits until the 3 x 3 neighbourhood of the tile has finished `need` phases.
+// Returns false (the same for the whole block) when the wait gave up.
+__device__ __forceinline__ bool march_wait(const MarchTile &m, const int *done, int need, int *err,
+                                           long long spin_limit) {
+    bool bad = false;
+    if (need > 0 && threadIdx.x < 9) {
+        const int dj = (int)threadIdx.x / 3 - 1, di = (int)threadIdx.x % 3 - 1;
+        const int J = wrap_index(m.J + dj, m.g.by), I = wrap_index(m.I + di, m.g.bx);
+        const int *flag = done + m.base + J * m.g.bx + I;
+        long long it = 0;
+        while (ld_acquire(flag) < need) {
+            if (++it > spin_limit || ((it & 255) == 0 && ld_relaxed(err) != 0)) {
+                bad = true;
+                break;
+            }
+            __nanosleep(32);
+        }
+        if (bad) atomicExch(err, 2);
+    }
+    return __syncthreads_or(bad) == 0;
+}
+
+template <class Body, class Op, class Loc>
+__global__ void __launch_bounds__(Body::kThreads, Body::kMinBlocks)
+march_kernel(Op op, Loc at, MarchRun<typename Op::S> run) {
+    typedef typename Op::S S;
+    __shared__ typename Body::Smem sm;
+    __shared__ int s_item;
+    const int nitems = run.NT * run.phases;
+    for (;;) {
+        if (threadIdx.x == 0) {
+            const int it = atomicAdd(run.queue, 1) + run.first;
+            s_item = ld_relaxed(run.err) ? nitems : it;
+        }
+        __syncthreads();
+        const int item = s_item;
+        if (item >= nitems) return;
+        const int j = item / run.NT, t = item - j * run.NT;
+        const MarchTile m = at(t);
+        if (!march_wait(m, run.done, j, run.err, run.spin_limit)) return;
+        const S *src = (j == 0 ? run.src : run.buf[(j - 1) & 1]) + m.soff;
+        Body::run(m.c ? Op(m.c) : op, m, src, run.buf[j & 1] + m.soff, run.K,
+                  j + 1 == run.phases ? run.last : run.K, j, sm);
+        __threadfence();
+        __syncthreads();
+        if (threadIdx.x == 0) add_release(run.done + t, 1);
+    }
+}
+
+// ------------------------------------------------------------------- heat
+// Two values of one plane in adjacent columns. Binary32 pairs go through the
+// packed instructions (one issue slot for two results; each result rounded as
+// by the scalar instruction).
+struct F2 {
+    unsigned long long v;
+    __device__ __forceinline__ float lo() const { return __uint_as_float((unsigned)v); }
+    __device__ __forceinline__ float hi() const { return __uint_as_float((unsigned)(v >> 32)); }
+};
+struct D2 {
+    double l, h;
+    __device__ __forceinline__ double lo() const { return l; }
+    __device__ __forceinline__ double hi() const { return h; }
+};
+struct L2 {
+    long long l, h;
+    __device__ __forceinline__ long long lo() const { return l; }
+    __device__ __forceinline__ long long hi() const { return h; }
+};
+__device__ __forceinline__ F2 two(float l, float h) {
+    F2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(l), "f"(h));
+    return r;
+}
+__device__ __forceinline__ D2 two(double l, double h) { return D2{l, h}; }
+__device__ __forceinline__ L2 two(long long l, long long h) { return L2{l, h}; }
+__device__ __forceinline__ F2 add2(F2 a, F2 b) {
+    F2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 mul2(F2 a, F2 b) {
+    F2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) {
+    F2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+    return r;
+}
+// a - b (the product by -1 is exact)
+__device__ __forceinline__ F2 sub2(F2 a, F2 b) { return fma2(b, two(-1.0f, -1.0f), a); }
+
+// Two adjacent columns' east values (the second's comes from the next lane), and
+// a row's pair sums E + S moved one column to the right, which makes them the
+// W + N sums of the row below.
+template <class V2>
+__device__ __forceinline__ V2 east_of(V2 v) {
+    return two(v.hi(), __shfl_down_sync(0xffffffffu, v.lo(), 1));
+}
+template <class V2>
+__device__ __forceinline__ V2 moved_right(V2 v) {
+    return two(__shfl_up_sync(0xffffffffu, v.hi(), 1), v.lo());
+}
+
+// The values a thread keeps for two points, and their update.
+template <class Op>
+struct HeatCell;
+template <>
+struct HeatCell<HeatOp> {
+    typedef double V;
+    typedef D2 V2;
+    static constexpr bool kComp = false;
+    double r;
+    __device__ __forceinline__ explicit HeatCell(const HeatOp &op) : r(op.r) {}
+    __device__ static __forceinline__ V ld(double v) { return v; }
+    __device__ static __forceinline__ double st(V v) { return v; }
+    __device__ __forceinline__ V2 pair(V2 a, V2 b) const {
+        return two(__dadd_rn(a.l, b.l), __dadd_rn(a.h, b.h));
+    }
+    __device__ __forceinline__ void next(V2 &u, V2 &, V2 pe, V2 pw) const {
+        u = two(__fma_rn(r, __fma_rn(-4.0, u.l, __dadd_rn(pe.l, pw.l)), u.l),
+                __fma_rn(r, __fma_rn(-4.0, u.h, __dadd_rn(pe.h, pw.h)), u.h));
+    }
+};
+// The heat update in a block's fixed-point unit (exact64.cuh).
+struct FixedCell {
+    typedef L2 V2;
+    static constexpr bool kComp = false;
+    FixedHeat f;
+    __device__ __forceinline__ V2 pair(V2 a, V2 b) const {
+        return two(f.sum(a.l, b.l), f.sum(a.h, b.h));
+    }
+    __device__ __forceinline__ void next(V2 &u, V2 &, V2 pe, V2 pw) {
+        u = two(f.next(u.l, pe.l, pw.l), f.next(u.h, pe.h, pw.h));
+    }
+};
+// The storage rounding of a pair.
+__device__ __forceinline__ F2 stored2(F2 a, const float *) { return a; }
+__device__ __forceinline__ F2 stored2(F2 a, const __nv_bfloat16 *) {
+    unsigned p;
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(p) : "f"(a.hi()), "f"(a.lo()));
+    return two(__uint_as_float(p << 16), __uint_as_float(p & 0xffff0000u));
+}
+template <class SS>
+struct HeatCell<HeatKahanOp<SS>> {
+    typedef float V;
+    typedef F2 V2;
+    static constexpr bool kComp = true;
+    F2 r;
+    __device__ __forceinline__ explicit HeatCell(const HeatKahanOp<SS> &op) : r(two(op.r, op.r)) {}
+    __device__ static __forceinline__ V ld(SS v) { return Store<SS>::ld(v); }
+    __device__ static __forceinline__ SS st(V v) { return Store<SS>::st(v); }
+    __device__ __forceinline__ V2 pair(V2 a, V2 b) const { return add2(a, b); }
+    __device__ __forceinline__ void next(V2 &u, V2 &c, V2 pe, V2 pw) const {
+        const SS *s = nullptr;
+        const F2 d = fma2(two(-4.0f, -4.0f), u, add2(pe, pw));
+        const F2 y = sub2(mul2(r, d), c);
+        const F2 un = stored2(add2(u, y), s);
+        c = stored2(sub2(sub2(un, u), y), s);
+        u = un;
+    }
+};
+
+// A block is WY warps over a region of 64 columns and R WY rows: a thread holds
+// R rows of two adjacent columns. A step: the warps' first and last rows go to
+// shared memory (two buffers in turn, one barrier a step), then each thread
+// walks down its rows. The outermost columns and rows of the region go wrong by
+// one more each step, which the ring covers; warps whose rows no later step
+// needs rest.
+template <class Op, int R_, int WY_, int MINB_, int K_>
+struct HeatMarch {
+    typedef typename Op::S S;
+    typedef HeatCell<Op> Cell;
+    typedef typename Cell::V V;
+    typedef typename Cell::V2 V2;
+    static constexpr int R = R_, WY = WY_, K = K_;   // K: steps a phase
+    static constexpr int kThreads = 32 * WY, kMinBlocks = MINB_;
+    static constexpr bool kInPlace = false;
+    static constexpr int kRows = R * WY;     // the region's, of 64 columns, ring included
+    static constexpr int kTileCols = 64 - 2 * even_ring(K), kTileRows = kRows - 2 * K;
+    static_assert(kTileCols >= 2 * K + 4 && kTileRows >= 2 * K, "a tile is at least K points wide");
+    static constexpr bool kFixed = std::is_same<Op, HeatOp>::value;
+    struct Smem {
+        V2 row[2][WY][2][32];    // a warp's first and last row
+        int high[WY], low[WY];   // its extremes (FP64)
+    };
+    struct alignas(2 * sizeof(S)) Two {
+        S a, b;
+    };
+    // Calls f(row, element of the thread's first column) for the thread's rows.
+    template <class F>
+    __device__ static __forceinline__ void each_row(const MarchTile &m, int gx, int gy, F &&f) {
+        const size_t nx = m.g.nx, back = nx - nx * m.g.ny;   // to the next row, to the first one
+        size_t at = (size_t)gy * nx + gx;
+#pragma unroll
+        for (int j = 0; j < R; ++j) {
+            f(j, at);
+            const bool last = ++gy == m.g.ny;
+            gy = last ? 0 : gy;
+            at += last ? back : nx;
+        }
+    }
+
+    // `steps` steps of the region's values.
+    template <class C, class T, int N>
+    __device__ static __forceinline__ void march(C &cell, T (&u)[R], T (&comp)[N], int rows, int r0,
+                                                 int lane, int wy, int steps, T (*edge)[WY][2][32]) {
+#pragma unroll 1
+        for (int s = 0; s < steps; ++s) {
+            T (*row)[2][32] = edge[s & 1];
+            row[wy][0][lane] = u[0];
+            row[wy][1][lane] = u[R - 1];
+            __syncthreads();
+            if (r0 + R <= s + 1 || r0 >= rows - 1 - s) continue;
+            const T above = wy > 0 ? row[wy > 0 ? wy - 1 : 0][1][lane] : u[0];
+            const T below = wy + 1 < WY && r0 + R < rows ? row[wy + 1 < WY ? wy + 1 : 0][0][lane]
+                                                         : u[R - 1];
+            T pp = cell.pair(east_of(above), u[0]);       // the row above's pair sums
+#pragma unroll
+            for (int j = 0; j < R; ++j) {
+                const T pe = cell.pair(east_of(u[j]), j + 1 < R ? u[j + 1 < R ? j + 1 : 0] : below);
+                cell.next(u[j], comp[N > 1 ? j : 0], pe, moved_right(pp));
+                pp = pe;
+            }
+        }
+    }
+
+    __device__ static __forceinline__ void run(const Op &op, const MarchTile &m, const S *src,
+                                               S *dst, int ring, int steps, int, Smem &sm) {
+        Cell cell(op);
+        const int lane = threadIdx.x & 31, wy = threadIdx.x >> 5;
+        const int c = 2 * lane, r0 = wy * R;
+        const int ring_x = even_ring(ring);
+        const int cols = m.w + 2 * ring_x, rows = m.h + 2 * ring;
+        const size_t plane = (size_t)m.g.nx * m.g.ny;
+        // (lanes and rows beyond the region repeat its last ones: values of the
+        // field's own size)
+        const int gx = wrap_index(m.x0 - ring_x + min(c, (cols - 1) & ~1), m.g.nx);
+        const int gy = wrap_index(m.y0 - ring + r0, m.g.ny);
+        // (tiles start at even columns, so with an even nx a thread's two columns
+        // are one aligned pair of an aligned plane)
+        const ptrdiff_t east = gx + 1 == m.g.nx ? 1 - m.g.nx : 1;
+        const bool pairs = (m.g.nx & 1) == 0 &&
+                           (((size_t)src | (size_t)dst) & (2 * sizeof(S) - 1)) == 0;
+        V2 u[R], comp[Cell::kComp ? R : 1];
+        const auto load = [&](auto &&get) {
+            each_row(m, gx, gy, [&](int j, size_t at) {
+                if (j == 0 || r0 + j < rows) {
+                    u[j] = get(src + at);
+                    if (Cell::kComp) comp[j] = get(src + plane + at);
+                } else {
+                    u[j] = u[j > 0 ? j - 1 : 0];
+                    if (Cell::kComp) comp[j] = comp[j > 0 ? j - 1 : 0];
+                }
+            });
+        };
+        const auto read = [&] {
+            if (pairs)
+                load([&](const S *p) {
+                    const Two t = *reinterpret_cast<const Two *>(p);
+                    return two(Cell::ld(t.a), Cell::ld(t.b));
+                });
+            else
+                load([&](const S *p) { return two(Cell::ld(p[0]), Cell::ld(p[east])); });
+        };
+        read();
+        bool done = false;
+        if constexpr (kFixed) {
+            // the block's extremes (upper words: of negative values, too, the larger
+            // word is the larger magnitude) decide on the unit
+            int high = INT_MIN, low = INT_MAX;
+#pragma unroll
+            for (int j = 0; j < R; ++j) {
+                const int l = __double2hiint(u[j].l), h = __double2hiint(u[j].h);
+                high = max(high, max(l, h));
+                low = min(low, min(l, h));
+            }
+            high = __reduce_max_sync(0xffffffffu, high);
+            low = __reduce_min_sync(0xffffffffu, low);
+            if (lane == 0) {
+                sm.high[wy] = high;
+                sm.low[wy] = low;
+            }
+            __syncthreads();
+#pragma unroll
+            for (int w = 0; w < WY; ++w) {
+                high = max(high, sm.high[w]);
+                low = min(low, sm.low[w]);
+            }
+            const int top = (high >> 20) & 0x7ff, bottom = (low >> 20) & 0x7ff;
+            FixedCell fixed{{heat_ratio(op.r), top - (kFixedBinades - 1),
+                             (unsigned)high & 0x80000000u, 0u}};
+            // one sign, normal, six binades at most, sums and the unit in range
+            if (fixed.f.R != 0 && (high ^ low) >= 0 && bottom >= fixed.f.e0 && fixed.f.e0 > 0 &&
+                top < 2040) {
+                L2 v[R], none[1];
+#pragma unroll
+                for (int j = 0; j < R; ++j) v[j] = two(fixed.f.from(u[j].l), fixed.f.from(u[j].h));
+                march(fixed, v, none, rows, r0, lane, wy, steps,
+                      reinterpret_cast<L2 (*)[WY][2][32]>(sm.row));
+                done = __syncthreads_or(fixed.f.failed()) == 0;
+                if (done) {
+#pragma unroll
+                    for (int j = 0; j < R; ++j) u[j] = two(fixed.f.to(v[j].l), fixed.f.to(v[j].h));
+                } else {
+                    read();
+                }
+            }
+        }
+        if (!done) march(cell, u, comp, rows, r0, lane, wy, steps, sm.row);
+        const bool one = c >= ring_x && c < ring_x + m.w;
+        const bool both = c + 1 >= ring_x && c + 1 < ring_x + m.w;
+        const int first = ring - r0, end = ring + m.h - r0;
+        if (pairs) {
+            if (one)
+                each_row(m, gx, gy, [&](int j, size_t at) {
+                    if (j >= first && j < end) {
+                        Two *p = reinterpret_cast<Two *>(dst + at);
+                        *p = Two{Cell::st(u[j].lo()), Cell::st(u[j].hi())};
+                        if (Cell::kComp)
+                            *reinterpret_cast<Two *>(dst + plane + at) =
+                                Two{Cell::st(comp[j].lo()), Cell::st(comp[j].hi())};
+                    }
+                });
+        } else {
+            each_row(m, gx, gy, [&](int j, size_t at) {
+                if (j < first || j >= end) return;
+                S *p = dst + at;
+                if (one) p[0] = Cell::st(u[j].lo());
+                if (both) p[east] = Cell::st(u[j].hi());
+                if (Cell::kComp && one) p[plane] = Cell::st(comp[j].lo());
+                if (Cell::kComp && both) p[(ptrdiff_t)plane + east] = Cell::st(comp[j].hi());
+            });
+        }
+    }
+};
+
+// The shapes an update's tiles come in, largest first. A shape is rows a thread,
+// warps, blocks an SM and steps a phase. Rows in registers and the region's
+// size save redundant work, steps a phase save passes over memory and waits,
+// and both cost warps an SM, which hide the shuffles' and the integer chains'
+// latency. Measured on the GB300 (ms for the whole advance):
+//   binary64, 4096², 500 steps: (8, 8, 3, 4) 36.4, (8, 4, 5, 4) 40.1,
+//     (4, 8, 4, 4) 40.4, (8, 8, 2, 4) 45.4, (8, 16, 1, 4) 52.6
+//   binary64, 768², 403 steps: (2, 8, 4, 3) 2.0, (4, 8, 4, 4) 2.2, (8, 4, 5, 4) 2.9
+//   binary64, 64², 512 steps: (1, 8, 4, 2) 0.68, (2, 8, 4, 3) 0.72, (1, 16, 2, 3) 0.73
+//   binary32, 2048², 2000 steps: (16, 4, 4, 8) 8.2, (8, 8, 4, 6) 8.9,
+//     (16, 8, 2, 12) 8.7; 1,024 grids of {32..512}²: 25.7, 27.6, 28.0
+template <class Op>
+struct MarchShapes;
+template <>
+struct MarchShapes<HeatOp> {
+    static constexpr int kCount = 4;
+    template <int I>
+    using Body = std::conditional_t<
+        I == 0, HeatMarch<HeatOp, 8, 8, 3, 4>,
+        std::conditional_t<I == 1, HeatMarch<HeatOp, 4, 8, 4, 4>,
+                           std::conditional_t<I == 2, HeatMarch<HeatOp, 2, 8, 4, 3>,
+                                              HeatMarch<HeatOp, 1, 8, 4, 2>>>>;
+};
+template <class SS>
+struct MarchShapes<HeatKahanOp<SS>> {
+    typedef HeatKahanOp<SS> Op;
+    static constexpr int kCount = 3;
+    template <int I>
+    using Body = std::conditional_t<
+        I == 0, HeatMarch<Op, 16, 4, 4, 8>,
+        std::conditional_t<I == 1, HeatMarch<Op, 8, 4, 4, 6>, HeatMarch<Op, 2, 8, 4, 4>>>;
+};
+
+// Tiles of many grids: the table lists each grid's tiles consecutively.
+struct ManyMarch {
+    const GridDesc *grids;
+    const int2 *tiles;           // (grid, tile within the grid)
+    __device__ __forceinline__ MarchTile operator()(int t) const {
+        const int2 e = tiles[t];
+        const GridDesc *gd = grids + e.x;
+        MarchTile m;
+        m.g = gd->m;
+        m.base = t - e.y;
+        m.soff = gd->state_off;
+        m.c = gd->c;
+        m.place(e.y);
+        return m;
+    }
+};
+
+// ----------------------------------------------------------- host side
+// Calls f with the body type of shape i.
+template <class Op, int I = 0, class F>
+inline cudaError_t with_march_shape(int i, F &&f) {
+    if constexpr (I < MarchShapes<Op>::kCount) {
+        if (i == I) return f((typename MarchShapes<Op>::template Body<I> *)nullptr);
+        return with_march_shape<Op, I + 1>(i, f);
+    } else {
+        return cudaErrorInvalidValue;
+    }
+}
+
+// How one grid is cut for a shape.
+template <class Op>
+inline MarchGrid march_cut(int shape, int nx, int ny) {
+    MarchGrid g{nx, ny, 0, 0};
+    with_march_shape<Op>(shape, [&](auto *body) {
+        typedef typename std::remove_pointer<decltype(body)>::type B;
+        // (even first columns: a tile may be one column wider than its share)
+        g.bx = nx <= B::kTileCols ? 1 : (nx + B::kTileCols - 2) / (B::kTileCols - 1);
+        g.by = (ny + B::kTileRows - 1) / B::kTileRows;
+        return cudaSuccess;
+    });
+    return g;
+}
+
+template <class Op>
+inline int march_steps(int shape) {
+    int k = 1;
+    with_march_shape<Op>(shape, [&](auto *body) {
+        k = std::remove_pointer<decltype(body)>::type::K;
+        return cudaSuccess;
+    });
+    return k;
+}
+
+// The largest shape that gives the GPU's 152 SMs three tiles each (all grids
+// together), else the smallest one.
+template <class Op>
+inline int march_shape(const int *nx, const int *ny, int count) {
+    int shape = 0;
+    for (; shape + 1 < MarchShapes<Op>::kCount; ++shape) {
+        long long tiles = 0;
+        for (int i = 0; i < count; ++i) {
+            const MarchGrid g = march_cut<Op>(shape, nx[i], ny[i]);
+            tiles += (long long)g.bx * g.by;
+        }
+        if (tiles >= 3 * 152) break;
+    }
+    return shape;
+}
+
+// Queues `steps` steps over NT tiles: reads `src`, writes b0, b1, b0, ... phase
+// by phase (src may be b1). sched: NT counters and the item counter. `launches`
+// is raised by the launches made, `*out` set to the buffer with the result.
+template <class Op, class Loc>
+inline cudaError_t march_advance(int shape, const Op &op, const Loc &at, int NT, const void *src,
+                                 void *b0, void *b1, int *sched, long long steps, int *err,
+                                 int first, long long spin_limit, void **out, long long *launches,
+                                 cudaStream_t st) {
+    typedef typename Op::S S;
+    return with_march_shape<Op>(shape, [&](auto *body) {
+        typedef typename std::remove_pointer<decltype(body)>::type B;
+        constexpr int K = B::K;
+        const auto kern = march_kernel<B, Op, Loc>;
+        if (B::kInPlace) b0 = b1 = const_cast<void *>(src);
+        int per_sm = 0, dev = 0, nsm = 0;
+        cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, B::kThreads, 0);
+        if (e != cudaSuccess) return e;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+        // items of one launch count in an int
+        // (an even number of phases: the stages of Euler alternate)
+        const long long most = (((1LL << 30) - 1) / NT + 2) & ~1LL;
+        while (steps > 0) {
+            const long long left = (steps + K - 1) / K;
+            MarchRun<S> run;
+            run.src = (const S *)src;
+            run.buf[0] = (S *)b0;
+            run.buf[1] = (S *)b1;
+            run.done = sched;
+            run.queue = sched + NT;
+            run.err = err;
+            run.NT = NT;
+            run.phases = (int)(left < most ? left : most);
+            run.K = K;
+            run.last = run.phases < left ? K : (int)(steps - (left - 1) * K);
+            run.first = first;
+            run.spin_limit = spin_limit;
+            if ((e = cudaMemsetAsync(sched, 0, ((size_t)NT + 1) * sizeof(int), st)) != cudaSuccess)
+                return e;
+            long long grid = (long long)(per_sm > 0 ? per_sm : 1) * nsm;
+            if (grid > 2LL * NT) grid = 2LL * NT;
+            if (grid > (long long)NT * run.phases) grid = (long long)NT * run.phases;
+            kern<<<(int)grid, B::kThreads, 0, st>>>(op, at, run);
+            if ((e = cudaGetLastError()) != cudaSuccess) return e;
+            *launches += 1;
+            steps -= (long long)(run.phases - 1) * K + run.last;
+            *out = run.buf[(run.phases - 1) & 1];
+            src = *out;
+            if (*out == b0) {
+                b0 = b1;
+                b1 = *out;
+            }
+        }
+        return cudaSuccess;
+    });
+}
+
+template <class Op>
+struct March {
+    static cudaError_t one(int shape, const MarchGrid &g, const double *c, const void *src,
+                           void *b0, void *b1, int *sched, long long steps, int *err, int first,
+                           long long spin_limit, void **out, long long *launches,
+                           cudaStream_t st) {
+        return march_advance(shape, Op(c), OneMarch{g}, g.bx * g.by, src, b0, b1, sched, steps,
+                             err, first, spin_limit, out, launches, st);
+    }
+    static cudaError_t many(int shape, const GridDesc *grids, const int2 *tiles, int NT,
+                            const double *c, const void *src, void *b0, void *b1, int *sched,
+                            long long steps, int *err, void **out, long long *launches,
+                            cudaStream_t st) {
+        return march_advance(shape, Op(c), ManyMarch{grids, tiles}, NT, src, b0, b1, sched, steps,
+                             err, 0, kPersistSpinLimit, out, launches, st);
+    }
+    static const MarchTable *table() {
+        static const MarchTable t = {&march_shape<Op>, &march_steps<Op>, &march_cut<Op>, &one,
+                                     &many};
+        return &t;
+    }
+};
+
+}  // namespace swept

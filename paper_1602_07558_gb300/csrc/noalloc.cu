@@ -9,11 +9,9 @@
 // other device memory this path touches is the file-scope array below, which
 // the CUDA runtime sets up when it loads this library's device code.
 //
-// The schedule and the kernels are the same as swept2d_advance's swept mode
-// (Up, then per half cycle the x/y Bridge launch and the Octahedron, a final
-// Down, then the remaining sub-steps with the naive kernel), so the result is
-// bit for bit that of a handle created with op SWEPT2D_OP_HEAT and advanced
-// with SWEPT2D_SWEPT from the same input.
+// The marching form of swept2d_advance (march.cuh) on the caller's buffers, so
+// the result is bit for bit that of a handle created with op SWEPT2D_OP_HEAT and
+// advanced with SWEPT2D_SWEPT from the same input.
 #include <cuda_runtime.h>
 
 #include <cstdio>
@@ -21,15 +19,16 @@
 
 #include "../../include/swept2d.h"
 #include "launch.cuh"
+#include "march_table.cuh"
 
 namespace {
 
 constexpr size_t kScratchBytes = SWEPT2D_STATIC_SCRATCH_BYTES;
 
 // Shared by every call on a device and kept until the process exits. Holds the
-// two panel buffers and, when the step count leaves a naive tail, one state
-// copy for its ping-pong. Nothing in it has to start at zero: every element a
-// call reads was written earlier in that same call.
+// second state buffer and the counters of the marching form. Nothing in it has
+// to start at zero: every element a call reads was written earlier in that same
+// call.
 static __device__ __align__(256) unsigned char g_scratch[kScratchBytes];
 
 void set_err(char *err, int errlen, const char *msg) {
@@ -110,59 +109,36 @@ extern "C" int swept2d_heat_advance_static(const double *u_in, double *u_out, in
     void *base = nullptr;
     int rc = scratch_address(&base, err, errlen);
     if (rc != SWEPT2D_OK) return rc;
-    char *sb = (char *)base;
-    void *up = sb;
-    void *br = sb + align256(panel_bytes);
-    double *tmp = (double *)(sb + 2 * align256(panel_bytes));
-
-    const swept::OpTable *t = swept::optable_heat();
-    const double consts[8] = {r, 0, 0, 0, 0, 0, 0, 0};
-    const swept::Tuning tn;   // 256 threads, per-level prefetch (the handle path's heat default)
     cudaStream_t st = (cudaStream_t)stream;
-    cudaError_t e = cudaSuccess;
-    auto check = [&](cudaError_t ce, const char *what) {
-        if (ce != cudaSuccess) {
-            char msg[200];
-            snprintf(msg, sizeof msg, "%s: %s", what, cudaGetErrorString(ce));
-            set_err(err, errlen, msg);
-            return false;
-        }
-        return true;
-    };
-    // The tail's ping-pong is arranged so that its last sub-step lands in u_out.
-    if (H == 0) {
-        if (rem == 0) {
-            e = cudaMemcpyAsync(u_out, u_in, state_bytes, cudaMemcpyDeviceToDevice, st);
-            return check(e, "copy") ? SWEPT2D_OK : SWEPT2D_ECUDA;
-        }
-        const double *src = u_in;
-        for (long long i = 0; i < rem; ++i) {
-            double *dst = ((rem - 1 - i) % 2 == 0) ? u_out : tmp;
-            if (!check(t->naive(G, consts, src, dst, (u64)i, st), "naive kernel")) return SWEPT2D_ECUDA;
-            src = dst;
-        }
-        return SWEPT2D_OK;
+    if (nsteps == 0) {
+        const cudaError_t e = cudaMemcpyAsync(u_out, u_in, state_bytes, cudaMemcpyDeviceToDevice, st);
+        if (e != cudaSuccess) set_err(err, errlen, cudaGetErrorString(e));
+        return e == cudaSuccess ? SWEPT2D_OK : SWEPT2D_ECUDA;
     }
-    double *swept_dst = (rem % 2 == 1) ? tmp : u_out;
-    if (!check(t->up(G, consts, u_in, up, 0, 0, st), "up kernel")) return SWEPT2D_ECUDA;
-    for (long long j = 0; j < H; ++j) {
-        const u64 g0 = (u64)j * half;
-        const int o = (j & 1) ? half : 0;
-        if (!check(t->bridge(G, consts, up, br, g0, nullptr, tn, st), "bridge kernel")) return SWEPT2D_ECUDA;
-        if (j + 1 < H) {
-            if (!check(t->octahedron(G, consts, br, up, o, g0, nullptr, tn, st), "octahedron kernel"))
-                return SWEPT2D_ECUDA;
-        } else {
-            if (!check(t->down(G, consts, br, swept_dst, o, g0, nullptr, tn, st), "down kernel"))
-                return SWEPT2D_ECUDA;
-        }
-    }
-    const double *src = swept_dst;
-    for (long long i = 0; i < rem; ++i) {
-        double *dst = (src == tmp) ? u_out : tmp;
-        if (!check(t->naive(G, consts, src, dst, (u64)(H * half + i), st), "naive kernel"))
-            return SWEPT2D_ECUDA;
-        src = dst;
+    // the scratch holds the second state buffer, the marching form's counters and
+    // an error word; two panel sets hold more than four times the state, so they
+    // fit wherever the check above passed
+    const swept::MarchTable *mt = swept::marchtable_heat();
+    const int shape = mt->shape(&nx, &ny, 1);
+    const swept::MarchGrid cut = mt->cut(shape, nx, ny);
+    void *tmp = base;
+    int *sched = (int *)((char *)base + align256(state_bytes));
+    int *errword = sched + cut.bx * cut.by + 1;
+    cudaError_t e = cudaMemsetAsync(errword, 0, sizeof(int), st);
+    // the buffers alternate phase by phase; the last phase writes u_out
+    const long long phases = (nsteps + mt->steps(shape) - 1) / mt->steps(shape);
+    void *b0 = (phases & 1) ? (void *)u_out : tmp, *b1 = (phases & 1) ? tmp : (void *)u_out;
+    const double consts[8] = {r, 0, 0, 0, 0, 0, 0, 0};
+    void *out = nullptr;
+    long long made = 0;
+    if (e == cudaSuccess)
+        e = mt->one(shape, cut, consts, u_in, b0, b1, sched, nsteps, errword, 0,
+                    swept::kPersistSpinLimit, &out, &made, st);
+    if (e != cudaSuccess) {
+        char msg[200];
+        snprintf(msg, sizeof msg, "marching kernel: %s", cudaGetErrorString(e));
+        set_err(err, errlen, msg);
+        return SWEPT2D_ECUDA;
     }
     return SWEPT2D_OK;
 }

@@ -26,6 +26,7 @@
 #include <cuda_bf16.h>
 
 #include <cstdint>
+#include <cstring>
 
 typedef unsigned long long u64;
 

@@ -1,0 +1,98 @@
+"""The marching form (every step of an advance in one launch) against the CPU
+oracle, bit for bit: tile and region edges, odd and tiny grids, step counts
+around a phase, and the FP64 heat's integer arithmetic on the values where it
+could differ from the FP64 operations."""
+import numpy as np
+import pytest
+
+from paper_1602_07558_gb300 import inputs
+from paper_1602_07558_gb300.swept2d import Swept2D, SweptBatch
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():  # pragma: no cover
+    pytest.skip("no CUDA device", allow_module_level=True)
+
+
+def swept(op, u0, nsteps, tile, params, dtype=None):
+    ny, nx = u0.shape[-2:]
+    with Swept2D(nx, ny, op=op, tile=tile, params=params, dtype=dtype) as s:
+        s.set_state(np.ascontiguousarray(u0.reshape(s.shape)))
+        s.advance(nsteps)
+        return s.get_state()
+
+
+def field(kind, nx, ny):
+    rng = np.random.default_rng(nx + 3 * ny)
+    smooth = inputs.smooth_field(nx, ny, seed=2)
+    smooth = smooth / np.abs(smooth).max()
+    return {
+        "one_binade": 1.5 + 0.2 * smooth,
+        "binades": 3.0 + 2.9 * smooth,                 # 0.1 .. 5.9: six binades
+        "negative": -2.0 - 0.5 * smooth,
+        "crossing": smooth,
+        "noise": rng.random((ny, nx)),
+        "mixed_sign_noise": rng.standard_normal((ny, nx)),
+        "ties": 1.0 + rng.integers(0, 2 ** 20, (ny, nx)) * 2.0 ** -52,
+        "few_bits": 1.0 + rng.integers(0, 8, (ny, nx)) / 8.0,
+        "powers": 2.0 ** rng.integers(-3, 3, (ny, nx)),
+        "constant": np.full((ny, nx), 1.0),
+        "zeros": np.zeros((ny, nx)),
+        "tiny": (1.0 + 0.3 * smooth) * 2.0 ** -1060,   # below the normal numbers
+        "smallest_normal": (1.0 + 0.3 * smooth) * 2.0 ** -1021,
+        "huge": (1.0 + 0.3 * smooth) * 2.0 ** 1019,
+    }[kind]
+
+
+@pytest.mark.parametrize("r", [0.2, 0.125, 0.1875, 0.2499999, 0.25, 0.1, 0.0, -0.05])
+@pytest.mark.parametrize("kind", ["one_binade", "binades", "negative", "crossing", "noise",
+                                  "mixed_sign_noise", "ties", "few_bits", "powers", "constant",
+                                  "zeros", "tiny", "smallest_normal", "huge"])
+def test_fp64_heat_integer_arithmetic_is_bitwise(oracle_lib, kind, r):
+    u0 = field(kind, 96, 64)
+    with np.errstate(all="ignore"):
+        ref = oracle_lib.heat(u0, r, 21)
+    assert np.array_equal(swept("heat", u0, 21, 32, (r,))[0], ref, equal_nan=True)
+
+
+def test_fp64_heat_keeps_infinities_and_nans_local(oracle_lib):
+    u0 = field("one_binade", 128, 96)
+    u0[5, 7], u0[60, 100] = np.inf, np.nan
+    ref = oracle_lib.heat(u0, 0.2, 9)
+    assert np.array_equal(swept("heat", u0, 9, 32, (0.2,))[0], ref, equal_nan=True)
+
+
+# grids that take each of the shapes, with one tile, several, and sides smaller than the ring
+@pytest.mark.parametrize("nx,ny,tile,nsteps", [
+    (4, 4, 4, 9), (8, 200, 4, 11), (200, 8, 4, 11), (30, 30, 6, 7),
+    (64, 48, 16, 1), (64, 48, 16, 2), (64, 48, 16, 3), (112, 96, 16, 13), (330, 1020, 10, 10),
+    (1120, 1100, 20, 9), (2056, 1608, 8, 9),
+])
+@pytest.mark.parametrize("op,dtype", [("heat", "f64"), ("heat_kahan", "f32"), ("heat_kahan", "bf16")])
+def test_march_edges_match_the_oracle(oracle_lib, op, dtype, nx, ny, tile, nsteps):
+    u = 1.0 + np.random.default_rng(nx).random((ny, nx))
+    if op == "heat":
+        ref = oracle_lib.heat(u, 0.2, nsteps)
+        assert np.array_equal(swept(op, u, nsteps, tile, (0.2,))[0], ref)
+        return
+    u = u.astype(np.float32)
+    if dtype == "bf16":
+        u = torch.from_numpy(u).to(torch.bfloat16).view(torch.int16).numpy().view(np.uint16)
+    ref_u, ref_c = oracle_lib.heat_kahan(u, np.zeros_like(u), 0.2, nsteps, storage=dtype)
+    got = swept(op, np.stack([u, np.zeros_like(u)]), nsteps, tile, (0.2,), dtype=dtype)
+    assert np.array_equal(got[0], ref_u) and np.array_equal(got[1], ref_c)
+
+
+def test_batch_of_odd_and_even_grids_matches_the_oracle(oracle_lib):
+    """Odd sides put the grids after them at odd offsets of the pool, where a
+    pair of columns is not an aligned pair."""
+    sizes = [(33, 47, 0), (64, 96, 32), (35, 31, 0), (130, 60, 10), (7, 5, 0)]
+    us = [1.0 + np.random.default_rng(i).random((ny, nx)) for i, (nx, ny, _) in enumerate(sizes)]
+    with SweptBatch([s[0] for s in sizes], [s[1] for s in sizes], [s[2] for s in sizes],
+                    op="heat", params=(0.2,)) as b:
+        b.set_state([u[None] for u in us])
+        b.advance(23)
+        got = b.split(b.get_state())
+    for u, g in zip(us, got):
+        assert np.array_equal(g[0], oracle_lib.heat(u, 0.2, 23))
