@@ -690,7 +690,7 @@ __device__ __forceinline__ void compute_rect_mid(const WaveOp &op, int, u64, con
         const int a = e + yy;                            // packed as for the heat update
         const double c = src[off], old = src[plane + off];
         const double d = __fma_rn(-4.0, c, __dadd_rn(aux[a + W1 + 1], aux[a]));
-        dst[off] = __fma_rn(op.C2, d, __dsub_rn(__dmul_rn(2.0, c), old));
+        dst[off] = op.next(c, old, d);
         dst[plane + off] = c;
     }
 }

@@ -213,7 +213,10 @@ struct EulerKahanOp {
 // 2D wave equation u_tt = c^2 laplace(u), leapfrog in time (Section 6's
 // experiment); point state (u^n, u^{n-1}):
 //   d = ((u_E + u_S) + (u_W + u_N)) - 4u,  u^{n+1} = (2u - u^{n-1}) + C^2 d (fused)
-// C2 = (c dt / dx)^2 is formed on the host.
+// C2 = (c dt / dx)^2 is formed on the host. 2u - u^{n-1} is one fused operation,
+// with the bits of the two: 2u is exact unless it overflows, which the last
+// binade's u do, to an infinity. A sixth FP64 operation a point saved for four
+// integer instructions (the 1024² grid: 15.0 to 13.0 ms for 1,000 steps).
 struct WaveOp {
     typedef double S;
     static constexpr int NV = 2, NST = 1, AUX = 1;   // aux: pair sums of a level
@@ -222,13 +225,20 @@ struct WaveOp {
     static constexpr bool INPLACE_AFTER_AUX = true;
     double C2;
     __host__ __device__ explicit WaveOp(const double *c) : C2(c[0]) {}
+    __device__ __forceinline__ double next(double u, double old, double d) const {
+        double x = __fma_rn(2.0, u, -old);
+        const int hi = __double2hiint(u);
+        if ((hi & 0x7ff00000) == 0x7fe00000)
+            x = __hiloint2double((hi & 0x80000000) | 0x7ff00000, 0);
+        return __fma_rn(C2, d, x);
+    }
     template <class A>
     __device__ __forceinline__ void operator()(int, u64, const A &a, S *out) const {
         const double c = a(0, 0, 0);
         const double pe = __dadd_rn(a(1, 0, 0), a(0, 1, 0));
         const double pw = __dadd_rn(a(-1, 0, 0), a(0, -1, 0));
         const double d = __fma_rn(-4.0, c, __dadd_rn(pe, pw));
-        out[0] = __fma_rn(C2, d, __dsub_rn(__dmul_rn(2.0, c), a(0, 0, 1)));
+        out[0] = next(c, a(0, 0, 1), d);
         out[1] = c;
     }
 };

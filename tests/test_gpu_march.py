@@ -96,3 +96,67 @@ def test_batch_of_odd_and_even_grids_matches_the_oracle(oracle_lib):
         got = b.split(b.get_state())
     for u, g in zip(us, got):
         assert np.array_equal(g[0], oracle_lib.heat(u, 0.2, 23))
+
+
+@pytest.mark.parametrize("scale", [1.0, 2.0 ** 1022, 2.0 ** 1023 * 1.2, 2.0 ** -1074 * 9])
+def test_wave_fused_difference_has_the_bits_of_two_operations(oracle_lib, scale):
+    """2u - u_old as one operation, also where 2u overflows, at infinities and
+    zeros of both signs and below the normal numbers."""
+    rng = np.random.default_rng(3)
+    u = (1.0 + 0.4 * rng.random((2, 48, 64))) * scale
+    u[0, 3, 4], u[1, 9, 9], u[0, 20:24, 20:24], u[1, 20:22] = np.inf, -np.inf, -0.0, 0.0
+    with np.errstate(all="ignore"):
+        ref_u, ref_old = oracle_lib.wave(u[0], u[1], 0.3 * 0.3, 11)
+    got = swept("wave", u, 11, 16, (0.3,))
+    assert np.array_equal(got[0], ref_u, equal_nan=True)
+    assert np.array_equal(got[1], ref_old, equal_nan=True)
+
+
+@pytest.mark.parametrize("nx,ny,tile,nsteps", [
+    (4, 4, 4, 3), (16, 60, 4, 4), (30, 30, 6, 5), (64, 48, 16, 6), (150, 150, 10, 3),
+    (330, 300, 10, 3), (1040, 1056, 16, 2),
+])
+@pytest.mark.parametrize("op,dtype", [("euler_rk2", "f64"), ("euler_kahan", "f32"),
+                                      ("euler_kahan", "bf16")])
+def test_euler_march_edges_match_the_oracle(oracle_lib, op, dtype, nx, ny, tile, nsteps):
+    """Each shape of the marching form and, in binary64, the sizes that stay with
+    the swept kernels; every plane (binary64: U) bit for bit."""
+    U = inputs.euler_pulse(nx, ny, 4, gamma=1.4)
+    if op == "euler_rk2":
+        u0 = np.concatenate([U, U])
+        a, dt = oracle_lib.euler_setup(U, 1.4, 0.3)
+        ref = oracle_lib.euler_rk2(U, 1.4, dt, 0.5, a, nsteps)
+    else:
+        U = U.astype(np.float32)
+        if dtype == "bf16":
+            U = torch.from_numpy(U).to(torch.bfloat16).view(torch.int16).numpy().view(np.uint16)
+        Uf = (oracle_lib.bf16_bits_to_f32(U) if dtype == "bf16" else U).astype(np.float64)
+        u0 = np.concatenate([U, U, np.zeros_like(U)])
+        a, dt = oracle_lib.euler_setup(Uf, 1.4, 0.3)
+        ref = oracle_lib.euler_kahan(u0, 1.4, dt, 0.5, a, nsteps, dtype)
+    got = swept(op, u0, nsteps, tile, (1.4, 0.3, 0.5), dtype=dtype)
+    assert np.array_equal(got[:len(ref)], ref)
+    with Swept2D(nx, ny, op=op, tile=tile, params=(1.4, 0.3, 0.5), dtype=dtype) as s:
+        s.set_state(u0)
+        s.advance(nsteps, mode="naive")
+        assert np.array_equal(got, s.get_state())      # the midpoint planes, too
+
+
+def test_euler_batch_of_uneven_grids_matches_the_single_grids():
+    sizes = [(33, 47, 0), (64, 96, 32), (35, 31, 0), (130, 60, 10)]
+    for op, dtype in (("euler_rk2", "f64"), ("euler_kahan", "f32")):
+        states = []
+        for i, (nx, ny, _) in enumerate(sizes):
+            U = inputs.euler_pulse(nx, ny, i, gamma=1.4)
+            states.append(np.concatenate([U, U] + ([np.zeros_like(U)] if dtype == "f32" else []))
+                          .astype(np.float32 if dtype == "f32" else np.float64))
+        with SweptBatch([s[0] for s in sizes], [s[1] for s in sizes], [s[2] for s in sizes], op=op,
+                        params=(1.4, 0.3, 0.5), dtype=dtype) as b:
+            b.set_state(states)
+            b.advance(7)
+            got = b.split(b.get_state())
+        for (nx, ny, _), u, g in zip(sizes, states, got):
+            with Swept2D(nx, ny, op=op, tile=0, params=(1.4, 0.3, 0.5), dtype=dtype) as s:
+                s.set_state(u)
+                s.advance(7, mode="naive")
+                assert np.array_equal(g, s.get_state())
