@@ -403,6 +403,13 @@ struct BatchLaunch {
                                      &down, &persistent, &persistent_all, &one_launch_smem};
         return &t;
     }
+    // an update whose batches always advance in the marching form (march.cuh)
+    static const BatchTable *naive_table() {
+        static const BatchTable t = {Op::NV, Op::NST, (int)sizeof(S), Op::STAGE,
+                                     &swept_smem_for<Op>, &naive, nullptr, nullptr, nullptr,
+                                     nullptr, nullptr, nullptr, &one_launch_smem};
+        return &t;
+    }
 };
 
 const BatchTable *batchtable_heat();

@@ -108,6 +108,10 @@ const swept::MarchTable *batch_march(int op, int dtype) {
     if (op == SWEPT2D_OP_HEAT_KAHAN)
         return dtype == SWEPT2D_F32 ? swept::marchtable_heat_kahan_f32()
                                     : swept::marchtable_heat_kahan_bf16();
+    if (op == SWEPT2D_OP_EULER_RK2) return swept::marchtable_euler();
+    if (op == SWEPT2D_OP_EULER_KAHAN)
+        return dtype == SWEPT2D_F32 ? swept::marchtable_euler_kahan_f32()
+                                    : swept::marchtable_euler_kahan_bf16();
     return nullptr;
 }
 
@@ -397,7 +401,8 @@ int swept2d_batch_create(swept2d_batch_t **out, int count, const int *nx, const 
         b->dt.assign(count, 0.0);
     }
     b->mt = batch_march(op, dtype);
-    if (b->mt) b->mshape = b->mt->shape(nx, ny, count);
+    if (b->mt) b->mshape = b->mt->shape(nx, ny, count, false);
+    if (b->mshape < 0) b->mt = nullptr;
     // grids, classes (by tile side), pooled offsets
     long long soff = 0, poff = 0;
     for (int i = 0; i < count; ++i) {
@@ -465,7 +470,7 @@ int swept2d_batch_create(swept2d_batch_t **out, int count, const int *nx, const 
         (e = cudaMalloc(&b->errword, sizeof(int))) != cudaSuccess ||
         (e = cudaMemset(b->errword, 0, sizeof(int))) != cudaSuccess)
         goto fail;
-    if (b->panel_bytes &&
+    if (b->panel_bytes && !b->mt &&      // (the marching form has no panels)
         ((e = cudaMalloc(&b->up, b->panel_bytes)) != cudaSuccess ||
          (e = cudaMalloc(&b->br, b->panel_bytes)) != cudaSuccess))
         goto fail;

@@ -1,7 +1,7 @@
 // Instantiation unit: the batched kernels of heat FP64, the hash test update and
 // Euler FP64, and the per-grid wave-speed reduction that fixes each Euler
-// grid's time step. The compensated binary32 forms (built for several tile
-// sides) have units of their own: batch_heat_kahan.cu, batch_euler_kahan.cu.
+// grid's time step. The compensated binary32 forms have units of their own:
+// batch_heat_kahan.cu, batch_euler_kahan.cu.
 #include "batch.cuh"
 
 namespace swept {

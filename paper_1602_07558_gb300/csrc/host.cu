@@ -173,6 +173,10 @@ const swept::MarchTable *march_for(int op, int dtype) {
         case SWEPT2D_OP_HEAT_KAHAN:
             return dtype == SWEPT2D_F32 ? swept::marchtable_heat_kahan_f32()
                                         : swept::marchtable_heat_kahan_bf16();
+        case SWEPT2D_OP_EULER_RK2: return swept::marchtable_euler();
+        case SWEPT2D_OP_EULER_KAHAN:
+            return dtype == SWEPT2D_F32 ? swept::marchtable_euler_kahan_f32()
+                                        : swept::marchtable_euler_kahan_bf16();
         default: return nullptr;
     }
 }
@@ -453,7 +457,10 @@ int swept2d_create(swept2d_t **out, int nx, int ny, int nvars, int nstages, int 
     }
     h->mt = tile ? march_for(op, dtype) : nullptr;
     if (h->mt) {
-        h->mshape = h->mt->shape(&nx, &ny, 1);
+        h->mshape = h->mt->shape(&nx, &ny, 1, false);
+        if (h->mshape < 0) h->mt = nullptr;
+    }
+    if (h->mt) {
         h->mgrid = h->mt->cut(h->mshape, nx, ny);
         if ((e = cudaMalloc(&h->msched, ((size_t)h->mgrid.bx * h->mgrid.by + 1) * sizeof(int))) !=
             cudaSuccess) {

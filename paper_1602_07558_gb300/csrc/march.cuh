@@ -174,13 +174,18 @@ __device__ __forceinline__ F2 sub2(F2 a, F2 b) { return fma2(b, two(-1.0f, -1.0f
 // Two adjacent columns' east values (the second's comes from the next lane), and
 // a row's pair sums E + S moved one column to the right, which makes them the
 // W + N sums of the row below.
-template <class V2>
-__device__ __forceinline__ V2 east_of(V2 v) {
-    return two(v.hi(), __shfl_down_sync(0xffffffffu, v.lo(), 1));
+// SEG: lanes that hold one run of columns (a warp may hold several).
+template <int SEG = 32>
+__device__ __forceinline__ unsigned seg_lanes() {
+    return SEG == 32 ? 0xffffffffu : ((1u << (SEG & 31)) - 1u) << (threadIdx.x & 31 & ~(SEG - 1));
 }
-template <class V2>
+template <int SEG = 32, class V2>
+__device__ __forceinline__ V2 east_of(V2 v) {
+    return two(v.hi(), __shfl_down_sync(seg_lanes<SEG>(), v.lo(), 1, SEG));
+}
+template <int SEG = 32, class V2>
 __device__ __forceinline__ V2 moved_right(V2 v) {
-    return two(__shfl_up_sync(0xffffffffu, v.hi(), 1), v.lo());
+    return two(__shfl_up_sync(seg_lanes<SEG>(), v.hi(), 1, SEG), v.lo());
 }
 
 // The values a thread keeps for two points, and their update.
@@ -416,8 +421,215 @@ struct HeatMarch {
     }
 };
 
-// The shapes an update's tiles come in, largest first. A shape is rows a thread,
-// warps, blocks an SM and steps a phase. Rows in registers and the region's
+// ------------------------------------------------------------------- Euler
+// Packed arithmetic on two columns, in the update's arithmetic type.
+__device__ __forceinline__ D2 add2(D2 a, D2 b) { return two(__dadd_rn(a.l, b.l), __dadd_rn(a.h, b.h)); }
+__device__ __forceinline__ D2 sub2(D2 a, D2 b) { return two(__dsub_rn(a.l, b.l), __dsub_rn(a.h, b.h)); }
+__device__ __forceinline__ D2 mul2(D2 a, D2 b) { return two(__dmul_rn(a.l, b.l), __dmul_rn(a.h, b.h)); }
+__device__ __forceinline__ D2 fma2(D2 a, D2 b, D2 c) {
+    return two(__fma_rn(a.l, b.l, c.l), __fma_rn(a.h, b.h, c.h));
+}
+// 1 / a, correctly rounded (the bits of the division)
+__device__ __forceinline__ D2 rcp2(D2 a) { return two(__drcp_rn(a.l), __drcp_rn(a.h)); }
+__device__ __forceinline__ F2 rcp2(F2 a) { return two(__frcp_rn(a.lo()), __frcp_rn(a.hi())); }
+template <int SEG, class V2>
+__device__ __forceinline__ V2 west_of(V2 v) { return moved_right<SEG>(v); }
+
+// One row of the stage's stencil values in a thread: W, and F1-F3, G1-G3 of the
+// two points (F0 = m and G0 = q are W's).
+template <class V2>
+struct EulerRow {
+    V2 w[4], F[3], G[3];
+};
+
+// One stage of the midpoint scheme per phase, in place: stage 0 reads U with its
+// neighbours and writes U*, stage 1 reads U* with its neighbours and writes U
+// (and C) at the point alone. SEG lanes walk down 2 SEG columns, two a thread,
+// with the rows above, at and below the current one in registers: every point's
+// primitives and fluxes are formed once and serve its four neighbours, the east
+// and west ones by shuffle. The outermost columns only supply neighbours. The
+// walks of a block take HR rows each and share nothing.
+template <class Op, int SEG_, int HR_, int WY_, int MINB_>
+struct EulerMarch {
+    typedef typename Op::S S;
+    static constexpr bool kWide = std::is_same<Op, EulerOp>::value;   // binary64, not compensated
+    typedef typename std::conditional<kWide, D2, F2>::type V2;
+    typedef typename std::conditional<kWide, double, float>::type V;
+    static constexpr int SEG = SEG_, HR = HR_, WY = WY_, K = 1;
+    static constexpr int kThreads = 32 * WY, kMinBlocks = MINB_;
+    static constexpr int kWalks = kThreads / SEG;
+    static constexpr bool kInPlace = true;
+    static constexpr int kRing = kWide ? 1 : 2;    // (aligned pairs for the narrow types)
+    static constexpr int kTileCols = 2 * SEG - 2 * kRing, kTileRows = HR * kWalks;
+    struct Smem {};
+    struct alignas(2 * sizeof(S)) Two {
+        S a, b;
+    };
+    __device__ static __forceinline__ V ld(S v) {
+        if constexpr (kWide) return v; else return Store<S>::ld(v);
+    }
+    __device__ static __forceinline__ V2 stored(V2 v) {
+        if constexpr (kWide) return v; else return stored2(v, (const S *)nullptr);
+    }
+    __device__ static __forceinline__ S st(V v) {
+        if constexpr (kWide) return v; else return Store<S>::st(v);
+    }
+
+    // The thread's two columns of a plane: aligned pairs (PAIRS), or the two
+    // elements, the second `east` of the first.
+    template <bool PAIRS>
+    struct Columns {
+        ptrdiff_t east;
+        bool one, both;     // this thread stores its first, its second column
+        __device__ __forceinline__ V2 get(const S *p) const {
+            if constexpr (PAIRS) {
+                const Two t = *reinterpret_cast<const Two *>(p);
+                return two(ld(t.a), ld(t.b));
+            }
+            return two(ld(p[0]), ld(p[east]));
+        }
+        __device__ __forceinline__ void put(S *p, V2 v) const {
+            if constexpr (PAIRS) {
+                if (one) *reinterpret_cast<Two *>(p) = Two{st(v.lo()), st(v.hi())};
+            } else {
+                if (one) p[0] = st(v.lo());
+                if (both) p[east] = st(v.hi());
+            }
+        }
+    };
+
+    __device__ static __forceinline__ V2 all(V c) { return two(c, c); }
+
+    __device__ static __forceinline__ void fluxes(const Op &op, EulerRow<V2> &r) {
+        const V2 m = r.w[1], q = r.w[2];
+        const V2 iv = rcp2(r.w[0]);
+        const V2 u = mul2(m, iv), v = mul2(q, iv);
+        const V2 ke = mul2(all(V(0.5)), fma2(m, u, mul2(q, v)));
+        const V2 pr = mul2(all(op.gm1), sub2(r.w[3], ke));
+        const V2 Ep = add2(r.w[3], pr);
+        r.F[0] = fma2(m, u, pr);
+        r.F[1] = mul2(q, u);
+        r.F[2] = mul2(Ep, u);
+        r.G[0] = mul2(m, v);
+        r.G[1] = fma2(q, v, pr);
+        r.G[2] = mul2(Ep, v);
+    }
+
+    // L of the conserved variable c at row `at` between rows `up` and `dn`.
+    template <int c>
+    __device__ static __forceinline__ V2 rate(const Op &op, const EulerRow<V2> &up,
+                                              const EulerRow<V2> &at, const EulerRow<V2> &dn) {
+        const V2 wE = east_of<SEG>(at.w[c]), wW = west_of<SEG>(at.w[c]);
+        const V2 f = c == 0 ? at.w[1] : at.F[c > 0 ? c - 1 : 0];
+        const V2 dF = sub2(east_of<SEG>(f), west_of<SEG>(f));
+        const V2 dG = c == 0 ? sub2(dn.w[2], up.w[2])
+                             : sub2(dn.G[c > 0 ? c - 1 : 0], up.G[c > 0 ? c - 1 : 0]);
+        const V2 lx = fma2(all(V(-2)), at.w[c], add2(wE, wW));
+        const V2 ly = fma2(all(V(-2)), at.w[c], add2(dn.w[c], up.w[c]));
+        const V2 diss = fma2(all(op.kax), lx, mul2(all(op.kay), ly));
+        const V2 flux = fma2(all(op.cx), dF, mul2(all(op.cy), dG));
+        return sub2(diss, flux);
+    }
+
+    // Stage `ST` of the rows [y, y + n) of the warp's columns.
+    template <int ST, bool PAIRS>
+    __device__ static __forceinline__ void walk(const Op &op, const MarchTile &m, S *state, int gx,
+                                                int c, int y, int n) {
+        const Columns<PAIRS> col{gx + 1 == m.g.nx ? 1 - m.g.nx : 1, c >= 0 && c < m.w,
+                                 c + 1 >= 0 && c + 1 < m.w};
+        const size_t nx = m.g.nx, plane = nx * m.g.ny;
+        const int ny = m.g.ny;
+        int gy = y == 0 ? ny - 1 : y - 1;            // the row that is read next
+        const S *p = state + (ST == 0 ? 0 : 4 * plane) + (size_t)gy * nx + gx;
+        V2 ahead[4];                                 // W of that row, read one row early
+        const auto fetch = [&] {
+#pragma unroll
+            for (int c = 0; c < 4; ++c) ahead[c] = col.get(p + c * plane);
+            const bool last = ++gy == ny;
+            gy = last ? 0 : gy;
+            p += last ? nx - plane : nx;
+        };
+        const auto next_row = [&](EulerRow<V2> &r) {
+#pragma unroll
+            for (int c = 0; c < 4; ++c) r.w[c] = ahead[c];
+        };
+        S *o = state + (size_t)y * nx + gx;          // the centre row's U
+        EulerRow<V2> A, B, C;
+        fetch();
+        next_row(A);
+        fetch();
+        fluxes(op, A);
+        next_row(B);
+        fetch();
+        fluxes(op, B);
+        const auto step = [&](const EulerRow<V2> &up, const EulerRow<V2> &at, EulerRow<V2> &dn,
+                              bool more) {
+            V2 U[4], Cc[4];
+            if constexpr (ST == 1) {
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    U[c] = col.get(o + c * plane);
+                    if constexpr (!kWide) Cc[c] = col.get(o + (8 + c) * plane);
+                }
+            }
+            next_row(dn);
+            if (more) fetch();
+            fluxes(op, dn);
+            const auto finish = [&](int c, V2 L) {
+                if constexpr (ST == 0) {
+                    col.put(o + (4 + c) * plane, stored(fma2(all(op.tau0), L, at.w[c])));
+                } else if constexpr (kWide) {
+                    col.put(o + c * plane, fma2(all(op.tau1), L, U[c]));
+                } else {
+                    const V2 yy = sub2(mul2(all(op.tau1), L), Cc[c]);
+                    const V2 un = stored(add2(U[c], yy));
+                    col.put(o + c * plane, un);
+                    col.put(o + (8 + c) * plane, sub2(sub2(un, U[c]), yy));
+                }
+            };
+            finish(0, rate<0>(op, up, at, dn));
+            finish(1, rate<1>(op, up, at, dn));
+            finish(2, rate<2>(op, up, at, dn));
+            finish(3, rate<3>(op, up, at, dn));
+            o += nx;
+        };
+        // (the row after the last one is read, but not the one after that)
+        for (int i = 0; i < n; i += 3) {
+            step(A, B, C, i + 1 < n);
+            if (i + 1 >= n) break;
+            step(B, C, A, i + 2 < n);
+            if (i + 2 >= n) break;
+            step(C, A, B, i + 3 < n);
+        }
+    }
+
+    __device__ static __forceinline__ void run(const Op &op, const MarchTile &m, const S *,
+                                               S *state, int, int, int phase, Smem &) {
+        const int walk_at = threadIdx.x / SEG;
+        const int c = 2 * (int)(threadIdx.x % SEG) - kRing;   // first column, from the tile's
+        const int nx = m.g.nx;
+        const int gx = wrap_index(m.x0 + c, nx);
+        const bool pairs = !kWide && (nx & 1) == 0 && ((size_t)state & (2 * sizeof(S) - 1)) == 0;
+        // the tile's rows, shared evenly
+        const int y = walk_at * m.h / kWalks, n = (walk_at + 1) * m.h / kWalks - y;
+        if (n == 0) return;
+        const auto stage = [&](auto st) {
+            constexpr int ST = decltype(st)::value;
+            if (!kWide && pairs)
+                walk<ST, !kWide>(op, m, state, gx, c, m.y0 + y, n);
+            else
+                walk<ST, false>(op, m, state, gx, c, m.y0 + y, n);
+        };
+        if ((phase & 1) == 0)
+            stage(std::integral_constant<int, 0>());
+        else
+            stage(std::integral_constant<int, 1>());
+    }
+};
+
+// The shapes an update's tiles come in, largest first.
+//
+// Heat: rows a thread, warps, blocks an SM and steps a phase. Rows in registers and the region's
 // size save redundant work, steps a phase save passes over memory and waits,
 // and both cost warps an SM, which hide the shuffles' and the integer chains'
 // latency. Measured on the GB300 (ms for the whole advance):
@@ -427,6 +639,19 @@ struct HeatMarch {
 //   binary64, 64², 512 steps: (1, 8, 4, 2) 0.68, (2, 8, 4, 3) 0.72, (1, 16, 2, 3) 0.73
 //   binary32, 2048², 2000 steps: (16, 4, 4, 8) 8.2, (8, 8, 4, 6) 8.9,
 //     (16, 8, 2, 12) 8.7; 1,024 grids of {32..512}²: 25.7, 27.6, 28.0
+//
+// Euler: lanes and rows a walk, warps, blocks an SM. More rows form fewer fluxes
+// twice; more blocks hide the loads' latency, as far as the three rows of values
+// stay in registers (binary64, at the FP64 pipe's rate, needs few); fewer lanes
+// waste less on narrow tiles and spread a small grid over more SMs.
+//   binary64, 32 stages, us, for the four shapes: 1024² 7567, 5049, 5779, 7536;
+//     512² 2720, 2669, 1481, 1924; 128 x 128 2714, 1416, 457, 336; 2048², 50 steps:
+//     56.7, 61.0 ms
+//   binary32, 2048², 200 steps, ms: (32, 32, 4, 4) 19.5, (32, 16, 4, 5) 19.5,
+//     (32, 16, 4, 6) 21.0, (32, 8, 4, 4) 21.4, (32, 32, 4, 3) 25.0; bfloat16: 14.2,
+//     16.0, 16.4, 16.8, 21.7; 256 grids binary32, 50 steps: 23.8, 24.7, 25.8, 27.9,
+//     30.1; 64 stages, us, for the five shapes: 1024² 1321, 614, 795, 1160, 1938;
+//     512² 1190, 466, 385, 307, 491; 128 x 128 1169, 411, 276, 216, 187
 template <class Op>
 struct MarchShapes;
 template <>
@@ -438,6 +663,29 @@ struct MarchShapes<HeatOp> {
         std::conditional_t<I == 1, HeatMarch<HeatOp, 4, 8, 4, 4>,
                            std::conditional_t<I == 2, HeatMarch<HeatOp, 2, 8, 4, 3>,
                                               HeatMarch<HeatOp, 1, 8, 4, 2>>>>;
+};
+template <>
+struct MarchShapes<EulerOp> {
+    static constexpr int kCount = 4;
+    template <int I>
+    using Body = std::conditional_t<
+        I == 0, EulerMarch<EulerOp, 32, 16, 4, 3>,
+        std::conditional_t<I == 1, EulerMarch<EulerOp, 16, 8, 4, 3>,
+                           std::conditional_t<I == 2, EulerMarch<EulerOp, 16, 2, 4, 3>,
+                                              EulerMarch<EulerOp, 8, 1, 2, 6>>>>;
+};
+template <class SS>
+struct MarchShapes<EulerKahanOp<SS>> {
+    typedef EulerKahanOp<SS> Op;
+    static constexpr int kCount = 5;
+    template <int I>
+    using Body = std::conditional_t<
+        I == 0, EulerMarch<Op, 32, 32, 4, 4>,
+        std::conditional_t<
+            I == 1, EulerMarch<Op, 32, 8, 4, 4>,
+            std::conditional_t<I == 2, EulerMarch<Op, 32, 4, 4, 4>,
+                               std::conditional_t<I == 3, EulerMarch<Op, 32, 2, 4, 4>,
+                                                  EulerMarch<Op, 32, 1, 4, 4>>>>>;
 };
 template <class SS>
 struct MarchShapes<HeatKahanOp<SS>> {
@@ -503,18 +751,34 @@ inline int march_steps(int shape) {
 }
 
 // The largest shape that gives the GPU's 152 SMs three tiles each (all grids
-// together), else the smallest one.
+// together), else the smallest one; -1 where the swept kernels do better, unless
+// `always`. That is only so in binary64, whose redundant points cost FP64 time:
+//  - heat, when its tiles fill less than 0.78 of their 64 columns and the grid is
+//    too large to be bound by latency (fields with a zero crossing in every tile,
+//    96 steps, us, swept / marching: 64 x 2048 292 / 437, 192 x 384 241 / 281, but
+//    48 x 512 221 / 181, 256 x 256 241 / 232, 1024 x 1024 1469 / 706);
+//  - Euler, in a middle range of sizes, where the SMs hold one small tile each
+//    (32 stages, us, swept / marching: 128 x 128 344 / 336, 160 x 160 355 / 436,
+//    256 x 256 576 / 727, 192 x 384 574 / 712, 320 x 320 827 / 778, 64 x 2048
+//    1134 / 970).
 template <class Op>
-inline int march_shape(const int *nx, const int *ny, int count) {
+inline int march_shape(const int *nx, const int *ny, int count, bool always) {
+    double points = 0, columns = 0;
     int shape = 0;
-    for (; shape + 1 < MarchShapes<Op>::kCount; ++shape) {
+    for (;; ++shape) {
         long long tiles = 0;
+        points = columns = 0;
         for (int i = 0; i < count; ++i) {
             const MarchGrid g = march_cut<Op>(shape, nx[i], ny[i]);
             tiles += (long long)g.bx * g.by;
+            points += (double)nx[i] * ny[i];
+            columns += 64.0 * g.bx * ny[i];
         }
-        if (tiles >= 3 * 152) break;
+        if (tiles >= 3 * 152 || shape + 1 == MarchShapes<Op>::kCount) break;
     }
+    if (always) return shape;
+    if (std::is_same<Op, HeatOp>::value && points > 28000 && points < 0.78 * columns) return -1;
+    if (std::is_same<Op, EulerOp>::value && points > 20000 && points < 90000) return -1;
     return shape;
 }
 

@@ -6,7 +6,8 @@ namespace swept {
 
 // Functions of one update's marching form (march_*.cu).
 struct MarchTable {
-    int (*shape)(const int *nx, const int *ny, int count);
+    // the shape for these grids; -1 (unless `always`): the swept kernels do better
+    int (*shape)(const int *nx, const int *ny, int count, bool always);
     int (*steps)(int shape);     // steps a phase
     MarchGrid (*cut)(int shape, int nx, int ny);
     // one grid (`g` its cut), or the tiles of a batch's table
@@ -21,5 +22,8 @@ struct MarchTable {
 const MarchTable *marchtable_heat();
 const MarchTable *marchtable_heat_kahan_f32();
 const MarchTable *marchtable_heat_kahan_bf16();
+const MarchTable *marchtable_euler();
+const MarchTable *marchtable_euler_kahan_f32();
+const MarchTable *marchtable_euler_kahan_bf16();
 
 }  // namespace swept

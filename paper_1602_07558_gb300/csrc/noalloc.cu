@@ -119,7 +119,7 @@ extern "C" int swept2d_heat_advance_static(const double *u_in, double *u_out, in
     // an error word; two panel sets hold more than four times the state, so they
     // fit wherever the check above passed
     const swept::MarchTable *mt = swept::marchtable_heat();
-    const int shape = mt->shape(&nx, &ny, 1);
+    const int shape = mt->shape(&nx, &ny, 1, true);
     const swept::MarchGrid cut = mt->cut(shape, nx, ny);
     void *tmp = base;
     int *sched = (int *)((char *)base + align256(state_bytes));
