@@ -57,6 +57,18 @@ struct FixedHeat {
     unsigned sign;               // 0 or 0x80000000
     unsigned wide;               // largest K seen, as the upper word of K + 2^55
 
+    // Sets the unit for values whose upper words lie in [low, high] as signed
+    // integers (of negative values, too, the larger word is the larger magnitude);
+    // false unless they are normal, of one sign and within the binades, r has a
+    // ratio, and sums stay finite.
+    __device__ __forceinline__ bool fits(double r, int high, int low) {
+        const int top = (high >> 20) & 0x7ff, bottom = (low >> 20) & 0x7ff;
+        R = heat_ratio(r);
+        e0 = top - (kFixedBinades - 1);
+        sign = (unsigned)high & 0x80000000u;
+        wide = 0;
+        return R != 0 && (high ^ low) >= 0 && bottom >= e0 && e0 > 0 && top < 2040;
+    }
     __device__ __forceinline__ long long from(double v) const {
         const long long b = __double_as_longlong(v);
         const int e = (__double2hiint(v) >> 20) & 0x7ff;

@@ -39,6 +39,9 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <climits>
+
+#include "exact64.cuh"
 #include "ops.cuh"
 
 namespace swept {
@@ -794,6 +797,13 @@ __device__ __forceinline__ void write_up_panels(const S *cur, int P, const Geom 
 }
 
 // ---------------------------------------------------------------- naive path
+// A naive launch may begin when the blocks of the one before it have left
+// (launch_after): this waits until that one's results, which the kernel reads,
+// are in memory.
+__device__ __forceinline__ void after_previous_launch() {
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");
+}
+
 // One sub-step over the whole grid: out = St(in) at every point.
 template <class Op>
 __global__ void __launch_bounds__(256) naive_kernel(Op op, Geom G, const typename Op::S *in,
@@ -802,6 +812,7 @@ __global__ void __launch_bounds__(256) naive_kernel(Op op, Geom G, const typenam
     const int x = blockIdx.x * 32 + (threadIdx.x & 31);
     const int y = blockIdx.y * 8 + (threadIdx.x >> 5);
     if (x >= G.nx || y >= G.ny) return;
+    after_previous_launch();
     const size_t plane = (size_t)G.nx * G.ny;
     GlobalAcc<S> acc(in, plane, G.nx, G.ny, x, y);
     S res[Op::NV];
@@ -811,39 +822,81 @@ __global__ void __launch_bounds__(256) naive_kernel(Op op, Geom G, const typenam
     for (int v = 0; v < Op::NV; ++v) out[v * plane + p] = res[v];
 }
 
-// Heat, naive path: each warp walks down a chunk of 31 columns over ROWS rows
-// (32 on large grids, fewer on small ones so that enough warps run); lane l
-// holds column x = 31 c + l - 1 (lane 0 only supplies the pair sum
-// of the column to the left). The east+south pair sum of row y-1 moves one lane
-// to the right with a shuffle and is the west+north pair sum at row y, so a
-// point costs about 4.1 FP64 operations, with the roundings of HeatOp.
+// The rows of the kernel below by the FP64 operations.
+template <int ROWS>
+__device__ __forceinline__ void naive_heat_rows(const double (&u)[ROWS + 2], double (&res)[ROWS],
+                                             double r) {
+    double pp = __dadd_rn(__shfl_down_sync(0xffffffffu, u[0], 1), u[1]);
+#pragma unroll
+    for (int j = 0; j < ROWS; ++j) {
+        const double pc = __dadd_rn(__shfl_down_sync(0xffffffffu, u[j + 1], 1), u[j + 2]);
+        const double s = __dadd_rn(pc, __shfl_up_sync(0xffffffffu, pp, 1));
+        res[j] = __fma_rn(r, __fma_rn(-4.0, u[j + 1], s), u[j + 1]);
+        pp = pc;
+    }
+}
+
+// Heat, naive path: a warp takes 30 columns (lane l holds column x = 30 c + l - 1,
+// the outer lanes only supply their neighbours) and ROWS rows. The rows are read
+// once; a row's east + south pair sums, moved one lane to the right, are the west
+// + north sums of the row below. Where the warp's values allow it the arithmetic
+// runs on the integer units (exact64.cuh), otherwise by the FP64 operations,
+// about 4.3 a point (one row a warp, on grids bound by latency, always takes
+// those). The integer units bound it. Measured on the GB300, us a step in a
+// graph, before (31 columns, FP64 operations): 1009 x 757 8.9 -> 6.3, 2048²
+// 39.7 -> 23.1, 4096² 136.6 -> 85.1 (8 rows; 4 rows 85.8, 16 rows 96.2).
 template <int ROWS>
 __global__ void __launch_bounds__(256) naive_heat_kernel(HeatOp op, Geom G, const double *in,
                                                          double *out) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int x = blockIdx.x * 31 + lane - 1;
-    if (x < 0) x += G.nx;
-    const bool active = lane > 0 && x < G.nx;
-    if (x >= G.nx) x %= G.nx;            // idle lanes read valid memory, store nothing
-    const int xe = x + 1 == G.nx ? 0 : x + 1;
+    int x = blockIdx.x * 30 + lane - 1;
+    const bool active = lane > 0 && lane < 31 && x < G.nx;
+    x = x < 0 ? G.nx - 1 : x % G.nx;      // idle lanes read valid memory, store nothing
     const int y0 = (blockIdx.y * 8 + warp) * ROWS;
     if (y0 >= G.ny) return;               // whole warp leaves together
-    const int y1 = min(y0 + ROWS, G.ny);
+    after_previous_launch();
+    const int n = min(ROWS, G.ny - y0);
     const size_t nx = G.nx;
-    int ym = y0 - 1;
-    if (ym < 0) ym += G.ny;
-    double c = in[(size_t)y0 * nx + x];
-    double pp = __dadd_rn(in[(size_t)ym * nx + xe], c);   // Pr(x, y0-1)
-    for (int y = y0; y < y1; ++y) {
-        const int ys = y + 1 == G.ny ? 0 : y + 1;
-        const double sd = in[(size_t)ys * nx + x];
-        const double pc = __dadd_rn(in[(size_t)y * nx + xe], sd);   // Pr(x, y)
-        const double q = __shfl_up_sync(0xffffffffu, pp, 1);         // Pr(x-1, y-1)
-        const double res = __fma_rn(op.r, __fma_rn(-4.0, c, __dadd_rn(pc, q)), c);
-        if (active) out[(size_t)y * nx + x] = res;
-        pp = pc;
-        c = sd;
+    double u[ROWS + 2];                   // rows y0 - 1 .. y0 + n, the last repeated
+#pragma unroll
+    for (int j = 0; j < ROWS + 2; ++j) {
+        int y = y0 - 1 + (j <= n ? j : n + 1);
+        y = y < 0 ? G.ny - 1 : (y == G.ny ? 0 : y);
+        u[j] = in[(size_t)y * nx + x];
     }
+    double res[ROWS];
+    bool done = false;
+    if constexpr (ROWS > 1) {
+        int high = INT_MIN, low = INT_MAX;
+#pragma unroll
+        for (int j = 0; j < ROWS + 2; ++j) {
+            high = max(high, __double2hiint(u[j]));
+            low = min(low, __double2hiint(u[j]));
+        }
+        high = __reduce_max_sync(0xffffffffu, high);
+        low = __reduce_min_sync(0xffffffffu, low);
+        FixedHeat f;
+        done = f.fits(op.r, high, low);
+        if (done) {
+            long long c = f.from(u[1]);
+            long long pp = f.sum(__shfl_down_sync(0xffffffffu, f.from(u[0]), 1), c);
+#pragma unroll
+            for (int j = 0; j < ROWS; ++j) {
+                const long long sd = f.from(u[j + 2]);
+                const long long pc = f.sum(__shfl_down_sync(0xffffffffu, c, 1), sd);
+                res[j] = f.to(f.next(c, pc, __shfl_up_sync(0xffffffffu, pp, 1)));
+                pp = pc;
+                c = sd;
+            }
+            done = !__any_sync(0xffffffffu, f.failed());
+        }
+    }
+    if (!done) naive_heat_rows<ROWS>(u, res, op.r);
+    if (!active) return;
+    double *o = out + (size_t)y0 * nx + x;
+#pragma unroll
+    for (int j = 0; j < ROWS; ++j)
+        if (j < n) o[j * nx] = res[j];
 }
 
 // Reduced-precision heat, naive path: lane = column, each warp walks ROWS rows
@@ -856,6 +909,7 @@ __global__ void __launch_bounds__(256) naive_heat_kahan_kernel(HeatKahanOp<SS> o
     const int x = blockIdx.x * 32 + lane;
     const int y0 = (blockIdx.y * 8 + warp) * ROWS;
     if (x >= G.nx || y0 >= G.ny) return;
+    after_previous_launch();
     const int y1 = min(y0 + ROWS, G.ny);
     const size_t nx = G.nx, plane = (size_t)G.nx * G.ny;
     const int xw = x == 0 ? G.nx - 1 : x - 1, xe = x + 1 == G.nx ? 0 : x + 1;

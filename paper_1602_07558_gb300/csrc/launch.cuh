@@ -108,26 +108,42 @@ inline cudaError_t allow_smem(K kernel, size_t bytes) {
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
+// Launches a naive kernel so that its blocks may be set up while the stream's
+// launch before it still runs; the kernel itself waits for that one's end
+// (after_previous_launch).
+template <class... P, class... A>
+inline cudaError_t launch_after(void (*kernel)(P...), dim3 grid, cudaStream_t st, A... args) {
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(kBlock);
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 template <class Op>
 struct Launch {
     typedef typename Op::S S;
     static cudaError_t naive(const Geom &G, const double *c, const void *in, void *out, u64 g,
                              cudaStream_t st) {
+        cudaError_t e;
         if constexpr (std::is_same<Op, HeatOp>::value) {
             // rows per warp: as many as keep about 32 warps per SM in flight
-            const long long chunks = (G.nx + 30) / 31;
-            int rows = 32;
+            const long long chunks = (G.nx + 29) / 30;
+            int rows = 8;
             while (rows > 1 && chunks * ((G.ny + rows - 1) / rows) < 152LL * 32) rows >>= 1;
             const int warps = (G.ny + rows - 1) / rows;
             dim3 grid((unsigned)chunks, (warps + 7) / 8);
             const Op op(c);
             switch (rows) {
-                case 32: naive_heat_kernel<32><<<grid, kBlock, 0, st>>>(op, G, (const S *)in, (S *)out); break;
-                case 16: naive_heat_kernel<16><<<grid, kBlock, 0, st>>>(op, G, (const S *)in, (S *)out); break;
-                case 8: naive_heat_kernel<8><<<grid, kBlock, 0, st>>>(op, G, (const S *)in, (S *)out); break;
-                case 4: naive_heat_kernel<4><<<grid, kBlock, 0, st>>>(op, G, (const S *)in, (S *)out); break;
-                case 2: naive_heat_kernel<2><<<grid, kBlock, 0, st>>>(op, G, (const S *)in, (S *)out); break;
-                default: naive_heat_kernel<1><<<grid, kBlock, 0, st>>>(op, G, (const S *)in, (S *)out); break;
+                case 8: e = launch_after(naive_heat_kernel<8>, grid, st, op, G, (const S *)in, (S *)out); break;
+                case 4: e = launch_after(naive_heat_kernel<4>, grid, st, op, G, (const S *)in, (S *)out); break;
+                case 2: e = launch_after(naive_heat_kernel<2>, grid, st, op, G, (const S *)in, (S *)out); break;
+                default: e = launch_after(naive_heat_kernel<1>, grid, st, op, G, (const S *)in, (S *)out); break;
             }
         } else if constexpr (std::is_same<Op, HeatKahanOp<float>>::value ||
                              std::is_same<Op, HeatKahanOp<__nv_bfloat16>>::value) {
@@ -138,17 +154,17 @@ struct Launch {
             dim3 grid((unsigned)chunks, (warps + 7) / 8);
             const Op op(c);
             switch (rows) {
-                case 16: naive_heat_kahan_kernel<S, 16><<<grid, kBlock, 0, st>>>(op, G, (const S *)in, (S *)out); break;
-                case 8: naive_heat_kahan_kernel<S, 8><<<grid, kBlock, 0, st>>>(op, G, (const S *)in, (S *)out); break;
-                case 4: naive_heat_kahan_kernel<S, 4><<<grid, kBlock, 0, st>>>(op, G, (const S *)in, (S *)out); break;
-                case 2: naive_heat_kahan_kernel<S, 2><<<grid, kBlock, 0, st>>>(op, G, (const S *)in, (S *)out); break;
-                default: naive_heat_kahan_kernel<S, 1><<<grid, kBlock, 0, st>>>(op, G, (const S *)in, (S *)out); break;
+                case 16: e = launch_after(naive_heat_kahan_kernel<S, 16>, grid, st, op, G, (const S *)in, (S *)out); break;
+                case 8: e = launch_after(naive_heat_kahan_kernel<S, 8>, grid, st, op, G, (const S *)in, (S *)out); break;
+                case 4: e = launch_after(naive_heat_kahan_kernel<S, 4>, grid, st, op, G, (const S *)in, (S *)out); break;
+                case 2: e = launch_after(naive_heat_kahan_kernel<S, 2>, grid, st, op, G, (const S *)in, (S *)out); break;
+                default: e = launch_after(naive_heat_kahan_kernel<S, 1>, grid, st, op, G, (const S *)in, (S *)out); break;
             }
         } else {
             dim3 grid((G.nx + 31) / 32, (G.ny + 7) / 8);
-            naive_kernel<Op><<<grid, kBlock, 0, st>>>(Op(c), G, (const S *)in, (S *)out, g);
+            e = launch_after(naive_kernel<Op>, grid, st, Op(c), G, (const S *)in, (S *)out, g);
         }
-        return cudaGetLastError();
+        return e;
     }
     static cudaError_t up(const Geom &G, const double *c, const void *state, void *up, int o,
                           u64 g0, cudaStream_t st) {

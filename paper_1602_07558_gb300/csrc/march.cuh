@@ -352,8 +352,7 @@ struct HeatMarch {
         read();
         bool done = false;
         if constexpr (kFixed) {
-            // the block's extremes (upper words: of negative values, too, the larger
-            // word is the larger magnitude) decide on the unit
+            // the block's extremes decide on the unit
             int high = INT_MIN, low = INT_MAX;
 #pragma unroll
             for (int j = 0; j < R; ++j) {
@@ -373,12 +372,8 @@ struct HeatMarch {
                 high = max(high, sm.high[w]);
                 low = min(low, sm.low[w]);
             }
-            const int top = (high >> 20) & 0x7ff, bottom = (low >> 20) & 0x7ff;
-            FixedCell fixed{{heat_ratio(op.r), top - (kFixedBinades - 1),
-                             (unsigned)high & 0x80000000u, 0u}};
-            // one sign, normal, six binades at most, sums and the unit in range
-            if (fixed.f.R != 0 && (high ^ low) >= 0 && bottom >= fixed.f.e0 && fixed.f.e0 > 0 &&
-                top < 2040) {
+            FixedCell fixed;
+            if (fixed.f.fits(op.r, high, low)) {
                 L2 v[R], none[1];
 #pragma unroll
                 for (int j = 0; j < R; ++j) v[j] = two(fixed.f.from(u[j].l), fixed.f.from(u[j].h));

@@ -160,3 +160,17 @@ def test_euler_batch_of_uneven_grids_matches_the_single_grids():
                 s.set_state(u)
                 s.advance(7, mode="naive")
                 assert np.array_equal(g, s.get_state())
+
+
+@pytest.mark.parametrize("nx,ny", [(1, 1), (2, 3), (29, 31), (30, 33), (31, 8), (61, 700), (1009, 757)])
+@pytest.mark.parametrize("kind", ["one_binade", "crossing", "noise"])
+def test_naive_heat_rows_and_launches_match_the_oracle(oracle_lib, kind, nx, ny):
+    """The naive kernel's column chunks and rows a warp (one, FP64 only, to
+    eight), in launches that follow each other without a gap, also in a graph."""
+    u0 = field(kind, nx, ny) if kind == "noise" or min(nx, ny) > 2 else np.full((ny, nx), 1.25)
+    ref = oracle_lib.heat(u0, 0.2, 13)
+    with Swept2D(nx, ny, op="heat", tile=0, params=(0.2,), stream=torch.cuda.Stream()) as s:
+        for graph in (False, True):
+            s.set_state(u0[None])
+            s.advance(13, mode="naive", graph=graph)
+            assert np.array_equal(s.get_state()[0], ref)
