@@ -251,6 +251,13 @@ __device__ __forceinline__ void mbar_inval(unsigned long long *bar) {
     asm volatile("mbarrier.inval.shared::cta.b64 [%0];\n" ::"r"(smem_u32(bar)) : "memory");
 }
 
+// A launch of the naive or the swept kernels may begin when the blocks of the one before it have left
+// (launch_after): this waits until that one's results, which the kernel reads,
+// are in memory.
+__device__ __forceinline__ void after_previous_launch() {
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");
+}
+
 // The threads that run one tile work item: the whole block (BlockTeam: every
 // kernel of the single-grid and per-class paths), or one of the block's teams
 // of T threads (TeamOf<T>: the one-launch batch kernel, whose blocks, sized for
@@ -797,13 +804,6 @@ __device__ __forceinline__ void write_up_panels(const S *cur, int P, const Geom 
 }
 
 // ---------------------------------------------------------------- naive path
-// A naive launch may begin when the blocks of the one before it have left
-// (launch_after): this waits until that one's results, which the kernel reads,
-// are in memory.
-__device__ __forceinline__ void after_previous_launch() {
-    asm volatile("griddepcontrol.wait;\n" ::: "memory");
-}
-
 // One sub-step over the whole grid: out = St(in) at every point.
 template <class Op>
 __global__ void __launch_bounds__(256) naive_kernel(Op op, Geom G, const typename Op::S *in,
@@ -979,6 +979,7 @@ __device__ __forceinline__ void up_tile(const Op &op, const Geom &G, const typen
 template <class Op, int NC = 0>
 __global__ void __launch_bounds__(SweptBounds<Op>::kThreads, SweptBounds<Op>::kMinBlocks)
 up_kernel(Op op, Geom G, const typename Op::S *state, typename Op::S *up, int o, u64 g0) {
+    after_previous_launch();
     up_tile(op, fixed_tile<NC>(G), state, up, o, g0, blockIdx.x, blockIdx.y);
 }
 
@@ -1135,6 +1136,7 @@ __device__ __forceinline__ void bridge_tile(const Op &op, const Geom &G, const t
 template <class Op, bool STG, int NC = 0>
 __global__ void __launch_bounds__(SweptBounds<Op>::kThreads, SweptBounds<Op>::kMinBlocks)
 bridge_kernel(Op op, Geom G, const typename Op::S *up, typename Op::S *br, u64 g0, int *err) {
+    after_previous_launch();
     bridge_tile<Op, STG>(op, fixed_tile<NC>(G), up, br, g0, err, blockIdx.x, blockIdx.y,
                          blockIdx.z == 1);
 }
@@ -1304,6 +1306,7 @@ template <class Op, bool STG, int NC = 0>
 __global__ void __launch_bounds__(SweptBounds<Op>::kThreads, SweptBounds<Op>::kMinBlocks)
 octahedron_kernel(Op op, Geom G, const typename Op::S *br, typename Op::S *up, int o, u64 g0,
                   int *err) {
+    after_previous_launch();
     octahedron_tile<Op, STG>(op, fixed_tile<NC>(G), br, up, o, g0, err, blockIdx.x, blockIdx.y);
 }
 
@@ -1336,6 +1339,7 @@ template <class Op, bool STG, int NC = 0>
 __global__ void __launch_bounds__(SweptBounds<Op>::kThreads, SweptBounds<Op>::kMinBlocks)
 down_kernel(Op op, Geom G, const typename Op::S *br, typename Op::S *state, int o, u64 g0,
             int *err) {
+    after_previous_launch();
     down_tile<Op, STG>(op, fixed_tile<NC>(G), br, state, o, g0, err, blockIdx.x, blockIdx.y);
 }
 

@@ -108,17 +108,19 @@ inline cudaError_t allow_smem(K kernel, size_t bytes) {
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
-// Launches a naive kernel so that its blocks may be set up while the stream's
-// launch before it still runs; the kernel itself waits for that one's end
-// (after_previous_launch).
+// Launches a naive or swept kernel so that it may begin as soon as the blocks of
+// the stream's launch before it have left; the kernel itself waits for that one's
+// results (after_previous_launch).
 template <class... P, class... A>
-inline cudaError_t launch_after(void (*kernel)(P...), dim3 grid, cudaStream_t st, A... args) {
+inline cudaError_t launch_after(void (*kernel)(P...), dim3 grid, int block, size_t smem,
+                                cudaStream_t st, A... args) {
     cudaLaunchAttribute at{};
     at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at.val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid;
-    cfg.blockDim = dim3(kBlock);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
@@ -140,10 +142,10 @@ struct Launch {
             dim3 grid((unsigned)chunks, (warps + 7) / 8);
             const Op op(c);
             switch (rows) {
-                case 8: e = launch_after(naive_heat_kernel<8>, grid, st, op, G, (const S *)in, (S *)out); break;
-                case 4: e = launch_after(naive_heat_kernel<4>, grid, st, op, G, (const S *)in, (S *)out); break;
-                case 2: e = launch_after(naive_heat_kernel<2>, grid, st, op, G, (const S *)in, (S *)out); break;
-                default: e = launch_after(naive_heat_kernel<1>, grid, st, op, G, (const S *)in, (S *)out); break;
+                case 8: e = launch_after(naive_heat_kernel<8>, grid, kBlock, 0, st, op, G, (const S *)in, (S *)out); break;
+                case 4: e = launch_after(naive_heat_kernel<4>, grid, kBlock, 0, st, op, G, (const S *)in, (S *)out); break;
+                case 2: e = launch_after(naive_heat_kernel<2>, grid, kBlock, 0, st, op, G, (const S *)in, (S *)out); break;
+                default: e = launch_after(naive_heat_kernel<1>, grid, kBlock, 0, st, op, G, (const S *)in, (S *)out); break;
             }
         } else if constexpr (std::is_same<Op, HeatKahanOp<float>>::value ||
                              std::is_same<Op, HeatKahanOp<__nv_bfloat16>>::value) {
@@ -154,15 +156,15 @@ struct Launch {
             dim3 grid((unsigned)chunks, (warps + 7) / 8);
             const Op op(c);
             switch (rows) {
-                case 16: e = launch_after(naive_heat_kahan_kernel<S, 16>, grid, st, op, G, (const S *)in, (S *)out); break;
-                case 8: e = launch_after(naive_heat_kahan_kernel<S, 8>, grid, st, op, G, (const S *)in, (S *)out); break;
-                case 4: e = launch_after(naive_heat_kahan_kernel<S, 4>, grid, st, op, G, (const S *)in, (S *)out); break;
-                case 2: e = launch_after(naive_heat_kahan_kernel<S, 2>, grid, st, op, G, (const S *)in, (S *)out); break;
-                default: e = launch_after(naive_heat_kahan_kernel<S, 1>, grid, st, op, G, (const S *)in, (S *)out); break;
+                case 16: e = launch_after(naive_heat_kahan_kernel<S, 16>, grid, kBlock, 0, st, op, G, (const S *)in, (S *)out); break;
+                case 8: e = launch_after(naive_heat_kahan_kernel<S, 8>, grid, kBlock, 0, st, op, G, (const S *)in, (S *)out); break;
+                case 4: e = launch_after(naive_heat_kahan_kernel<S, 4>, grid, kBlock, 0, st, op, G, (const S *)in, (S *)out); break;
+                case 2: e = launch_after(naive_heat_kahan_kernel<S, 2>, grid, kBlock, 0, st, op, G, (const S *)in, (S *)out); break;
+                default: e = launch_after(naive_heat_kahan_kernel<S, 1>, grid, kBlock, 0, st, op, G, (const S *)in, (S *)out); break;
             }
         } else {
             dim3 grid((G.nx + 31) / 32, (G.ny + 7) / 8);
-            e = launch_after(naive_kernel<Op>, grid, st, Op(c), G, (const S *)in, (S *)out, g);
+            e = launch_after(naive_kernel<Op>, grid, kBlock, 0, st, Op(c), G, (const S *)in, (S *)out, g);
         }
         return e;
     }
@@ -173,9 +175,8 @@ struct Launch {
             constexpr int NC = decltype(nc)::value;
             cudaError_t e = allow_smem(up_kernel<Op, NC>, sm);
             if (e != cudaSuccess) return e;
-            up_kernel<Op, NC><<<dim3(G.T, G.Q), kBlock, sm, st>>>(Op(c), G, (const S *)state,
-                                                                  (S *)up, o, g0);
-            return cudaGetLastError();
+            return launch_after(up_kernel<Op, NC>, dim3(G.T, G.Q), kBlock, sm, st, Op(c), G,
+                                (const S *)state, (S *)up, o, g0);
         });
     }
     template <bool STG>
@@ -186,9 +187,8 @@ struct Launch {
             constexpr int NC = decltype(nc)::value;
             cudaError_t e = allow_smem(bridge_kernel<Op, STG, NC>, sm);
             if (e != cudaSuccess) return e;
-            bridge_kernel<Op, STG, NC><<<dim3(G.T, G.Q, 2), threads, sm, st>>>(
-                Op(c), G, (const S *)up, (S *)br, g0, err);
-            return cudaGetLastError();
+            return launch_after(bridge_kernel<Op, STG, NC>, dim3(G.T, G.Q, 2), threads, sm, st,
+                                Op(c), G, (const S *)up, (S *)br, g0, err);
         });
     }
     // A bridge's levels are thin rectangles (W + H = n), and its block is
@@ -212,9 +212,8 @@ struct Launch {
             constexpr int NC = decltype(nc)::value;
             cudaError_t e = allow_smem(octahedron_kernel<Op, STG, NC>, sm);
             if (e != cudaSuccess) return e;
-            octahedron_kernel<Op, STG, NC><<<dim3(G.T, G.Q), threads, sm, st>>>(
-                Op(c), G, (const S *)br, (S *)up, o, g0, err);
-            return cudaGetLastError();
+            return launch_after(octahedron_kernel<Op, STG, NC>, dim3(G.T, G.Q), threads, sm, st,
+                                Op(c), G, (const S *)br, (S *)up, o, g0, err);
         });
     }
     static cudaError_t octahedron(const Geom &G, const double *c, const void *br, void *up, int o,
@@ -230,9 +229,8 @@ struct Launch {
             constexpr int NC = decltype(nc)::value;
             cudaError_t e = allow_smem(down_kernel<Op, STG, NC>, sm);
             if (e != cudaSuccess) return e;
-            down_kernel<Op, STG, NC><<<dim3(G.T, G.Q), threads, sm, st>>>(
-                Op(c), G, (const S *)br, (S *)state, o, g0, err);
-            return cudaGetLastError();
+            return launch_after(down_kernel<Op, STG, NC>, dim3(G.T, G.Q), threads, sm, st, Op(c),
+                                G, (const S *)br, (S *)state, o, g0, err);
         });
     }
     static cudaError_t down(const Geom &G, const double *c, const void *br, void *state, int o,

@@ -216,7 +216,7 @@ struct EulerKahanOp {
 // C2 = (c dt / dx)^2 is formed on the host. 2u - u^{n-1} is one fused operation,
 // with the bits of the two: 2u is exact unless it overflows, which the last
 // binade's u do, to an infinity. A sixth FP64 operation a point saved for four
-// integer instructions (the 1024² grid: 15.0 to 13.0 ms for 1,000 steps).
+// integer instructions (the 1024² grid: 14.9 to 13.0 ms for 1,000 steps).
 struct WaveOp {
     typedef double S;
     static constexpr int NV = 2, NST = 1, AUX = 1;   // aux: pair sums of a level
