@@ -15,8 +15,7 @@ namespace swept {
 
 // Tile and block tables hold (grid index, tile or block index within the grid).
 
-// NC > 0: every grid of the launch's class has tile side NC (see fixed_tile).
-template <class Op, int NC = 0>
+template <class Op>
 __global__ void __launch_bounds__(kMaxSweptThreads) batch_up_kernel(const GridDesc *grids,
                                                                     const int2 *tile_grid,
                                                                     const typename Op::S *state,
@@ -25,10 +24,10 @@ __global__ void __launch_bounds__(kMaxSweptThreads) batch_up_kernel(const GridDe
     const int2 e = tile_grid[blockIdx.x];
     const GridDesc gd = grids[e.x];
     const int J = e.y / gd.G.T, I = e.y - J * gd.G.T;
-    up_tile(Op(gd.c), fixed_tile<NC>(gd.G), state + gd.state_off, up + gd.panel_off, o, g0, I, J);
+    up_tile(Op(gd.c), gd.G, state + gd.state_off, up + gd.panel_off, o, g0, I, J);
 }
 
-template <class Op, bool STG, int NC = 0>
+template <class Op, bool STG>
 __global__ void __launch_bounds__(kMaxSweptThreads) batch_bridge_kernel(const GridDesc *grids,
                                                                         const int2 *tile_grid,
                                                                         const typename Op::S *up,
@@ -37,29 +36,29 @@ __global__ void __launch_bounds__(kMaxSweptThreads) batch_bridge_kernel(const Gr
     const int2 e = tile_grid[blockIdx.x];
     const GridDesc gd = grids[e.x];
     const int J = e.y / gd.G.T, I = e.y - J * gd.G.T;
-    bridge_tile<Op, STG>(Op(gd.c), fixed_tile<NC>(gd.G), up + gd.panel_off, br + gd.panel_off,
+    bridge_tile<Op, STG>(Op(gd.c), gd.G, up + gd.panel_off, br + gd.panel_off,
                          g0, err, I, J, blockIdx.y == 1);
 }
 
-template <class Op, bool STG, int NC = 0>
+template <class Op, bool STG>
 __global__ void __launch_bounds__(kMaxSweptThreads) batch_octahedron_kernel(
     const GridDesc *grids, const int2 *tile_grid, const typename Op::S *br, typename Op::S *up,
     int o, u64 g0, int *err) {
     const int2 e = tile_grid[blockIdx.x];
     const GridDesc gd = grids[e.x];
     const int J = e.y / gd.G.T, I = e.y - J * gd.G.T;
-    octahedron_tile<Op, STG>(Op(gd.c), fixed_tile<NC>(gd.G), br + gd.panel_off,
+    octahedron_tile<Op, STG>(Op(gd.c), gd.G, br + gd.panel_off,
                              up + gd.panel_off, o, g0, err, I, J);
 }
 
-template <class Op, bool STG, int NC = 0>
+template <class Op, bool STG>
 __global__ void __launch_bounds__(kMaxSweptThreads) batch_down_kernel(
     const GridDesc *grids, const int2 *tile_grid, const typename Op::S *br, typename Op::S *state,
     int o, u64 g0, int *err) {
     const int2 e = tile_grid[blockIdx.x];
     const GridDesc gd = grids[e.x];
     const int J = e.y / gd.G.T, I = e.y - J * gd.G.T;
-    down_tile<Op, STG>(Op(gd.c), fixed_tile<NC>(gd.G), br + gd.panel_off, state + gd.state_off,
+    down_tile<Op, STG>(Op(gd.c), gd.G, br + gd.panel_off, state + gd.state_off,
                        o, g0, err, I, J);
 }
 
@@ -84,12 +83,12 @@ struct GridTiles {
     }
 };
 
-template <class Op, bool STG, int NC = 0>
+template <class Op, bool STG>
 __global__ void __launch_bounds__(256) batch_persistent_kernel(
     const GridDesc *grids, const int2 *tile_grid, int ntiles, int n, typename Op::S *state,
     typename Op::S *up, typename Op::S *br, int *stage, int *queue, int H, u64 g0, int *err) {
     // the update's constants come from each item's grid (TileAt::c)
-    persistent_loop<Op, STG, NC>(Op(grids[0].c), GridTiles{grids, tile_grid}, ntiles, n, state,
+    persistent_loop<Op, STG>(Op(grids[0].c), GridTiles{grids, tile_grid}, ntiles, n, state,
                                  up, br, stage, queue, H, g0, err, 0, kPersistSpinLimit);
 }
 
@@ -98,7 +97,7 @@ __global__ void __launch_bounds__(256) batch_persistent_kernel(
 // barrier and shared-memory slice, or the whole block) each take the class's
 // items, one at a time, from the class's own counter, and run them as that
 // class's own launch would (its tile table, counters, tile side and number of
-// half cycles; the tile side fixed at compile time for 16, 32 and 64). A block
+// half cycles). A block
 // goes on to the next class once its teams find the class's counter past its
 // last item, so the classes overlap at the class boundaries. An item waits
 // only for the same class's earlier items, handed out before it and held by
@@ -118,27 +117,19 @@ struct ClassRuns {
 
 // Threads of the one-launch kernel's blocks, and the team that runs one item
 // of a class with tile side n (0: the whole block). Small tiles, whose levels
-// are short, run several per block: heat in binary32 / bfloat16 one warp per
-// tile-16 item and four per tile-32 item; the other updates two warps per
-// tile-16 item (their tile-16 slice is 4x larger). Larger tiles take the block.
+// are short, run several per block: two warps per tile-16 item. Larger tiles take
+// the block.
 constexpr int kOneLaunchThreads = 256;
-template <class Op>
-__host__ __device__ constexpr int one_launch_team(int n) {
-    if constexpr (std::is_same<Op, HeatKahanOp<float>>::value ||
-                  std::is_same<Op, HeatKahanOp<__nv_bfloat16>>::value)
-        return n <= 16 ? 32 : (n <= 32 ? 128 : 0);
-    else
-        return n <= 16 ? 64 : 0;
-}
+__host__ __device__ constexpr int one_launch_team(int n) { return n <= 16 ? 64 : 0; }
 // Shared memory of a one-launch block for a class of tile side n: its teams'
 // slices, or one swept block.
 template <class Op, bool STG>
 inline size_t one_launch_class_smem(int n) {
-    const int T = one_launch_team<Op>(n);
+    const int T = one_launch_team(n);
     return T ? (size_t)(kOneLaunchThreads / T) * team_slice<Op, STG>(n) : down_smem<Op>(n, STG);
 }
 
-template <class Op, bool STG, int NC, class Tm>
+template <class Op, bool STG, class Tm>
 __device__ __forceinline__ bool run_class(const GridDesc *grids, const ClassRun &c,
                                           typename Op::S *state, typename Op::S *up,
                                           typename Op::S *br, u64 g0, int *err) {
@@ -154,24 +145,11 @@ __device__ __forceinline__ bool run_class(const GridDesc *grids, const ClassRun 
         Tm::sync();
         const int item = mine;
         if (item >= nitems) return true;
-        if (!persistent_item<Op, STG, NC, Tm>(Op(grids[0].c), GridTiles{grids, c.tiles},
+        if (!persistent_item<Op, STG, Tm>(Op(grids[0].c), GridTiles{grids, c.tiles},
                                               c.ntiles, c.n, state, up, br, c.stage, c.H, g0,
                                               err, item, kPersistSpinLimit, nullptr))
             return false;
     }
-}
-
-// The team for tile side N (a compile-time case of the class's side)
-template <class Op, bool STG, int N>
-__device__ __forceinline__ bool run_class_n(const GridDesc *grids, const ClassRun &c,
-                                            typename Op::S *state, typename Op::S *up,
-                                            typename Op::S *br, u64 g0, int *err) {
-    constexpr int NC = FixedTiles<Op>::value ? N : 0;
-    constexpr int T = one_launch_team<Op>(N);
-    if constexpr (T > 0 && T < kOneLaunchThreads)
-        return run_class<Op, STG, NC, TeamOf<T>>(grids, c, state, up, br, g0, err);
-    else
-        return run_class<Op, STG, NC, BlockTeam>(grids, c, state, up, br, g0, err);
 }
 
 template <class Op, bool STG>
@@ -181,14 +159,10 @@ __global__ void __launch_bounds__(kOneLaunchThreads) batch_persistent_all_kernel
     for (int k = 0; k < runs.count; ++k) {
         const ClassRun c = runs.r[k];
         bool ok;
-        switch (c.n) {
-            case 16: ok = run_class_n<Op, STG, 16>(grids, c, state, up, br, g0, err); break;
-            case 32: ok = run_class_n<Op, STG, 32>(grids, c, state, up, br, g0, err); break;
-            case 64: ok = run_class_n<Op, STG, 64>(grids, c, state, up, br, g0, err); break;
-            default:
-                ok = run_class<Op, STG, 0, BlockTeam>(grids, c, state, up, br, g0, err);
-                break;
-        }
+        if (one_launch_team(c.n))
+            ok = run_class<Op, STG, TeamOf<one_launch_team(16)>>(grids, c, state, up, br, g0, err);
+        else
+            ok = run_class<Op, STG, BlockTeam>(grids, c, state, up, br, g0, err);
         // every team of the block leaves the class before the team shape changes
         if (__syncthreads_or(!ok)) return;
     }
@@ -263,28 +237,22 @@ struct BatchLaunch {
     static cudaError_t up(const GridDesc *d, const int2 *tg, int ntiles, int n, const void *state,
                           void *upp, int o, u64 g0, cudaStream_t st) {
         const size_t sm = up_smem<Op>(n);
-        return with_tile<Op>(n, [&](auto nc) {
-            constexpr int NC = decltype(nc)::value;
-            cudaError_t e = allow_smem(batch_up_kernel<Op, NC>, sm);
-            if (e != cudaSuccess) return e;
-            batch_up_kernel<Op, NC><<<ntiles, kBlock, sm, st>>>(d, tg, (const S *)state, (S *)upp,
-                                                                o, g0);
-            return cudaGetLastError();
-        });
+        cudaError_t e = allow_smem(batch_up_kernel<Op>, sm);
+        if (e != cudaSuccess) return e;
+        batch_up_kernel<Op><<<ntiles, kBlock, sm, st>>>(d, tg, (const S *)state, (S *)upp,
+                                                            o, g0);
+        return cudaGetLastError();
     }
     template <bool STG>
     static cudaError_t bridge_t(const GridDesc *d, const int2 *tg, int ntiles, int n,
                                 const void *upp, void *br, u64 g0, int *err, int threads,
                                 cudaStream_t st) {
         const size_t sm = bridge_smem<Op>(n, STG);
-        return with_tile<Op>(n, [&](auto nc) {
-            constexpr int NC = decltype(nc)::value;
-            cudaError_t e = allow_smem(batch_bridge_kernel<Op, STG, NC>, sm);
-            if (e != cudaSuccess) return e;
-            batch_bridge_kernel<Op, STG, NC><<<dim3(ntiles, 2), threads, sm, st>>>(
-                d, tg, (const S *)upp, (S *)br, g0, err);
-            return cudaGetLastError();
-        });
+        cudaError_t e = allow_smem(batch_bridge_kernel<Op, STG>, sm);
+        if (e != cudaSuccess) return e;
+        batch_bridge_kernel<Op, STG><<<dim3(ntiles, 2), threads, sm, st>>>(
+            d, tg, (const S *)upp, (S *)br, g0, err);
+        return cudaGetLastError();
     }
     static cudaError_t bridge(const GridDesc *d, const int2 *tg, int ntiles, int n,
                               const void *upp, void *br, u64 g0, int *err, const Tuning &tn,
@@ -296,14 +264,11 @@ struct BatchLaunch {
     static cudaError_t oct_t(const GridDesc *d, const int2 *tg, int ntiles, int n, const void *br,
                              void *upp, int o, u64 g0, int *err, int threads, cudaStream_t st) {
         const size_t sm = down_smem<Op>(n, STG);
-        return with_tile<Op>(n, [&](auto nc) {
-            constexpr int NC = decltype(nc)::value;
-            cudaError_t e = allow_smem(batch_octahedron_kernel<Op, STG, NC>, sm);
-            if (e != cudaSuccess) return e;
-            batch_octahedron_kernel<Op, STG, NC><<<ntiles, threads, sm, st>>>(
-                d, tg, (const S *)br, (S *)upp, o, g0, err);
-            return cudaGetLastError();
-        });
+        cudaError_t e = allow_smem(batch_octahedron_kernel<Op, STG>, sm);
+        if (e != cudaSuccess) return e;
+        batch_octahedron_kernel<Op, STG><<<ntiles, threads, sm, st>>>(
+            d, tg, (const S *)br, (S *)upp, o, g0, err);
+        return cudaGetLastError();
     }
     static cudaError_t octahedron(const GridDesc *d, const int2 *tg, int ntiles, int n,
                                   const void *br, void *upp, int o, u64 g0, int *err,
@@ -315,14 +280,11 @@ struct BatchLaunch {
     static cudaError_t down_t(const GridDesc *d, const int2 *tg, int ntiles, int n, const void *br,
                               void *state, int o, u64 g0, int *err, int threads, cudaStream_t st) {
         const size_t sm = down_smem<Op>(n, STG);
-        return with_tile<Op>(n, [&](auto nc) {
-            constexpr int NC = decltype(nc)::value;
-            cudaError_t e = allow_smem(batch_down_kernel<Op, STG, NC>, sm);
-            if (e != cudaSuccess) return e;
-            batch_down_kernel<Op, STG, NC><<<ntiles, threads, sm, st>>>(d, tg, (const S *)br,
-                                                                        (S *)state, o, g0, err);
-            return cudaGetLastError();
-        });
+        cudaError_t e = allow_smem(batch_down_kernel<Op, STG>, sm);
+        if (e != cudaSuccess) return e;
+        batch_down_kernel<Op, STG><<<ntiles, threads, sm, st>>>(d, tg, (const S *)br,
+                                                                    (S *)state, o, g0, err);
+        return cudaGetLastError();
     }
     static cudaError_t down(const GridDesc *d, const int2 *tg, int ntiles, int n, const void *br,
                             void *state, int o, u64 g0, int *err, const Tuning &tn,
@@ -335,23 +297,20 @@ struct BatchLaunch {
                                     void *state, void *upp, void *br, int *sched, int H, u64 g0,
                                     int *err, int threads, cudaStream_t st) {
         const size_t sm = down_smem<Op>(n, STG);
-        return with_tile<Op>(n, [&](auto nc) {
-            constexpr int NC = decltype(nc)::value;
-            const auto kern = batch_persistent_kernel<Op, STG, NC>;
-            cudaError_t e = allow_smem(kern, sm);
-            if (e != cudaSuccess) return e;
-            int per_sm = 0, dev = 0, nsm = 0;
-            if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, sm)) !=
-                cudaSuccess)
-                return e;
-            cudaGetDevice(&dev);
-            cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-            const long long grid =
-                persistent_grid(per_sm, nsm, ntiles, persistent_items(ntiles, H));
-            kern<<<(int)grid, threads, sm, st>>>(d, tg, ntiles, n, (S *)state, (S *)upp, (S *)br,
-                                                 sched, sched + ntiles, H, g0, err);
-            return cudaGetLastError();
-        });
+        const auto kern = batch_persistent_kernel<Op, STG>;
+        cudaError_t e = allow_smem(kern, sm);
+        if (e != cudaSuccess) return e;
+        int per_sm = 0, dev = 0, nsm = 0;
+        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, sm)) !=
+            cudaSuccess)
+            return e;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+        const long long grid =
+            persistent_grid(per_sm, nsm, ntiles, persistent_items(ntiles, H));
+        kern<<<(int)grid, threads, sm, st>>>(d, tg, ntiles, n, (S *)state, (S *)upp, (S *)br,
+                                             sched, sched + ntiles, H, g0, err);
+        return cudaGetLastError();
     }
     static cudaError_t persistent(const GridDesc *d, const int2 *tg, int ntiles, int n,
                                   void *state, void *upp, void *br, int *sched, int H, u64 g0,

@@ -72,17 +72,6 @@ struct GridDesc {
 
 __host__ __device__ inline int panel_stride(int n) { return ((n * n / 2 + n) + 7) & ~7; }
 
-// The geometry a swept kernel works with: NC > 0 fixes the tile side at compile
-// time (the launch picks such an instantiation only when G.n == NC), so every
-// shared-memory pitch and plane offset of the inlined level code is a constant
-// and folds into the load and store instructions; NC = 0 keeps G.n.
-template <int NC>
-__device__ __forceinline__ Geom fixed_tile(const Geom &G) {
-    Geom g = G;
-    if constexpr (NC > 0) g.n = NC;
-    return g;
-}
-
 // Updates whose levels are computed in place in one level buffer.
 template <class Op>
 __host__ __device__ constexpr bool one_buffer() { return Op::INPLACE || Op::INPLACE_AFTER_AUX; }
@@ -282,25 +271,17 @@ struct TeamOf {
     __device__ __forceinline__ static unsigned size() { return T; }
     __device__ __forceinline__ static int index() { return (int)threadIdx.x / T; }
     __device__ __forceinline__ static void sync() {
-        if constexpr (T == 32)
-            __syncwarp();
-        else
-            asm volatile("bar.sync %0, %1;\n" ::"r"(1 + index()), "n"(T) : "memory");
+        asm volatile("bar.sync %0, %1;\n" ::"r"(1 + index()), "n"(T) : "memory");
     }
     __device__ __forceinline__ static int sync_or(int p) {
-        if constexpr (T == 32) {
-            __syncwarp();
-            return __any_sync(0xffffffffu, p);
-        } else {
-            int r;
-            asm volatile(
-                "{\n .reg .pred q, o;\n setp.ne.s32 q, %1, 0;\n"
-                " bar.red.or.pred o, %2, %3, q;\n selp.s32 %0, 1, 0, o;\n}\n"
-                : "=r"(r)
-                : "r"(p), "r"(1 + index()), "n"(T)
-                : "memory");
-            return r;
-        }
+        int r;
+        asm volatile(
+            "{\n .reg .pred q, o;\n setp.ne.s32 q, %1, 0;\n"
+            " bar.red.or.pred o, %2, %3, q;\n selp.s32 %0, 1, 0, o;\n}\n"
+            : "=r"(r)
+            : "r"(p), "r"(1 + index()), "n"(T)
+            : "memory");
+        return r;
     }
 };
 
@@ -483,67 +464,6 @@ __device__ __forceinline__ void compute_rect_mid(const HeatOp &op, int, u64, con
         const double sum = __dadd_rn(aux[a + W1 + 1], aux[a]);
         dst[off] = __fma_rn(op.r, __fma_rn(-4.0, c, sum), c);
     }
-}
-
-// Reduced-precision heat: each thread updates a column strip of up to R
-// points of the rectangle. All of the strip's loads (R + 2 centre-column
-// values, R compensations, R east and R west values: 4 per point instead of 6)
-// are issued before its R independent updates, so they overlap, and the index
-// walk runs once per strip; full strips take a path without per-row guards.
-// Same values as HeatKahanOp::operator().
-template <class SS, int R, bool FULL>
-__device__ __forceinline__ void heat_kahan_strip(const HeatKahanOp<SS> &op,
-                                                 const SS *__restrict__ src, SS *__restrict__ dst,
-                                                 int P, int plane, int off, int rows) {
-    typedef Store<SS> St;
-    float u[R + 2], cv[R], ue[R], uw[R];
-#pragma unroll
-    for (int r = 0; r < R + 2; ++r)              // u[r]: row r - 1 of the strip, -1 .. rows
-        u[r] = (FULL || r <= rows + 1) ? St::ld(src[off + (r - 1) * P]) : 0.0f;
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-        const int o = off + r * P;
-        const bool in = FULL || r < rows;
-        cv[r] = in ? St::ld(src[plane + o]) : 0.0f;
-        ue[r] = in ? St::ld(src[o + 1]) : 0.0f;
-        uw[r] = in ? St::ld(src[o - 1]) : 0.0f;
-    }
-#pragma unroll
-    for (int r = 0; r < R; ++r)
-        if (FULL || r < rows)
-            op.update(u[r + 1], cv[r], ue[r], u[r + 2], uw[r], u[r], dst[off + r * P],
-                      dst[plane + off + r * P]);
-}
-
-template <class Tm, int R, class SS>
-__device__ __forceinline__ void heat_kahan_rect(const HeatKahanOp<SS> &op,
-                                                const SS *__restrict__ src, SS *__restrict__ dst,
-                                                int P, int x0, int y0, int W, int H) {
-    const int plane = P * P;
-    const int nb = (H + R - 1) / R;
-    for (LinearWalk w(W, (int)Tm::rank(), (int)Tm::size()); w.yy < nb; w.next(W)) {
-        const int yb = w.yy * R;
-        const int rows = H - yb;
-        const int off = (y0 + yb + 1) * P + (x0 + w.xx + 1);
-        if (rows >= R)
-            heat_kahan_strip<SS, R, true>(op, src, dst, P, plane, off, R);
-        else
-            heat_kahan_strip<SS, R, false>(op, src, dst, P, plane, off, rows);
-    }
-}
-// Strips of 4 points at tile 64, of 2 on smaller tiles, whose short levels
-// have fewer strips to share among the threads (measured: the 1,024-grid
-// batch at tiles 16 and 32 247 -> 262 G updates/s with strips of 2, the 2048²
-// grid at tile 64 421 -> 410 with strips of 2 and 379 with strips of 8).
-template <class Tm = BlockTeam, class SS>
-__device__ __forceinline__ void compute_rect(const HeatKahanOp<SS> &op, int, u64,
-                                             const SS *__restrict__ src, SS *__restrict__ dst,
-                                             SS *, int P, int x0, int y0, int W, int H) {
-    if (W <= 0 || H <= 0) return;
-    if (P > 34)
-        heat_kahan_rect<Tm, 4>(op, src, dst, P, x0, y0, W, H);
-    else
-        heat_kahan_rect<Tm, 2>(op, src, dst, P, x0, y0, W, H);
 }
 
 // Euler: the primitives (u, v, p, E + p) of every point of the rectangle grown
@@ -976,11 +896,11 @@ __device__ __forceinline__ void up_tile(const Op &op, const Geom &G, const typen
     up_body<Op, Tm>(op, G, buf0, buf1, aux, P, g0, up, J * G.T + I, 0);
 }
 
-template <class Op, int NC = 0>
+template <class Op>
 __global__ void __launch_bounds__(SweptBounds<Op>::kThreads, SweptBounds<Op>::kMinBlocks)
 up_kernel(Op op, Geom G, const typename Op::S *state, typename Op::S *up, int o, u64 g0) {
     after_previous_launch();
-    up_tile(op, fixed_tile<NC>(G), state, up, o, g0, blockIdx.x, blockIdx.y);
+    up_tile(op, G, state, up, o, g0, blockIdx.x, blockIdx.y);
 }
 
 // ------------------------------------------- Bridges (Algorithms 2 and 3)
@@ -1133,11 +1053,11 @@ __device__ __forceinline__ void bridge_tile(const Op &op, const Geom &G, const t
     }
 }
 
-template <class Op, bool STG, int NC = 0>
+template <class Op, bool STG>
 __global__ void __launch_bounds__(SweptBounds<Op>::kThreads, SweptBounds<Op>::kMinBlocks)
 bridge_kernel(Op op, Geom G, const typename Op::S *up, typename Op::S *br, u64 g0, int *err) {
     after_previous_launch();
-    bridge_tile<Op, STG>(op, fixed_tile<NC>(G), up, br, g0, err, blockIdx.x, blockIdx.y,
+    bridge_tile<Op, STG>(op, G, up, br, g0, err, blockIdx.x, blockIdx.y,
                          blockIdx.z == 1);
 }
 
@@ -1302,12 +1222,12 @@ __device__ __forceinline__ void octahedron_tile(const Op &op, const Geom &G,
     up_body<Op, Tm>(op, G, buf0, buf1, aux, P, g0 + h, up, J * G.T + I, h & 1);
 }
 
-template <class Op, bool STG, int NC = 0>
+template <class Op, bool STG>
 __global__ void __launch_bounds__(SweptBounds<Op>::kThreads, SweptBounds<Op>::kMinBlocks)
 octahedron_kernel(Op op, Geom G, const typename Op::S *br, typename Op::S *up, int o, u64 g0,
                   int *err) {
     after_previous_launch();
-    octahedron_tile<Op, STG>(op, fixed_tile<NC>(G), br, up, o, g0, err, blockIdx.x, blockIdx.y);
+    octahedron_tile<Op, STG>(op, G, br, up, o, g0, err, blockIdx.x, blockIdx.y);
 }
 
 // K4: final Down of an advance; writes the tile at level h to the state.
@@ -1335,12 +1255,12 @@ __device__ __forceinline__ void down_tile(const Op &op, const Geom &G, const typ
     }
 }
 
-template <class Op, bool STG, int NC = 0>
+template <class Op, bool STG>
 __global__ void __launch_bounds__(SweptBounds<Op>::kThreads, SweptBounds<Op>::kMinBlocks)
 down_kernel(Op op, Geom G, const typename Op::S *br, typename Op::S *state, int o, u64 g0,
             int *err) {
     after_previous_launch();
-    down_tile<Op, STG>(op, fixed_tile<NC>(G), br, state, o, g0, err, blockIdx.x, blockIdx.y);
+    down_tile<Op, STG>(op, G, br, state, o, g0, err, blockIdx.x, blockIdx.y);
 }
 
 // ------------------------------------------------------- persistent form
@@ -1423,7 +1343,7 @@ __host__ __device__ inline long long persistent_items(long long NT, long long H)
 // One work item of the persistent form (every thread of the team calls it
 // with the same item): wait for the item's neighbourhood, run it, count it.
 // Returns false when a wait gave up (the team must stop).
-template <class Op, bool STG, int NC = 0, class Tm = BlockTeam, class Loc>
+template <class Op, bool STG, class Tm = BlockTeam, class Loc>
 __device__ __forceinline__ bool persistent_item(const Op &op, const Loc &at, int NT, int n,
                                                 typename Op::S *state, typename Op::S *upp,
                                                 typename Op::S *br, int *stage, int H, u64 g0,
@@ -1432,7 +1352,7 @@ __device__ __forceinline__ bool persistent_item(const Op &op, const Loc &at, int
     __shared__ int s_fail_team[kMaxTeams];
     int &s_fail = s_fail_team[Tm::index()];
     long long t_start = 0, t_ready = 0;
-    const int h = (NC > 0 ? NC : n) / 2;
+    const int h = n / 2;
     // decode: kind 0 first Up, 1 bridge (xb: x-bridge), 2 octahedron or Down
     int kind, t, j = 0, need = 0;
     bool xb = false;
@@ -1455,7 +1375,7 @@ __device__ __forceinline__ bool persistent_item(const Op &op, const Loc &at, int
         }
     }
     const TileAt w = at(t);
-    const Geom G = fixed_tile<NC>(w.G);
+    const Geom G = w.G;
     const int I = w.I, J = w.J;
     const Op opi = w.c ? Op(w.c) : op;
     if (Tm::rank() == 0) s_fail = 0;
@@ -1519,7 +1439,7 @@ __device__ __forceinline__ bool persistent_item(const Op &op, const Loc &at, int
     return true;
 }
 
-template <class Op, bool STG, int NC = 0, class Loc>
+template <class Op, bool STG, class Loc>
 __device__ __forceinline__ void persistent_loop(const Op &op, const Loc &at, int NT, int n,
                                                 typename Op::S *state, typename Op::S *upp,
                                                 typename Op::S *br, int *stage, int *queue, int H,
@@ -1535,19 +1455,18 @@ __device__ __forceinline__ void persistent_loop(const Op &op, const Loc &at, int
         __syncthreads();
         const int item = s_item;
         if (item >= nitems) return;
-        if (!persistent_item<Op, STG, NC>(op, at, NT, n, state, upp, br, stage, H, g0, err, item,
+        if (!persistent_item<Op, STG>(op, at, NT, n, state, upp, br, stage, H, g0, err, item,
                                           spin_limit, trace))
             return;
     }
 }
 
-template <class Op, bool STG, int NC = 0>
+template <class Op, bool STG>
 __global__ void __launch_bounds__(kMaxPersistentThreads)
 persistent_kernel(Op op, Geom G, typename Op::S *state, typename Op::S *upp, typename Op::S *br,
                   int *stage, int *queue, int H, u64 g0, int *err, int first,
                   long long spin_limit, unsigned *trace) {
-    const Geom Gf = fixed_tile<NC>(G);
-    persistent_loop<Op, STG, NC>(op, OneGrid{Gf}, Gf.T * Gf.Q, Gf.n, state, upp, br, stage, queue,
+    persistent_loop<Op, STG>(op, OneGrid{G}, G.T * G.Q, G.n, state, upp, br, stage, queue,
                                  H, g0, err, first, spin_limit, trace);
 }
 
