@@ -12,7 +12,11 @@
  * downward pyramid of one half cycle and the upward pyramid of the next act on
  * the same tile in the same frame, so they run fused in one kernel (the
  * "octahedron"): two launches per n/2 sub-steps, or one persistent launch per
- * advance (SWEPT2D_PERSISTENT). A plain one-kernel-per-sub-step path (mode
+ * advance (SWEPT2D_PERSISTENT). The heat and Euler updates' swept modes instead
+ * advance in the marching form where it is faster: one launch in which blocks
+ * take tiles of their own choice through several steps in registers, computing a
+ * ring around them redundantly (the same bits; the caller's tile side, threads
+ * and staging then only decide what is accepted). A plain one-kernel-per-sub-step path (mode
  * SWEPT2D_NAIVE) uses the same point-update code and gives bitwise identical
  * results. Many independent grids of uneven sizes share launches through the
  * swept2d_batch_* calls.
@@ -164,7 +168,7 @@ int swept2d_set_state(swept2d_t *h, const void *src, int src_is_device);
 /* Advance nsteps whole time steps (nsteps*nstages sub-steps) with mode
  * SWEPT2D_SWEPT or SWEPT2D_NAIVE. The swept mode runs
  * H = floor(nsteps*nstages / (n/2)) half cycles and the remaining sub-steps
- * with the naive kernel. Asynchronous on the handle's stream; the state is in
+ * with the naive kernel, or the marching form. Asynchronous on the handle's stream; the state is in
  * natural storage when the work completes. Errors: EINVAL (nsteps < 0, swept
  * mode on a naive-only handle), ESTATE (no set_state yet), ECUDA. */
 int swept2d_advance(swept2d_t *h, long long nsteps, int mode);
@@ -240,7 +244,8 @@ int swept2d_set_tuning(swept2d_t *h, int threads, int stage);
 #define SWEPT2D_K_COUNT       7
 int swept2d_set_timing(swept2d_t *h, int on);
 
-/* Per-item trace of the persistent form (a measurement aid; no counterpart in
+/* Per-item trace of the persistent swept form (also for the updates that
+ * otherwise march; a measurement aid; no counterpart in
  * the paper). With a device buffer of `items` pairs of unsigned 32-bit words
  * (the caller's; the library allocates nothing for it), every later persistent
  * advance of the handle records, for work item i in the kernel's order (tiles
@@ -337,8 +342,8 @@ int swept2d_batch_query_grid(const swept2d_batch_t *b, int grid, int what, doubl
  * Memory. It calls no cudaMalloc, cudaFree or other allocating routine. Its only
  * scratch is a static device array of SWEPT2D_STATIC_SCRATCH_BYTES in this
  * library, which every GPU that loads the library holds until the process
- * exits. It needs 2 * 4 * (n*n/2 + n) * 8 bytes per tile (the two panel
- * buffers; n*n/2 + n rounded up to a multiple of 8) plus nx*ny*8 bytes when
+ * exits. It asks for 2 * 4 * (n*n/2 + n) * 8 bytes per tile (two panel
+ * sets; n*n/2 + n rounded up to a multiple of 8) plus nx*ny*8 bytes when
  * nsteps is not a multiple of n/2, each part
  * rounded up to 256 bytes; larger grids are rejected with SWEPT2D_EINVAL and a
  * message. Nothing in the scratch needs to start at zero.
