@@ -460,7 +460,8 @@ def roofline(w, kern, peaks, esize, nvars):
     n, N = w.tile, w.grid
     launches, ms = kern.get("march", (0, 0.0))
     if launches:                       # the marching form: every step in one launch
-        upd = N * N * w.nsteps // launches
+        stages = 2 if w.op.startswith("euler") else 1
+        upd = N * N * w.nsteps * stages // launches
         hbm_bytes = 2 * N * N * nvars * esize // launches
         out = {"kernel": "march", "avg_launch_ms": ms / launches, "updates_per_launch": upd,
                "hbm_bytes_per_launch": hbm_bytes, "traffic": None, "traffic_source": None}

@@ -4,8 +4,9 @@
 // Grids that share a tile side n form a class. For each class the schedule of
 // one swept advance is the single-grid one (Up, then per half cycle the bridge
 // launch and the octahedron, a final Down, a naive tail), each launch covering
-// every tile of every grid of the class. Grids created with tile 0 only ever
-// take naive steps. A naive tail with an odd number of sub-steps ends in the
+// every tile of every grid of the class. Grids created with tile 0 take naive
+// steps there. Updates with a marching form (march.cuh) advance every grid in
+// that instead, in one launch, where it is faster for the batch. A naive tail with an odd number of sub-steps ends in the
 // second state copy, from which the class's grids are copied back, so the
 // pooled state stays in the first copy between calls.
 #include <cuda_runtime.h>
@@ -178,6 +179,20 @@ int batch_run(swept2d_batch *b, long long total, int mode) {
     const bool one_launch = (mode & SWEPT2D_ONE_LAUNCH) != 0;
     mode &= ~(SWEPT2D_PERSISTENT | SWEPT2D_ONE_LAUNCH);
     const u64 g_start = (u64)b->substeps;
+    if (mode == SWEPT2D_NAIVE && b->mt &&
+        swept::naive_walks(b->op == SWEPT2D_OP_EULER_RK2, b->op == SWEPT2D_OP_EULER_KAHAN,
+                           (double)b->cells)) {      // in place
+        for (long long s = 0; s < total; ++s) {
+            int rc = blaunch(b, "batched naive kernel", [&] {
+                return b->mt->phase_many(b->mshape, b->d_grids, b->d_mtiles, (int)b->mtiles.size(),
+                                         b->grids[0].c, b->state, (int)((g_start + s) & 1),
+                                         b->stream);
+            });
+            if (rc) return rc;
+        }
+        b->substeps += total;
+        return SWEPT2D_OK;
+    }
     if (mode == SWEPT2D_NAIVE) {
         void *cur = b->state, *other = b->state2;
         int rc = batch_naive(b, b->d_all_blocks, (int)b->all_blocks.size(), total, g_start, &cur,

@@ -8,6 +8,8 @@
 //   between half cycles j, j+1:  Octahedron = Down(j) + Up(j+1)  -> up panels
 //   after the last half cycle:   Down -> state (frame (H mod 2) h, periodic wrap)
 //   then r naive sub-steps.
+// Updates with a marching form (march.cuh) take that for the whole advance
+// instead, where it is faster for the grid.
 // The frame offset alternates 0, h, 0, ... (the paper's shift by half a tile
 // after each half cycle, Section 4); on one GPU a frame is only an index offset.
 #include <cuda_runtime.h>
@@ -55,6 +57,10 @@ struct swept2d {
     int mshape = 0;
     swept::MarchGrid mgrid{};
     int *msched = nullptr;
+    // the naive path's launches by its walks (Euler): the grid's shape and cut
+    const swept::MarchTable *nt = nullptr;
+    int nshape = 0;
+    swept::MarchGrid ngrid{};
     cudaStream_t stream = nullptr;
     void *state = nullptr, *state2 = nullptr, *up = nullptr, *br = nullptr;
     unsigned long long *scratch8 = nullptr;
@@ -216,6 +222,15 @@ void free_all(swept2d *h) {
 int naive_substeps(swept2d *h, long long count) {
     for (long long s = 0; s < count; ++s) {
         const u64 g = (u64)h->substeps;
+        if (h->nt) {                     // in place
+            int rc = launch(h, SWEPT2D_K_NAIVE, "naive kernel", [&] {
+                return h->nt->phase_one(h->nshape, h->ngrid, h->consts, h->state, (int)(g & 1),
+                                        h->stream);
+            });
+            if (rc) return rc;
+            h->substeps += 1;
+            continue;
+        }
         int rc = launch(h, SWEPT2D_K_NAIVE, "naive kernel", [&] {
             return h->ops->naive(h->G, h->consts, h->state, h->state2, g, h->stream);
         });
@@ -454,6 +469,12 @@ int swept2d_create(swept2d_t **out, int nx, int ny, int nvars, int nstages, int 
             cuda_fail(h, e, "panel allocation");
             return bail(e == cudaErrorMemoryAllocation ? SWEPT2D_ENOMEM : SWEPT2D_ECUDA);
         }
+    }
+    if (swept::naive_walks(op == SWEPT2D_OP_EULER_RK2, op == SWEPT2D_OP_EULER_KAHAN,
+                           (double)nx * ny)) {
+        h->nt = march_for(op, dtype);
+        h->nshape = h->nt->shape(&nx, &ny, 1, true);
+        h->ngrid = h->nt->cut(h->nshape, nx, ny);
     }
     h->mt = tile ? march_for(op, dtype) : nullptr;
     if (h->mt) {

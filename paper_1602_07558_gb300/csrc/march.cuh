@@ -20,6 +20,7 @@
 
 #include "exact64.cuh"
 #include "kernels.cuh"
+#include "launch.cuh"
 #include "march_table.cuh"
 
 namespace swept {
@@ -125,6 +126,18 @@ march_kernel(Op op, Loc at, MarchRun<typename Op::S> run) {
         __syncthreads();
         if (threadIdx.x == 0) add_release(run.done + t, 1);
     }
+}
+
+// One phase of an update computed in place, one tile a block: the naive path's
+// launch per sub-step.
+template <class Body, class Op, class Loc>
+__global__ void __launch_bounds__(Body::kThreads, Body::kMinBlocks)
+march_phase_kernel(Op op, Loc at, typename Op::S *state, int phase) {
+    __shared__ typename Body::Smem sm;
+    const MarchTile m = at(blockIdx.x);
+    const Op own = m.c ? Op(m.c) : op;
+    after_previous_launch();
+    Body::run(own, m, state + m.soff, state + m.soff, Body::K, Body::K, phase, sm);
 }
 
 // ------------------------------------------------------------------- heat
@@ -834,8 +847,30 @@ inline cudaError_t march_advance(int shape, const Op &op, const Loc &at, int NT,
     });
 }
 
+// One phase over NT tiles of an update computed in place.
+template <class Op, class Loc>
+inline cudaError_t march_phase(int shape, const Op &op, const Loc &at, int NT, void *state,
+                               int phase, cudaStream_t st) {
+    return with_march_shape<Op>(shape, [&](auto *body) {
+        typedef typename std::remove_pointer<decltype(body)>::type B;
+        if constexpr (B::kInPlace)
+            return launch_after(march_phase_kernel<B, Op, Loc>, dim3(NT), B::kThreads, 0, st, op, at,
+                                (typename Op::S *)state, phase);
+        else
+            return cudaErrorInvalidValue;
+    });
+}
+
 template <class Op>
 struct March {
+    static cudaError_t phase_one(int shape, const MarchGrid &g, const double *c, void *state,
+                                 int phase, cudaStream_t st) {
+        return march_phase(shape, Op(c), OneMarch{g}, g.bx * g.by, state, phase, st);
+    }
+    static cudaError_t phase_many(int shape, const GridDesc *grids, const int2 *tiles, int NT,
+                                  const double *c, void *state, int phase, cudaStream_t st) {
+        return march_phase(shape, Op(c), ManyMarch{grids, tiles}, NT, state, phase, st);
+    }
     static cudaError_t one(int shape, const MarchGrid &g, const double *c, const void *src,
                            void *b0, void *b1, int *sched, long long steps, int *err, int first,
                            long long spin_limit, void **out, long long *launches,
@@ -852,7 +887,7 @@ struct March {
     }
     static const MarchTable *table() {
         static const MarchTable t = {&march_shape<Op>, &march_steps<Op>, &march_cut<Op>, &one,
-                                     &many};
+                                     &many, &phase_one, &phase_many};
         return &t;
     }
 };

@@ -174,3 +174,30 @@ def test_naive_heat_rows_and_launches_match_the_oracle(oracle_lib, kind, nx, ny)
             s.set_state(u0[None])
             s.advance(13, mode="naive", graph=graph)
             assert np.array_equal(s.get_state()[0], ref)
+
+
+@pytest.mark.parametrize("op,dtype", [("euler_rk2", "f64"), ("euler_kahan", "f32"),
+                                      ("euler_kahan", "bf16")])
+@pytest.mark.parametrize("nx,ny", [(13, 7), (61, 62), (457, 449)])
+def test_naive_euler_launches_match_the_oracle(oracle_lib, op, dtype, nx, ny):
+    """The naive path's walks (binary64, and the larger binary32 / bfloat16
+    grids), on odd sides that no tile divides, split over two advances."""
+    U = inputs.euler_pulse(nx, ny, 4, gamma=1.4)
+    if op == "euler_kahan":
+        U = U.astype(np.float32)
+        if dtype == "bf16":
+            U = torch.from_numpy(U).to(torch.bfloat16).view(torch.int16).numpy().view(np.uint16)
+    Uf = (oracle_lib.bf16_bits_to_f32(U) if dtype == "bf16" else U).astype(np.float64)
+    a, dt = oracle_lib.euler_setup(Uf, 1.4, 0.3)
+    if op == "euler_rk2":
+        u0, ref = np.concatenate([U, U]), oracle_lib.euler_rk2(U, 1.4, dt, 0.5, a, 5)
+    else:
+        u0 = np.concatenate([U, U, np.zeros_like(U)])
+        ref = oracle_lib.euler_kahan(u0, 1.4, dt, 0.5, a, 5, dtype)
+    with Swept2D(nx, ny, op=op, tile=0, params=(1.4, 0.3, 0.5), dtype=dtype,
+                 stream=torch.cuda.Stream()) as s:
+        s.set_state(u0)
+        s.advance(2, mode="naive")
+        s.advance(3, mode="naive", graph=True)
+        got = s.get_state()
+    assert np.array_equal(got[:len(ref)], ref)
