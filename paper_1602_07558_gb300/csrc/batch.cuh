@@ -184,6 +184,7 @@ __global__ void __launch_bounds__(256) batch_naive_kernel(const GridDesc *grids,
     const int x = bx * 32 + (threadIdx.x & 31);
     const int y = by * 8 + (threadIdx.x >> 5);
     if (x >= gd.G.nx || y >= gd.G.ny) return;
+    after_previous_launch();
     const size_t plane = (size_t)gd.G.nx * gd.G.ny;
     GlobalAcc<S> acc(in + gd.state_off, plane, gd.G.nx, gd.G.ny, x, y);
     S res[Op::NV];
@@ -231,8 +232,8 @@ struct BatchLaunch {
     typedef typename Op::S S;
     static cudaError_t naive(const GridDesc *d, const int2 *bg, int nblocks, const void *in,
                              void *out, u64 g, cudaStream_t st) {
-        batch_naive_kernel<Op><<<nblocks, kBlock, 0, st>>>(d, bg, (const S *)in, (S *)out, g);
-        return cudaGetLastError();
+        return launch_after(batch_naive_kernel<Op>, dim3(nblocks), kBlock, 0, st, d, bg,
+                            (const S *)in, (S *)out, g);
     }
     static cudaError_t up(const GridDesc *d, const int2 *tg, int ntiles, int n, const void *state,
                           void *upp, int o, u64 g0, cudaStream_t st) {
