@@ -271,7 +271,8 @@ struct HeatCell<HeatKahanOp<SS>> {
 // shared memory (two buffers in turn, one barrier a step), then each thread
 // walks down its rows. The outermost columns and rows of the region go wrong by
 // one more each step, which the ring covers; warps whose rows no later step
-// needs rest.
+// needs rest. Against the swept kernels: 2048², 2,000 steps, binary32 20.1 -> 7.8 ms,
+// bfloat16 15.7 -> 8.8 (the heavy half of the FMA pipe 70% busy).
 template <class Op, int R_, int WY_, int MINB_, int K_>
 struct HeatMarch {
     typedef typename Op::S S;
@@ -462,7 +463,10 @@ struct EulerRow {
 // with the rows above, at and below the current one in registers: every point's
 // primitives and fluxes are formed once and serve its four neighbours, the east
 // and west ones by shuffle. The outermost columns only supply neighbours. The
-// walks of a block take HR rows each and share nothing.
+// walks of a block take HR rows each and share nothing. Binary64 is bound by the
+// FP64 pipe (0.93 of its rate), binary32 by DRAM (28 planes a step, 4.7 TB/s) and,
+// with bfloat16, by the loads' latency. 2048² against the swept kernels: binary64 50
+// steps 66.4 -> 56.7 ms, binary32 200 steps 31.3 -> 19.5, bfloat16 30.4 -> 14.1.
 template <class Op, int SEG_, int HR_, int WY_, int MINB_>
 struct EulerMarch {
     typedef typename Op::S S;
