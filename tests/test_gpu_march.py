@@ -112,6 +112,28 @@ def test_wave_fused_difference_has_the_bits_of_two_operations(oracle_lib, scale)
     assert np.array_equal(got[1], ref_old, equal_nan=True)
 
 
+@pytest.mark.parametrize("mode", ["swept", "naive"])
+def test_wave_difference_where_the_double_overflows(mode):
+    """u of both signs in the last binade, whose double is an infinity, over old
+    values that are NaN, infinities of either sign, and finite: one step against
+    the update's operations one by one. (4u overflows there, too: the fused d is
+    the neighbours' sum where that is an infinity, and -4u's infinity elsewhere.)"""
+    u, old = np.full((16, 32), 1e308), np.zeros((16, 32))
+    u[:, 16:] = -1.5e308
+    old[:] = np.tile([np.nan, np.inf, -np.inf, 1e308, -1e308, 0.0, -0.0, 3.0], (16, 4))
+    with np.errstate(all="ignore"):
+        s = (np.roll(u, -1, 1) + np.roll(u, -1, 0)) + (np.roll(u, 1, 1) + np.roll(u, 1, 0))
+        d = np.where(np.isinf(s), s, s - 4.0 * u)
+        want = 0.3 * 0.3 * d + (2.0 * u - old)
+    assert np.isnan(want).any() and np.isinf(want).any()
+    with Swept2D(32, 16, op="wave", tile=4, params=(0.3,)) as sw:
+        sw.set_state(np.stack([u, old]))
+        sw.advance(1, mode=mode)
+        got = sw.get_state()
+    assert np.array_equal(got[0], want, equal_nan=True)
+    assert np.array_equal(got[1], u)
+
+
 @pytest.mark.parametrize("nx,ny,tile,nsteps", [
     (4, 4, 4, 3), (16, 60, 4, 4), (30, 30, 6, 5), (64, 48, 16, 6), (150, 150, 10, 3),
     (330, 300, 10, 3), (1040, 1056, 16, 2),
