@@ -361,10 +361,20 @@ int swept2d_batch_query_grid(const swept2d_batch_t *b, int grid, int what, doubl
  *
  * Errors: SWEPT2D_EINVAL (bad sizes or pointers, grid too large for the
  * scratch), SWEPT2D_ECUDA; a message goes to err (errlen bytes, may be NULL).
+ * The call has returned by the time a kernel's bounded neighbourhood wait could
+ * give up (a handle's SWEPT2D_ETIMEOUT): u_out is then NaN at every point.
  */
 #define SWEPT2D_STATIC_SCRATCH_BYTES ((size_t)32 << 20)
 int swept2d_heat_advance_static(const double *u_in, double *u_out, int nx, int ny, int tile,
                                 double r, long long nsteps, void *stream, char *err, int errlen);
+
+/* Self-test of that: queues an advance of a few steps whose first phase is
+ * skipped, so that every block's wait gives up after spin_limit polls (>= 1, see
+ * swept2d_selftest_wait_timeout) and u_out becomes NaN. Returns and errors as
+ * swept2d_heat_advance_static (SWEPT2D_OK once it is queued). */
+int swept2d_selftest_static_timeout(const double *u_in, double *u_out, int nx, int ny, int tile,
+                                    double r, long long spin_limit, void *stream, char *err,
+                                    int errlen);
 
 #ifdef __cplusplus
 }

@@ -801,8 +801,9 @@ inline int march_shape(const int *nx, const int *ny, int count, bool always) {
 }
 
 // Queues `steps` steps over NT tiles: reads `src`, writes b0, b1, b0, ... phase
-// by phase (src may be b1). sched: NT counters and the item counter. `launches`
-// is raised by the launches made, `*out` set to the buffer with the result.
+// by phase (src may be b1). sched: NT counters and the item counter; without `err`
+// the word after them is the error word and is cleared with them. `launches` is
+// raised by the launches made, `*out` set to the buffer with the result.
 template <class Op, class Loc>
 inline cudaError_t march_advance(int shape, const Op &op, const Loc &at, int NT, const void *src,
                                  void *b0, void *b1, int *sched, long long steps, int *err,
@@ -822,6 +823,8 @@ inline cudaError_t march_advance(int shape, const Op &op, const Loc &at, int NT,
         // items of one launch count in an int
         // (an even number of phases: the stages of Euler alternate)
         const long long most = (((1LL << 30) - 1) / NT + 2) & ~1LL;
+        size_t words = (size_t)NT + (err ? 1 : 2);
+        if (!err) err = sched + NT + 1;
         while (steps > 0) {
             const long long left = (steps + K - 1) / K;
             MarchRun<S> run;
@@ -837,8 +840,8 @@ inline cudaError_t march_advance(int shape, const Op &op, const Loc &at, int NT,
             run.last = run.phases < left ? K : (int)(steps - (left - 1) * K);
             run.first = first;
             run.spin_limit = spin_limit;
-            if ((e = cudaMemsetAsync(sched, 0, ((size_t)NT + 1) * sizeof(int), st)) != cudaSuccess)
-                return e;
+            if ((e = cudaMemsetAsync(sched, 0, words * sizeof(int), st)) != cudaSuccess) return e;
+            words = (size_t)NT + 1;
             long long grid = (long long)(per_sm > 0 ? per_sm : 1) * nsm;
             if (grid > 2LL * NT) grid = 2LL * NT;
             if (grid > (long long)NT * run.phases) grid = (long long)NT * run.phases;

@@ -11,7 +11,9 @@
 //
 // The marching form of swept2d_advance (march.cuh) on the caller's buffers, so
 // the result is bit for bit that of a handle created with op SWEPT2D_OP_HEAT and
-// advanced with SWEPT2D_SWEPT from the same input.
+// advanced with SWEPT2D_SWEPT from the same input. The call has returned before a
+// wait of that form could give up, and its caller has no handle to ask: a last
+// kernel then overwrites u_out with NaN.
 #include <cuda_runtime.h>
 
 #include <cstdio>
@@ -57,11 +59,19 @@ int scratch_address(void **out, char *err, int errlen) {
     return SWEPT2D_OK;
 }
 
-}  // namespace
+// u = NaN everywhere if the launch before this one recorded a failure.
+__global__ void __launch_bounds__(256) spoil_if_failed(const int *err, double *u, size_t n) {
+    swept::after_previous_launch();
+    if (*err == 0) return;
+    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n;
+         i += (size_t)gridDim.x * blockDim.x)
+        u[i] = __longlong_as_double(0x7ff8000000000000LL);
+}
 
-extern "C" int swept2d_heat_advance_static(const double *u_in, double *u_out, int nx, int ny,
-                                           int tile, double r, long long nsteps, void *stream,
-                                           char *err, int errlen) {
+// The advance; `skip` (the wait-timeout self-test): its first phase is skipped.
+int advance_static(const double *u_in, double *u_out, int nx, int ny, int tile, double r,
+                   long long nsteps, bool skip, long long spin_limit, void *stream, char *err,
+                   int errlen) {
     set_err(err, errlen, "");
     if (!u_in || !u_out) {
         set_err(err, errlen, "u_in and u_out must be device pointers");
@@ -121,19 +131,21 @@ extern "C" int swept2d_heat_advance_static(const double *u_in, double *u_out, in
     const swept::MarchTable *mt = swept::marchtable_heat();
     const int shape = mt->shape(&nx, &ny, 1, true);
     const swept::MarchGrid cut = mt->cut(shape, nx, ny);
+    const int tiles = cut.bx * cut.by;
     void *tmp = base;
     int *sched = (int *)((char *)base + align256(state_bytes));
-    int *errword = sched + cut.bx * cut.by + 1;
-    cudaError_t e = cudaMemsetAsync(errword, 0, sizeof(int), st);
     // the buffers alternate phase by phase; the last phase writes u_out
+    if (skip) nsteps = 2LL * mt->steps(shape);
     const long long phases = (nsteps + mt->steps(shape) - 1) / mt->steps(shape);
     void *b0 = (phases & 1) ? (void *)u_out : tmp, *b1 = (phases & 1) ? tmp : (void *)u_out;
     const double consts[8] = {r, 0, 0, 0, 0, 0, 0, 0};
     void *out = nullptr;
     long long made = 0;
+    cudaError_t e = mt->one(shape, cut, consts, u_in, b0, b1, sched, nsteps, nullptr,
+                            skip ? tiles : 0, spin_limit, &out, &made, st);
     if (e == cudaSuccess)
-        e = mt->one(shape, cut, consts, u_in, b0, b1, sched, nsteps, errword, 0,
-                    swept::kPersistSpinLimit, &out, &made, st);
+        e = swept::launch_after(spoil_if_failed, dim3(152), 256, 0, st, sched + tiles + 1, u_out,
+                                (size_t)nx * ny);
     if (e != cudaSuccess) {
         char msg[200];
         snprintf(msg, sizeof msg, "marching kernel: %s", cudaGetErrorString(e));
@@ -142,3 +154,25 @@ extern "C" int swept2d_heat_advance_static(const double *u_in, double *u_out, in
     }
     return SWEPT2D_OK;
 }
+
+}  // namespace
+
+extern "C" {
+
+int swept2d_heat_advance_static(const double *u_in, double *u_out, int nx, int ny, int tile,
+                                double r, long long nsteps, void *stream, char *err, int errlen) {
+    return advance_static(u_in, u_out, nx, ny, tile, r, nsteps, false, swept::kPersistSpinLimit,
+                          stream, err, errlen);
+}
+
+int swept2d_selftest_static_timeout(const double *u_in, double *u_out, int nx, int ny, int tile,
+                                    double r, long long spin_limit, void *stream, char *err,
+                                    int errlen) {
+    if (spin_limit < 1) {
+        set_err(err, errlen, "selftest: spin_limit < 1");
+        return SWEPT2D_EINVAL;
+    }
+    return advance_static(u_in, u_out, nx, ny, tile, r, 1, true, spin_limit, stream, err, errlen);
+}
+
+}  // extern "C"

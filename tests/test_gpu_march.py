@@ -134,6 +134,32 @@ def test_wave_difference_where_the_double_overflows(mode):
     assert np.array_equal(got[1], u)
 
 
+@pytest.mark.parametrize("nx,ny,tile", [(64, 64, 16), (4, 4, 4), (768, 768, 16)])
+def test_static_advance_makes_a_timed_out_wait_visible(oracle_lib, nx, ny, tile):
+    """The call without a handle: u_out is NaN everywhere after a wait that gave
+    up, and the next call is not touched by it."""
+    import ctypes
+    from paper_1602_07558_gb300.swept2d import EINVAL, OK, heat_advance_static, lib
+    u0 = inputs.uniform(nx, ny, seed=4)
+    d_in = torch.from_numpy(u0).to("cuda")
+    d_out = torch.zeros_like(d_in)
+    stream = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    f = lib().swept2d_selftest_static_timeout
+    f.argtypes = [ctypes.c_void_p] * 2 + [ctypes.c_int] * 3 + [ctypes.c_double, ctypes.c_longlong] \
+        + [ctypes.c_void_p, ctypes.c_char_p, ctypes.c_int]
+    call = lambda limit: f(d_in.data_ptr(), d_out.data_ptr(), nx, ny, tile, 0.2, limit,
+                           stream.cuda_stream, None, 0)
+    assert call(0) == EINVAL
+    assert call(1000) == OK
+    stream.synchronize()
+    assert torch.isnan(d_out).all()
+    assert np.array_equal(d_in.cpu().numpy(), u0)
+    heat_advance_static(d_in, d_out, nx, ny, tile, 0.2, 13, stream=stream)
+    stream.synchronize()
+    assert np.array_equal(d_out.cpu().numpy(), oracle_lib.heat(u0, 0.2, 13))
+
+
 @pytest.mark.parametrize("nx,ny,tile,nsteps", [
     (4, 4, 4, 3), (16, 60, 4, 4), (30, 30, 6, 5), (64, 48, 16, 6), (150, 150, 10, 3),
     (330, 300, 10, 3), (1040, 1056, 16, 2),
