@@ -772,8 +772,9 @@ __global__ void __launch_bounds__(256) naive_heat_kernel(HeatOp op, Geom G, cons
     int x = blockIdx.x * 30 + lane - 1;
     const bool active = lane > 0 && lane < 31 && x < G.nx;
     x = x < 0 ? G.nx - 1 : x % G.nx;      // idle lanes read valid memory, store nothing
-    const int y0 = (blockIdx.y * 8 + warp) * ROWS;
-    if (y0 >= G.ny) return;               // whole warp leaves together
+    const unsigned first = ((blockIdx.z * gridDim.y + blockIdx.y) * 8 + warp) * ROWS;
+    if (first >= (unsigned)G.ny) return;  // whole warp leaves together
+    const int y0 = (int)first;
     after_previous_launch();
     const int n = min(ROWS, G.ny - y0);
     const size_t nx = G.nx;

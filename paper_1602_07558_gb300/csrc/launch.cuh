@@ -111,8 +111,9 @@ struct Launch {
             const long long chunks = (G.nx + 29) / 30;
             int rows = 8;
             while (rows > 1 && chunks * ((G.ny + rows - 1) / rows) < 152LL * 32) rows >>= 1;
-            const int warps = (G.ny + rows - 1) / rows;
-            dim3 grid((unsigned)chunks, (warps + 7) / 8);
+            const unsigned bands = ((unsigned)((G.ny + rows - 1) / rows) + 7) / 8;
+            // (65535 blocks along y hold 4.2 M rows; taller grids go on along z)
+            dim3 grid((unsigned)chunks, bands < 65535 ? bands : 65535, (bands + 65534) / 65535);
             const Op op(c);
             switch (rows) {
                 case 8: e = launch_after(naive_heat_kernel<8>, grid, kBlock, 0, st, op, G, (const S *)in, (S *)out); break;

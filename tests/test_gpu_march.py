@@ -224,6 +224,15 @@ def test_naive_heat_rows_and_launches_match_the_oracle(oracle_lib, kind, nx, ny)
             assert np.array_equal(s.get_state()[0], ref)
 
 
+@pytest.mark.parametrize("nx,ny", [(1, 65535 * 64 + 3), (2, 65535 * 64)])
+def test_naive_heat_takes_more_rows_than_a_launch_has_blocks_along_y(oracle_lib, nx, ny):
+    u0 = np.random.default_rng(ny).random((ny, nx))
+    with Swept2D(nx, ny, op="heat", tile=0, params=(0.2,)) as s:
+        s.set_state(u0[None])
+        s.advance(3, mode="naive")
+        assert np.array_equal(s.get_state()[0], oracle_lib.heat(u0, 0.2, 3))
+
+
 @pytest.mark.parametrize("op,dtype", [("euler_rk2", "f64"), ("euler_kahan", "f32"),
                                       ("euler_kahan", "bf16")])
 @pytest.mark.parametrize("nx,ny", [(13, 7), (61, 62), (457, 449)])
