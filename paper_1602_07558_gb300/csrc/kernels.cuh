@@ -765,16 +765,16 @@ __device__ __forceinline__ void naive_heat_rows(const double (&u)[ROWS + 2], dou
 // those). The integer units bound it. Measured on the GB300, us a step in a
 // graph, before (31 columns, FP64 operations): 1009 x 757 8.9 -> 6.3, 2048²
 // 39.7 -> 23.1, 4096² 136.6 -> 85.1 (8 rows; 4 rows 85.8, 16 rows 96.2).
-template <int ROWS>
+// TALL: of a grid with more rows than a launch has blocks along y, those from `top`.
+template <int ROWS, bool TALL = false>
 __global__ void __launch_bounds__(256) naive_heat_kernel(HeatOp op, Geom G, const double *in,
-                                                         double *out) {
+                                                         double *out, int top) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int x = blockIdx.x * 30 + lane - 1;
     const bool active = lane > 0 && lane < 31 && x < G.nx;
     x = x < 0 ? G.nx - 1 : x % G.nx;      // idle lanes read valid memory, store nothing
-    const unsigned first = ((blockIdx.z * gridDim.y + blockIdx.y) * 8 + warp) * ROWS;
-    if (first >= (unsigned)G.ny) return;  // whole warp leaves together
-    const int y0 = (int)first;
+    const int y0 = (TALL ? top : 0) + (blockIdx.y * 8 + warp) * ROWS;
+    if (y0 >= G.ny) return;               // whole warp leaves together
     after_previous_launch();
     const int n = min(ROWS, G.ny - y0);
     const size_t nx = G.nx;

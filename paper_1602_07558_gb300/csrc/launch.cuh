@@ -111,15 +111,22 @@ struct Launch {
             const long long chunks = (G.nx + 29) / 30;
             int rows = 8;
             while (rows > 1 && chunks * ((G.ny + rows - 1) / rows) < 152LL * 32) rows >>= 1;
-            const unsigned bands = ((unsigned)((G.ny + rows - 1) / rows) + 7) / 8;
-            // (65535 blocks along y hold 4.2 M rows; taller grids go on along z)
-            dim3 grid((unsigned)chunks, bands < 65535 ? bands : 65535, (bands + 65534) / 65535);
             const Op op(c);
+            const long long bands = ((G.ny + rows - 1LL) / rows + 7) / 8, most = 65535;
+            if (bands > most) {            // (so many rows always come eight a warp)
+                e = cudaSuccess;
+                for (long long b = 0; b < bands && e == cudaSuccess; b += most)
+                    e = launch_after(naive_heat_kernel<8, true>,
+                                     dim3((unsigned)chunks, (unsigned)(bands - b < most ? bands - b : most)),
+                                     kBlock, 0, st, op, G, (const S *)in, (S *)out, (int)(b * 64));
+                return e;
+            }
+            dim3 grid((unsigned)chunks, (unsigned)bands);
             switch (rows) {
-                case 8: e = launch_after(naive_heat_kernel<8>, grid, kBlock, 0, st, op, G, (const S *)in, (S *)out); break;
-                case 4: e = launch_after(naive_heat_kernel<4>, grid, kBlock, 0, st, op, G, (const S *)in, (S *)out); break;
-                case 2: e = launch_after(naive_heat_kernel<2>, grid, kBlock, 0, st, op, G, (const S *)in, (S *)out); break;
-                default: e = launch_after(naive_heat_kernel<1>, grid, kBlock, 0, st, op, G, (const S *)in, (S *)out); break;
+                case 8: e = launch_after(naive_heat_kernel<8>, grid, kBlock, 0, st, op, G, (const S *)in, (S *)out, 0); break;
+                case 4: e = launch_after(naive_heat_kernel<4>, grid, kBlock, 0, st, op, G, (const S *)in, (S *)out, 0); break;
+                case 2: e = launch_after(naive_heat_kernel<2>, grid, kBlock, 0, st, op, G, (const S *)in, (S *)out, 0); break;
+                default: e = launch_after(naive_heat_kernel<1>, grid, kBlock, 0, st, op, G, (const S *)in, (S *)out, 0); break;
             }
         } else if constexpr (std::is_same<Op, HeatKahanOp<float>>::value ||
                              std::is_same<Op, HeatKahanOp<__nv_bfloat16>>::value) {
