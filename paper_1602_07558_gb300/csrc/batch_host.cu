@@ -61,6 +61,7 @@ struct swept2d_batch {
     // tile) and counters (one per tile, the item counter)
     const swept::MarchTable *mt = nullptr;
     int mshape = 0;
+    bool naive_walks = false;   // the naive sub-steps take its walks, too
     std::vector<int2> mtiles;
     int2 *d_mtiles = nullptr;
     int *msched = nullptr;
@@ -179,9 +180,7 @@ int batch_run(swept2d_batch *b, long long total, int mode) {
     const bool one_launch = (mode & SWEPT2D_ONE_LAUNCH) != 0;
     mode &= ~(SWEPT2D_PERSISTENT | SWEPT2D_ONE_LAUNCH);
     const u64 g_start = (u64)b->substeps;
-    if (mode == SWEPT2D_NAIVE && b->mt &&
-        swept::naive_walks(b->op == SWEPT2D_OP_EULER_RK2, b->op == SWEPT2D_OP_EULER_KAHAN,
-                           (double)b->cells)) {      // in place
+    if (mode == SWEPT2D_NAIVE && b->naive_walks) {   // in place
         for (long long s = 0; s < total; ++s) {
             int rc = blaunch(b, "batched naive kernel", [&] {
                 return b->mt->phase_many(b->mshape, b->d_grids, b->d_mtiles, (int)b->mtiles.size(),
@@ -457,6 +456,9 @@ int swept2d_batch_create(swept2d_batch_t **out, int count, const int *nx, const 
             b->all_blocks.push_back(make_int2(i, k));
         }
     }
+    b->naive_walks = b->mt && swept::batch_naive_walks(op == SWEPT2D_OP_EULER_RK2,
+                                                       op == SWEPT2D_OP_EULER_KAHAN,
+                                                       (double)b->cells);
     b->state_bytes = (size_t)soff * bt->esize;
     b->panel_bytes = (size_t)poff * bt->esize;
     cudaError_t e = cudaSuccess;

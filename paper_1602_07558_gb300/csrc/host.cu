@@ -470,11 +470,11 @@ int swept2d_create(swept2d_t **out, int nx, int ny, int nvars, int nstages, int 
             return bail(e == cudaErrorMemoryAllocation ? SWEPT2D_ENOMEM : SWEPT2D_ECUDA);
         }
     }
-    if (swept::naive_walks(op == SWEPT2D_OP_EULER_RK2, op == SWEPT2D_OP_EULER_KAHAN,
-                           (double)nx * ny)) {
-        h->nt = march_for(op, dtype);
-        h->nshape = h->nt->shape(&nx, &ny, 1, true);
-        h->ngrid = h->nt->cut(h->nshape, nx, ny);
+    h->nt = march_for(op, dtype);
+    if (h->nt) {
+        h->nshape = h->nt->naive_shape(nx, ny);
+        if (h->nshape < 0) h->nt = nullptr;
+        else h->ngrid = h->nt->cut(h->nshape, nx, ny);
     }
     h->mt = tile ? march_for(op, dtype) : nullptr;
     if (h->mt) {

@@ -800,6 +800,83 @@ inline int march_shape(const int *nx, const int *ny, int count, bool always) {
     return shape;
 }
 
+// ---------------------------------------------- the naive path's walks (Euler)
+// What a step (two launches) of the naive path takes, in µs: `more` for each wave of
+// blocks that run at once beside `base`. In binary64 a block has an SM for itself,
+// as the FP64 pipe is the bound, and the waves are whole; otherwise the resident
+// blocks of an SM end at different times, and the second wave alone costs an extra.
+struct WaveCost {
+    double base, more;
+    int wave;
+    double least;               // however few the blocks
+    bool whole;
+    double operator()(long long blocks) const {
+        double w = (double)((blocks + wave - 1) / wave);
+        if (!whole && w > 1) {
+            w = (double)blocks / wave + 0.1;
+            if (w < 1.65) w = 1.65;
+        }
+        const double t = base + more * w;
+        return t > least ? t : least;
+    }
+};
+// By shape; last: a thread a point, in blocks of 32 x 8 points, which forms
+// its four neighbours' fluxes, too, but has the shorter chain. Measured on the
+// GB300, us a step in a graph, walks by shape 0, 1, ... / a thread a point:
+//   binary64: 64 x 64 166, 88, 28.0, 17.2 / 18.6; 64 x 512 167, 88, 28.2, 25.3 / 18.8;
+//     256 x 256 167, 88, 28.5, 40.2 / 34.6; 384 x 384 167, 88, 75, 74.7 / 67;
+//     1024 x 65 -, -, 51, 40 / 35; 512 x 512 167, 88, 99, 131 / 116;
+//     1024 x 1024 320, 332, 383, 483 / 441; 2048 x 2048 1260, 1218, 1420, 1885 / 1748
+//   binary32: 400 x 300 36, 13, 8.9, 7.3, 8.7 / 6.1; 128 x 2048 37, 13.6, 10.0, 12.4, 14.5
+//     / 9.8; 272 x 1056 35, 13.8, 10.0, 11.9, 13.9 / 10.8; 512 x 512 38, 13.2, 9.8, 8.1,
+//     11.2 / 9.6; 1024 x 1024 39, 19.6, 22.5, 26.6, 38.6 / 39.1; 2048 x 2048 98, 102, 112,
+//     120, 167 / 164; bfloat16: 272 x 1056 44, 15.9, 11.1, 13.0, 14.5 / 11.0; 1024 x 1024
+//     47, 20.2, 23.2, 28.1, 39.2 / 31.3; 2048 x 2048 67, 77, 88, 106, 152 / 142
+template <class Op>
+inline const WaveCost *naive_costs() {
+    return nullptr;
+}
+template <>
+inline const WaveCost *naive_costs<EulerOp>() {
+    static const WaveCost c[] = {{6, 157, 152, 0, true},
+                                 {8, 79.5, 152, 0, true},
+                                 {4.5, 23.7, 152, 0, true},
+                                 {2.5, 7.5, 152, 17.2, true},
+                                 {2.4, 16.3, 152, 0, true}};
+    return c;
+}
+template <>
+inline const WaveCost *naive_costs<EulerKahanOp<float>>() {
+    static const WaveCost c[] = {{-15, 55, 608, 0, false},   {-4, 20, 608, 0, false},
+                                 {-2.1, 12.5, 608, 0, false}, {2, 6.2, 608, 0, false},
+                                 {1.8, 4.6, 608, 0, false},   {1, 5, 608, 0, false}};
+    return c;
+}
+template <>
+inline const WaveCost *naive_costs<EulerKahanOp<__nv_bfloat16>>() {
+    static const WaveCost c[] = {{-12, 57, 608, 0, false},   {-4, 20, 608, 0, false},
+                                 {-1.0, 12.5, 608, 0, false}, {2.4, 6.3, 608, 0, false},
+                                 {2.1, 4.7, 608, 0, false},   {1, 5, 608, 0, false}};
+    return c;
+}
+
+template <class Op>
+inline int naive_shape(int nx, int ny) {
+    const WaveCost *cost = naive_costs<Op>();
+    if (!cost) return -1;
+    int best = -1;
+    double least = cost[MarchShapes<Op>::kCount](((nx + 31LL) / 32) * ((ny + 7) / 8));
+    for (int s = 0; s < MarchShapes<Op>::kCount; ++s) {
+        const MarchGrid g = march_cut<Op>(s, nx, ny);
+        const double t = cost[s]((long long)g.bx * g.by);
+        if (t < least) {
+            least = t;
+            best = s;
+        }
+    }
+    return best;
+}
+
 // Queues `steps` steps over NT tiles: reads `src`, writes b0, b1, b0, ... phase
 // by phase (src may be b1). sched: NT counters and the item counter; without `err`
 // the word after them is the error word and is cleared with them. `launches` is
@@ -899,8 +976,9 @@ struct March {
                              err, 0, kPersistSpinLimit, out, launches, st);
     }
     static const MarchTable *table() {
-        static const MarchTable t = {&march_shape<Op>, &march_steps<Op>, &march_cut<Op>, &one,
-                                     &many, &phase_one, &phase_many};
+        static const MarchTable t = {&march_shape<Op>, &march_steps<Op>, &march_cut<Op>,
+                                     &naive_shape<Op>, &one, &many, &phase_one,
+                                     &phase_many};
         return &t;
     }
 };

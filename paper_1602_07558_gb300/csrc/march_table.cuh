@@ -10,6 +10,9 @@ struct MarchTable {
     int (*shape)(const int *nx, const int *ny, int count, bool always);
     int (*steps)(int shape);     // steps a phase
     MarchGrid (*cut)(int shape, int nx, int ny);
+    // the shape whose walks (phase_one) are the quickest for the naive sub-steps of
+    // one grid, -1 for a thread a point
+    int (*naive_shape)(int nx, int ny);
     // one grid (`g` its cut), or the tiles of a batch's table
     cudaError_t (*one)(int shape, const MarchGrid &g, const double *c, const void *src, void *b0,
                        void *b1, int *sched, long long steps, int *err, int first,
@@ -24,13 +27,12 @@ struct MarchTable {
                               const double *c, void *state, int phase, cudaStream_t);
 };
 
-// Whether Euler's naive sub-steps, one launch each, are walks of the marching form
-// (every point's fluxes formed once) rather than a thread a point, which forms its
-// four neighbours' fluxes but has the shorter chain. Measured on the GB300, us a
-// step in a graph, a thread a point / walks: binary64 64² 18.3 / 16.8, 200² 34.4 /
-// 25.0, 2048² 1747 / 1260; binary32 64² 3.7 / 4.5, 400 x 300 6.1 / 6.1, 1009 x 757
-// 24.5 / 18.6, 2048² 163 / 98.6; bfloat16 400 x 300 6.1 / 6.3, 2048² 141 / 66.
-inline bool naive_walks(bool euler, bool euler_kahan, double points) {
+// Whether a batch's naive sub-steps are walks (phase_many) rather than a thread a
+// point. Measured on the GB300, us a step in a graph, a thread a point / walks:
+// binary64 64 grids of 16..48 53 / 42, 256 of 32..96 470 / 469, 256 of 32..512 7498 /
+// 5478; binary32 64 of 16..48 8.2 / 8.6, 40 of 64..160 20.6 / 18.7, 256 of 32..96 48 /
+// 33, 256 of 32..512 808 / 420.
+inline bool batch_naive_walks(bool euler, bool euler_kahan, double points) {
     return euler || (euler_kahan && points >= 2e5);
 }
 

@@ -258,3 +258,37 @@ def test_naive_euler_launches_match_the_oracle(oracle_lib, op, dtype, nx, ny):
         s.advance(3, mode="naive", graph=True)
         got = s.get_state()
     assert np.array_equal(got[:len(ref)], ref)
+
+
+@pytest.mark.parametrize("nx,ny", [(64, 512), (65, 1000), (1000, 65), (272, 1056), (512, 512),
+                                   (1030, 1001)])
+@pytest.mark.parametrize("op,dtype", [("euler_rk2", "f64"), ("euler_kahan", "f32"),
+                                      ("euler_kahan", "bf16")])
+def test_naive_euler_gives_the_same_bits_by_walks_and_by_points(oracle_lib, op, dtype, nx, ny):
+    """Grids on both sides of the choice between a thread a point and the walks of
+    each shape against the oracle; a batch of the one grid, which may choose the
+    other, gives the same midpoint planes, too."""
+    U = inputs.euler_pulse(nx, ny, 4, gamma=1.4)
+    np_dtype = np.float64
+    if op == "euler_kahan":
+        U = U.astype(np.float32)
+        np_dtype = np.float32
+        if dtype == "bf16":
+            U = torch.from_numpy(U).to(torch.bfloat16).view(torch.int16).numpy().view(np.uint16)
+            np_dtype = np.uint16
+    Uf = (oracle_lib.bf16_bits_to_f32(U) if dtype == "bf16" else U).astype(np.float64)
+    a, dt = oracle_lib.euler_setup(Uf, 1.4, 0.3)
+    u0 = np.concatenate([U, U] + ([np.zeros_like(U)] if op == "euler_kahan" else []))
+    ref = oracle_lib.euler_rk2(U, 1.4, dt, 0.5, a, 3) if op == "euler_rk2" else \
+        oracle_lib.euler_kahan(u0, 1.4, dt, 0.5, a, 3, dtype)
+    with Swept2D(nx, ny, op=op, tile=0, params=(1.4, 0.3, 0.5), dtype=dtype) as s:
+        s.set_state(u0)
+        s.advance(1, mode="naive")
+        s.advance(2, mode="naive")
+        got = s.get_state()
+    with SweptBatch([nx], [ny], [0], op=op, params=(1.4, 0.3, 0.5), dtype=dtype) as b:
+        b.set_state([u0.astype(np_dtype)])
+        b.advance(3, mode="naive")
+        other = b.split(b.get_state())[0]
+    assert np.array_equal(got[:len(ref)], ref)
+    assert np.array_equal(got, other)
