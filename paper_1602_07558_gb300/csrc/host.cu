@@ -51,9 +51,11 @@ struct swept2d {
     int nx = 0, ny = 0, nv = 0, nst = 0, n = 0, op = 0, dtype = 0, esize = 0;
     Geom G{};
     const OpTable *ops = nullptr;
-    // the update's marching form (nullptr: none), the grid's shape and cut for
-    // it, and its counters (one per tile, the item counter)
+    // the update's marching form (nullptr: none), whether the swept mode and the
+    // persistent one take it, the grid's shape and cut for it, and its counters (one
+    // per tile, the item counter)
     const swept::MarchTable *mt = nullptr;
+    bool marches[2] = {false, false};
     int mshape = 0;
     swept::MarchGrid mgrid{};
     int *msched = nullptr;
@@ -262,7 +264,7 @@ int march_substeps(swept2d *h, long long total, int first, long long spin_limit)
 
 int swept_substeps(swept2d *h, long long total, bool persistent) {
     // (a trace records the items of the persistent swept form)
-    if (h->mt && !(persistent && h->trace))
+    if (h->mt && h->marches[persistent] && !(persistent && h->trace))
         return march_substeps(h, total, 0, swept::kPersistSpinLimit);
     const int half = h->n / 2;
     const long long H = total / half;
@@ -478,8 +480,12 @@ int swept2d_create(swept2d_t **out, int nx, int ny, int nvars, int nstages, int 
     }
     h->mt = tile ? march_for(op, dtype) : nullptr;
     if (h->mt) {
-        h->mshape = h->mt->shape(&nx, &ny, 1, false);
-        if (h->mshape < 0) h->mt = nullptr;
+        for (int p = 0; p < 2; ++p) {
+            const int shape = h->mt->shape(&nx, &ny, &tile, 1, p != 0);
+            h->marches[p] = shape >= 0;
+            if (shape >= 0) h->mshape = shape;
+        }
+        if (!h->marches[0] && !h->marches[1]) h->mt = nullptr;
     }
     if (h->mt) {
         h->mgrid = h->mt->cut(h->mshape, nx, ny);
@@ -567,11 +573,12 @@ int swept2d_selftest_wait_timeout(swept2d_t *h, long long spin_limit) {
     if (rc) return rc;
     // the first phase's items skipped: every item taken waits for a counter that
     // nothing releases
-    const int NT = h->mt ? h->mgrid.bx * h->mgrid.by : h->G.T * h->G.Q;
+    const bool march = h->mt && h->marches[1];
+    const int NT = march ? h->mgrid.bx * h->mgrid.by : h->G.T * h->G.Q;
     cudaError_t e = cudaMemsetAsync(h->sched, 0, ((size_t)h->G.T * h->G.Q + 1) * sizeof(int),
                                     h->stream);
     if (e != cudaSuccess) return cuda_fail(h, e, "selftest schedule reset");
-    if (h->mt)
+    if (march)
         rc = march_substeps(h, 2LL * h->nst * h->mt->steps(h->mshape), NT, spin_limit);
     else rc = launch(h, SWEPT2D_K_OCTAHEDRON, "persistent kernel (wait-timeout self-test)", [&] {
         return h->ops->persistent(h->G, h->consts, h->state, h->up, h->br, h->sched, 1,

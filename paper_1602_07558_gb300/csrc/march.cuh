@@ -16,6 +16,7 @@
 // blocks is resident. Waits are bounded, as in the persistent form.
 #pragma once
 #include <climits>
+#include <cmath>
 #include <type_traits>
 
 #include "exact64.cuh"
@@ -768,35 +769,120 @@ inline int march_steps(int shape) {
     return k;
 }
 
-// The largest shape that gives the GPU's 152 SMs three tiles each (all grids
-// together), else the smallest one; -1 where the swept kernels do better, unless
-// `always`. That is only so in binary64, whose redundant points cost FP64 time:
-//  - heat, when its tiles fill less than 0.78 of their 64 columns and the grid is
-//    too large to be bound by latency (fields with a zero crossing in every tile,
-//    96 steps, us, swept / marching: 64 x 2048 292 / 437, 192 x 384 241 / 281, but
-//    48 x 512 221 / 181, 256 x 256 241 / 232, 1024 x 1024 1469 / 706);
-//  - Euler, in a middle range of sizes, where the SMs hold one small tile each
-//    (32 stages, us, swept / marching: 128 x 128 344 / 336, 160 x 160 355 / 436,
-//    256 x 256 576 / 727, 192 x 384 574 / 712, 320 x 320 827 / 778, 64 x 2048
-//    1134 / 970).
+// All grids' tiles in a shape.
 template <class Op>
-inline int march_shape(const int *nx, const int *ny, int count, bool always) {
-    double points = 0, columns = 0;
-    int shape = 0;
-    for (;; ++shape) {
-        long long tiles = 0;
-        points = columns = 0;
-        for (int i = 0; i < count; ++i) {
-            const MarchGrid g = march_cut<Op>(shape, nx[i], ny[i]);
-            tiles += (long long)g.bx * g.by;
-            points += (double)nx[i] * ny[i];
-            columns += 64.0 * g.bx * ny[i];
-        }
-        if (tiles >= 3 * 152 || shape + 1 == MarchShapes<Op>::kCount) break;
+inline long long march_tiles(int shape, const int *nx, const int *ny, int count) {
+    long long tiles = 0;
+    for (int i = 0; i < count; ++i) {
+        const MarchGrid g = march_cut<Op>(shape, nx[i], ny[i]);
+        tiles += (long long)g.bx * g.by;
     }
-    if (always) return shape;
-    if (std::is_same<Op, HeatOp>::value && points > 28000 && points < 0.78 * columns) return -1;
-    if (std::is_same<Op, EulerOp>::value && points > 20000 && points < 90000) return -1;
+    return tiles;
+}
+
+// Binary64 Euler: the µs of a step (two stages). A step of one tile alone takes
+// `alone`; with more than about 76 tiles blocks share an SM's FP64 pipe, up to 2.7
+// times that, and many tiles take `each`, where a walk of a grid of few rows is
+// shorter (a row more forms fluxes at either end). Measured on the GB300, tiles: µs -
+//   shape 0: 20: 170, 85: 255, 136: 319, 475: 523, 1088: 1142
+//   shape 1: 72: 89, 96: 142, 170: 200, 288: 249, 576: 323, 2272: 1218
+//   shape 2: 60: 28.8, 96: 45, 168: 61, 336: 75, 576: 92, 1152: 185, 2304: 365
+//   shape 3: 96: 19.0, 260: 28, 512: 42, 1000: 49, 1440: 68, 2560: 120
+inline double euler_march_cost(int shape, const int *nx, const int *ny, int count) {
+    double tiles = 0, full = 0;
+    with_march_shape<EulerOp>(shape, [&](auto *body) {
+        typedef typename std::remove_pointer<decltype(body)>::type B;
+        for (int i = 0; i < count; ++i) {
+            const MarchGrid g = march_cut<EulerOp>(shape, nx[i], ny[i]);
+            const double rows = (double)ny[i] / g.by / B::kWalks;
+            tiles += (double)g.bx * g.by;
+            full += (double)g.bx * g.by * ((rows < 1 ? 1 : rows) + 2) / (B::HR + 2);
+        }
+        return cudaSuccess;
+    });
+    static const double alone[] = {169.6, 88.6, 28.5, 17.4}, each[] = {1.05, 0.537, 0.1585, 0.047},
+                        spread[] = {75, 75, 75, 306};
+    double crowd = 1.0 + (tiles - 76) / spread[shape];
+    crowd = crowd < 1.0 ? 1.0 : crowd > 2.7 ? 2.7 : crowd;
+    const double one = alone[shape] * crowd, all = each[shape] * full;
+    return one > all ? one : all;
+}
+// The same of the swept kernels, whose launches are per tile side n (0: the naive
+// ones): n = 8: 64 tiles 18.4, 400: 33, 1024: 81, 4096: 282; n = 16: 144: 22, 256: 36,
+// 576: 71, 1024: 119; n = 32: 64: 47, 144: 53, 256: 99, 400: 149, 576: 196, 1024: 342;
+// n = 40: 64: 67, 144: 82, 256: 164, 400: 245, 576: 327 (whole waves of the SMs, as the
+// tiles grow). One persistent launch takes more where the tiles about fill the SMs:
+// n = 16: 144: 29, n = 32: 64: 57, 144: 82, 256: 94, 576: 191.
+inline double euler_swept_cost(int n, double tiles, bool persistent) {
+    if (n == 0) return 18.7 + 16.3 / 152 * tiles;
+    double t = 17.3 + 0.00442 * std::pow((double)n, 2.6);
+    const double wave = n >= 20 ? 0.6 + 0.01 * n : 0.38 + 0.0225 * n;   // of each after the first
+    if (persistent && tiles > 200) return t * (1.0 + wave * (tiles / 152 - 0.95 + 0.004 * n));
+    const double more = (double)(((long long)tiles - 1) / 152);
+    if (n >= 20)
+        t *= tiles <= 100 ? 0.88 : 1.0 + wave * (more == 1 ? 0.93 : more);
+    else if (more > 0)
+        t *= more == 1 ? 1.16 + 0.028 * n : more == 2 ? 1.25 + 0.067 * n : 1.0 + wave * more;
+    if (!persistent || tiles <= 48) return t;
+    if (n >= 36) return 1.05 * t;
+    return t * (tiles > 100 ? 1.0 + (n < 25 ? 0.02 * n : 0.5) : n < 20 ? 1.06 : 1.25);
+}
+inline double euler_swept_cost(const int *nx, const int *ny, const int *tile, int count,
+                               bool persistent) {
+    double t = 0;
+    for (int i = 0; i < count; ++i) {
+        const int n = tile[i];
+        bool seen = false;
+        for (int k = 0; k < i && !seen; ++k) seen = tile[k] == n;
+        if (seen) continue;
+        double tiles = 0;
+        for (int k = i; k < count; ++k)
+            if (tile[k] == n)
+                tiles += n ? (double)(nx[k] / n) * (ny[k] / n)
+                           : (double)((nx[k] + 31) / 32) * ((ny[k] + 7) / 8);
+        t += euler_swept_cost(n, tiles, persistent);
+    }
+    return t;
+}
+
+// The shape for these grids (all together) with the callers' tile sides, -1 where
+// the swept kernels (as a persistent launch or not) do better; without tile sides, a
+// shape in any case.
+//  - The largest shape that gives the GPU's 152 SMs three tiles each, else the
+//    smallest one. Binary64 heat, whose redundant points may cost FP64 time, stays
+//    with the swept kernels when its tiles fill less than 0.78 of their 64 columns
+//    and the grid is too large to be bound by latency (fields with a zero crossing in
+//    every tile, 96 steps, us, swept / marching: 64 x 2048 292 / 437, 192 x 384 241 /
+//    281, but 48 x 512 221 / 181, 256 x 256 241 / 232, 1024 x 1024 1469 / 706).
+//  - Binary64 Euler, bound by the FP64 pipe in either form: the least of the costs
+//    above (us a step, swept at the tile given / marching: 64 x 2048, 32, 54 / 61;
+//    384 x 384, 32, 54 / 68; 48 x 512, 16, 22 / 27; 128 x 512, 32, 47 / 43; 256 grids
+//    of 32..96 460 / 385, by the largest shape that fills the SMs 450).
+template <class Op>
+inline int march_shape(const int *nx, const int *ny, const int *tile, int count, bool persistent) {
+    if constexpr (std::is_same<Op, EulerOp>::value) {
+        int best = 0;
+        double least = 0;
+        for (int s = 0; s < MarchShapes<Op>::kCount; ++s) {
+            const double t = euler_march_cost(s, nx, ny, count);
+            if (s == 0 || t < least) {
+                least = t;
+                best = s;
+            }
+        }
+        return tile && euler_swept_cost(nx, ny, tile, count, persistent) < least ? -1 : best;
+    }
+    int shape = 0;
+    while (march_tiles<Op>(shape, nx, ny, count) < 3 * 152 && shape + 1 < MarchShapes<Op>::kCount)
+        ++shape;
+    if (tile && std::is_same<Op, HeatOp>::value) {
+        double points = 0, columns = 0;
+        for (int i = 0; i < count; ++i) {
+            points += (double)nx[i] * ny[i];
+            columns += 64.0 * march_cut<Op>(shape, nx[i], ny[i]).bx * ny[i];
+        }
+        if (points > 28000 && points < 0.78 * columns) return -1;
+    }
     return shape;
 }
 

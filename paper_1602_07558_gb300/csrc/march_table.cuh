@@ -6,8 +6,10 @@ namespace swept {
 
 // Functions of one update's marching form (march_*.cu).
 struct MarchTable {
-    // the shape for these grids; -1 (unless `always`): the swept kernels do better
-    int (*shape)(const int *nx, const int *ny, int count, bool always);
+    // the shape for these grids; -1 where the swept kernels with these tile sides, in
+    // the launch-per-phase or the persistent form, do better (without tile sides, a
+    // shape in any case)
+    int (*shape)(const int *nx, const int *ny, const int *tile, int count, bool persistent);
     int (*steps)(int shape);     // steps a phase
     MarchGrid (*cut)(int shape, int nx, int ny);
     // the shape whose walks (phase_one) are the quickest for the naive sub-steps of

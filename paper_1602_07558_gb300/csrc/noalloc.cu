@@ -129,7 +129,7 @@ int advance_static(const double *u_in, double *u_out, int nx, int ny, int tile, 
     // an error word; two panel sets hold more than four times the state, so they
     // fit wherever the check above passed
     const swept::MarchTable *mt = swept::marchtable_heat();
-    const int shape = mt->shape(&nx, &ny, 1, true);
+    const int shape = mt->shape(&nx, &ny, nullptr, 1, false);
     const swept::MarchGrid cut = mt->cut(shape, nx, ny);
     const int tiles = cut.bx * cut.by;
     void *tmp = base;

@@ -292,3 +292,21 @@ def test_naive_euler_gives_the_same_bits_by_walks_and_by_points(oracle_lib, op, 
         other = b.split(b.get_state())[0]
     assert np.array_equal(got[:len(ref)], ref)
     assert np.array_equal(got, other)
+
+
+@pytest.mark.parametrize("mode,graph", [("swept", False), ("swept", True), ("persistent", False)])
+@pytest.mark.parametrize("nx,ny,tile", [(64, 2048, 32), (384, 384, 32), (48, 512, 16), (128, 512, 32),
+                                        (560, 70, 10), (2000, 40, 8)])
+def test_binary64_euler_gives_the_same_bits_in_either_form(oracle_lib, nx, ny, tile, mode, graph):
+    """Grids on both sides of the choice between the swept kernels and the marching
+    form's shapes, which differs between the two swept modes; five steps (a tail of
+    sub-steps that fill no half cycle), then three more."""
+    U = inputs.euler_pulse(nx, ny, 4, gamma=1.4)
+    a, dt = oracle_lib.euler_setup(U, 1.4, 0.3)
+    ref = oracle_lib.euler_rk2(U, 1.4, dt, 0.5, a, 8)
+    with Swept2D(nx, ny, op="euler_rk2", tile=tile, params=(1.4, 0.3, 0.5),
+                 stream=torch.cuda.Stream()) as s:
+        s.set_state(np.concatenate([U, U]))
+        s.advance(5, mode=mode, graph=graph)
+        s.advance(3, mode=mode, graph=graph)
+        assert np.array_equal(s.get_state()[:4], ref)
