@@ -51,9 +51,9 @@ struct swept2d {
     int nx = 0, ny = 0, nv = 0, nst = 0, n = 0, op = 0, dtype = 0, esize = 0;
     Geom G{};
     const OpTable *ops = nullptr;
-    // the update's marching form (nullptr: none), whether the swept mode and the
-    // persistent one take it, the grid's shape and cut for it, and its counters (one
-    // per tile, the item counter)
+    // the update's marching form (nullptr: none or never taken), whether the swept
+    // mode and the persistent one take it, the grid's shape and cut for it, and its
+    // counters (one per tile, the item counter)
     const swept::MarchTable *mt = nullptr;
     bool marches[2] = {false, false};
     int mshape = 0;
@@ -264,9 +264,17 @@ int march_substeps(swept2d *h, long long total, int first, long long spin_limit)
 
 int swept_substeps(swept2d *h, long long total, bool persistent) {
     // (a trace records the items of the persistent swept form)
-    if (h->mt && h->marches[persistent] && !(persistent && h->trace))
-        return march_substeps(h, total, 0, swept::kPersistSpinLimit);
     const int half = h->n / 2;
+    if (h->mt && !(persistent && h->trace)) {
+        // (binary64 Euler: what fills no half cycle has the marching form or naive
+        // launches to choose from, whichever form the longer advances take)
+        const bool any = h->op == SWEPT2D_OP_EULER_RK2 && total < half;
+        if ((any || h->marches[persistent]) &&
+            h->mt->is_short(h->mshape, h->nx, h->ny, h->n, total))
+            return naive_substeps(h, total);
+        if (any || h->marches[persistent])
+            return march_substeps(h, total, 0, swept::kPersistSpinLimit);
+    }
     const long long H = total / half;
     const long long rem = total - H * half;
     if (H > 0 && persistent) {
@@ -480,12 +488,10 @@ int swept2d_create(swept2d_t **out, int nx, int ny, int nvars, int nstages, int 
     }
     h->mt = tile ? march_for(op, dtype) : nullptr;
     if (h->mt) {
-        for (int p = 0; p < 2; ++p) {
-            const int shape = h->mt->shape(&nx, &ny, &tile, 1, p != 0);
-            h->marches[p] = shape >= 0;
-            if (shape >= 0) h->mshape = shape;
-        }
-        if (!h->marches[0] && !h->marches[1]) h->mt = nullptr;
+        h->mshape = h->mt->shape(&nx, &ny, nullptr, 1, false);
+        for (int p = 0; p < 2; ++p)
+            h->marches[p] = h->mt->shape(&nx, &ny, &tile, 1, p != 0) >= 0;
+        if (!h->marches[0] && !h->marches[1] && op != SWEPT2D_OP_EULER_RK2) h->mt = nullptr;
     }
     if (h->mt) {
         h->mgrid = h->mt->cut(h->mshape, nx, ny);

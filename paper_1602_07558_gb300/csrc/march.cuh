@@ -817,7 +817,8 @@ inline double euler_swept_cost(int n, double tiles, bool persistent) {
     if (n == 0) return 18.7 + 16.3 / 152 * tiles;
     double t = 17.3 + 0.00442 * std::pow((double)n, 2.6);
     const double wave = n >= 20 ? 0.6 + 0.01 * n : 0.38 + 0.0225 * n;   // of each after the first
-    if (persistent && tiles > 200) return t * (1.0 + wave * (tiles / 152 - 0.95 + 0.004 * n));
+    if (persistent && tiles > 200)                // (13 µs a wave at n = 8, 17.5, 47.5 at n = 32)
+        return (t - 5.3) * (n >= 20 ? std::ceil(tiles / 152) : tiles / 152 + 0.2);
     const double more = (double)(((long long)tiles - 1) / 152);
     if (n >= 20)
         t *= tiles <= 100 ? 0.88 : 1.0 + wave * (more == 1 ? 0.93 : more);
@@ -963,6 +964,34 @@ inline int naive_shape(int nx, int ny) {
     return best;
 }
 
+// Whether an advance of one grid by `substeps` sub-steps is quicker as so many naive
+// launches than as one launch in the marching form, whose ring and first phase it
+// then has alone (a batch's naive launches take a thread a point: it marches). Measured on the GB300, us by the stream, naive launches / marching:
+//   heat binary64: 256 x 256, 2 steps 10.9 / 12.9, 4: 19.1 / 19.0; 768 x 768, 2: 22 / 27,
+//     4: 43 / 40; 2048 x 2048, 2: 46 / 74, 6: 140 / 157 (mixed signs 251 / 290), 16: 370 /
+//     371; 4096 x 4096, 6: 510 / 514 (mixed signs 836 / 1090)
+//   heat binary32: 256 x 256, 1 step 5.4 / 10.3, 2: 9.8 / 9.9, 3: 14.4 / 9.8; 2048 x 2048, 1:
+//     15.9 / 33, 2: 28 / 33, 3: 41 / 33
+//   Euler binary32: 256 x 256, 1 step 11.9 / 15.8, 2: 20.3 / 22.2, 3: 28.6 / 28.8
+//   Euler binary64 (by both forms' costs; never more than the caller's half cycle, which
+//     the swept form would not fill either): 80 x 320, 3 steps 76 / 104; 384 x 192, 3: 126 /
+//     147; 64 x 64, 1: 24 / 21
+template <class Op>
+inline bool march_short(int shape, int nx, int ny, int tile, long long substeps) {
+    if constexpr (std::is_same<Op, HeatOp>::value) {
+        return substeps <= 3 || (substeps <= 6 && (double)nx * ny >= 2e6);
+    } else if constexpr (std::is_same<Op, EulerOp>::value) {
+        if (substeps >= tile / 2) return false;
+        const int s = naive_shape<Op>(nx, ny);
+        const WaveCost cost = naive_costs<Op>()[s < 0 ? MarchShapes<Op>::kCount : s];
+        const double naive = cost(s < 0 ? ((nx + 31LL) / 32) * ((ny + 7) / 8)
+                                        : march_tiles<Op>(s, &nx, &ny, 1));
+        return 0.5 * (double)substeps * (naive - euler_march_cost(shape, &nx, &ny, 1)) < 6;
+    } else {
+        return substeps <= 2 * Op::NST;
+    }
+}
+
 // Queues `steps` steps over NT tiles: reads `src`, writes b0, b1, b0, ... phase
 // by phase (src may be b1). sched: NT counters and the item counter; without `err`
 // the word after them is the error word and is cleared with them. `launches` is
@@ -1063,8 +1092,8 @@ struct March {
     }
     static const MarchTable *table() {
         static const MarchTable t = {&march_shape<Op>, &march_steps<Op>, &march_cut<Op>,
-                                     &naive_shape<Op>, &one, &many, &phase_one,
-                                     &phase_many};
+                                     &march_short<Op>, &naive_shape<Op>, &one, &many,
+                                     &phase_one, &phase_many};
         return &t;
     }
 };

@@ -12,6 +12,8 @@ struct MarchTable {
     int (*shape)(const int *nx, const int *ny, const int *tile, int count, bool persistent);
     int (*steps)(int shape);     // steps a phase
     MarchGrid (*cut)(int shape, int nx, int ny);
+    // whether an advance of so few sub-steps of one grid is quicker by naive launches
+    bool (*is_short)(int shape, int nx, int ny, int tile, long long substeps);
     // the shape whose walks (phase_one) are the quickest for the naive sub-steps of
     // one grid, -1 for a thread a point
     int (*naive_shape)(int nx, int ny);

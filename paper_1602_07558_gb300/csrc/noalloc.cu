@@ -133,15 +133,27 @@ int advance_static(const double *u_in, double *u_out, int nx, int ny, int tile, 
     const swept::MarchGrid cut = mt->cut(shape, nx, ny);
     const int tiles = cut.bx * cut.by;
     void *tmp = base;
+    const double consts[8] = {r, 0, 0, 0, 0, 0, 0, 0};
+    cudaError_t e = cudaSuccess;
+    if (!skip && mt->is_short(shape, nx, ny, tile, nsteps)) {
+        // naive launches, the last of which lands in u_out
+        const void *src = u_in;
+        for (long long i = 0; i < nsteps && e == cudaSuccess; ++i) {
+            void *dst = (nsteps - 1 - i) % 2 == 0 ? (void *)u_out : tmp;
+            e = swept::optable_heat()->naive(G, consts, src, dst, (unsigned long long)i, st);
+            src = dst;
+        }
+        if (e != cudaSuccess) set_err(err, errlen, cudaGetErrorString(e));
+        return e == cudaSuccess ? SWEPT2D_OK : SWEPT2D_ECUDA;
+    }
     int *sched = (int *)((char *)base + align256(state_bytes));
     // the buffers alternate phase by phase; the last phase writes u_out
     if (skip) nsteps = 2LL * mt->steps(shape);
     const long long phases = (nsteps + mt->steps(shape) - 1) / mt->steps(shape);
     void *b0 = (phases & 1) ? (void *)u_out : tmp, *b1 = (phases & 1) ? tmp : (void *)u_out;
-    const double consts[8] = {r, 0, 0, 0, 0, 0, 0, 0};
     void *out = nullptr;
     long long made = 0;
-    cudaError_t e = mt->one(shape, cut, consts, u_in, b0, b1, sched, nsteps, nullptr,
+    e = mt->one(shape, cut, consts, u_in, b0, b1, sched, nsteps, nullptr,
                             skip ? tiles : 0, spin_limit, &out, &made, st);
     if (e == cudaSuccess)
         e = swept::launch_after(spoil_if_failed, dim3(152), 256, 0, st, sched + tiles + 1, u_out,

@@ -310,3 +310,35 @@ def test_binary64_euler_gives_the_same_bits_in_either_form(oracle_lib, nx, ny, t
         s.advance(5, mode=mode, graph=graph)
         s.advance(3, mode=mode, graph=graph)
         assert np.array_equal(s.get_state()[:4], ref)
+
+
+@pytest.mark.parametrize("op,dtype,nx,ny,tile", [
+    ("heat", "f64", 64, 48, 16), ("heat", "f64", 2048, 1024, 64), ("heat_kahan", "f32", 64, 48, 16),
+    ("heat_kahan", "bf16", 64, 48, 16), ("euler_rk2", "f64", 80, 320, 40),
+    ("euler_kahan", "f32", 64, 48, 16), ("euler_kahan", "bf16", 64, 48, 16)])
+def test_short_advances_take_naive_launches_with_the_same_bits(op, dtype, nx, ny, tile):
+    """Up to a few sub-steps an advance in a swept mode is one naive launch each; every
+    split of eight steps, by stream and by graph, ends in the same state."""
+    if op.startswith("euler"):
+        U, params = inputs.euler_pulse(nx, ny, 4, gamma=1.4), (1.4, 0.3, 0.5)
+        u0 = np.concatenate([U, U] + ([np.zeros_like(U)] if op == "euler_kahan" else []))
+    else:
+        u, params = 1.0 + np.random.default_rng(1).random((1, ny, nx)), (0.2,)
+        u0 = np.concatenate([u] + ([np.zeros_like(u)] if op == "heat_kahan" else []))
+    if dtype != "f64":
+        u0 = u0.astype(np.float32)
+    if dtype == "bf16":
+        u0 = torch.from_numpy(u0).to(torch.bfloat16).view(torch.int16).numpy().view(np.uint16)
+    with Swept2D(nx, ny, op=op, tile=tile, params=params, dtype=dtype,
+                 stream=torch.cuda.Stream()) as s:
+        results = []
+        for split in ([8], [1] * 8, [2] * 4, [3, 4, 1], [7, 1]):
+            for mode, graph in (("swept", False), ("persistent", True), ("naive", False)):
+                s.set_state(u0)
+                launches = s.query("launches")
+                for k in split:
+                    s.advance(k, mode=mode, graph=graph)
+                if split == [1] * 8:
+                    assert s.query("launches") - launches == 8 * s.nstages
+                results.append(s.get_state())
+    assert all(np.array_equal(results[0], r) for r in results)
