@@ -4,11 +4,12 @@
 // SM can issue 76 others; the heat update has four FP64 operations, p = a + b
 // (the pair sum, shared by two points), s = p1 + p2, d = fma(-4, c, s) and
 // u' = fma(r, d, c). Here the magnitudes of a block whose values have one sign
-// are 64-bit integers in one unit, a quarter of the last place of binade e0,
-// which represents the normal numbers of the binades e0 .. e0 + 5 exactly:
+// are 64-bit integers in one unit, a quarter of the last place of the lowest one's
+// binade e0, which represents the normal numbers of the binades e0 .. e0 + 5 exactly:
 //  - a sum is an integer addition and a rounding, to nearest even, to the 53
 //    leading bits (the position of the first bit gives the rounding's);
-//  - K = s / 4 - c is a multiple of 4, and d = 4 K is exact while |K| < 2^55;
+//  - K = s / 4 - c is a multiple of 4, and d = 4 K is exact while |K| < 2^55, twice
+//    the lowest value of binade e0: always, if the values differ by less;
 //  - r d = 4 r K = R K 2^-64 with a 64-bit integer R for r in [1/8, 1/4), a
 //    128-bit product whose lower half only tells whether something lies below
 //    the unit; the unit's two bits below a last place are enough for the same
@@ -19,7 +20,8 @@
 // operations; blocks on a zero crossing, or with values more than a factor of 32
 // to 64 apart, take them from the start. Measured on the GB300: 4096², 500 steps,
 // 36.5 ms with this (the integer ALU 68% busy), 67.4 by the FP64 operations of the
-// swept kernels (their pipe 95% busy).
+// swept kernels (their pipe 95% busy). On the host the same functions serve to compare
+// them with the FP64 operations.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -38,17 +40,25 @@ __host__ __device__ inline unsigned long long heat_ratio(double r) {
 constexpr int kFixedBinades = 6;
 
 // Position of the first set bit of a positive value's upper word.
-__device__ __forceinline__ int first_bit(long long v) {
+__host__ __device__ __forceinline__ int first_bit(long long v) {
+#ifdef __CUDA_ARCH__
     int p;
     asm("bfind.u32 %0, %1;" : "=r"(p) : "r"((unsigned)(v >> 32)));
     return p;
+#else
+    return 31 - __builtin_clz((unsigned)(v >> 32));
+#endif
 }
 
 // v rounded to its 53 leading bits, to nearest even (2^53 < v < 2^63).
-__device__ __forceinline__ long long leading_53(long long v) {
+__host__ __device__ __forceinline__ long long leading_53(long long v) {
     const int at = first_bit(v) - 20;            // the last of the 53 bits
     unsigned below;
+#ifdef __CUDA_ARCH__
     asm("bmsk.clamp.b32 %0, 0, %1;" : "=r"(below) : "r"(at));
+#else
+    below = (1u << at) - 1u;
+#endif
     return (v + ((below >> 1) + (((unsigned)v >> at) & 1u))) & ~(long long)below;
 }
 
@@ -62,31 +72,35 @@ struct FixedHeat {
     // Sets the unit for values whose upper words lie in [low, high] as signed
     // integers (of negative values, too, the larger word is the larger magnitude);
     // false unless they are normal, of one sign and within the binades, r has a
-    // ratio, and sums stay finite.
-    __device__ __forceinline__ bool fits(double r, int high, int low) {
-        const int top = (high >> 20) & 0x7ff, bottom = (low >> 20) & 0x7ff;
-        R = heat_ratio(r);
-        e0 = top - (kFixedBinades - 1);
+    // ratio (heat_ratio(r)), and sums stay finite.
+    __host__ __device__ __forceinline__ bool fits(unsigned long long ratio, int high, int low) {
+        const int top = (high >> 20) & 0x7ff;
+        R = ratio;
+        e0 = (low >> 20) & 0x7ff;
         sign = (unsigned)high & 0x80000000u;
         wide = 0;
-        return R != 0 && (high ^ low) >= 0 && bottom >= e0 && e0 > 0 && top < 2040;
+        return R != 0 && (high ^ low) >= 0 && top - e0 < kFixedBinades && e0 > 0 && top < 2040;
     }
-    __device__ __forceinline__ long long from(double v) const {
-        const long long b = __double_as_longlong(v);
-        const int e = (__double2hiint(v) >> 20) & 0x7ff;
+    __host__ __device__ __forceinline__ long long from(double v) const {
+        long long b;
+        memcpy(&b, &v, 8);
+        const int e = (int)(b >> 52) & 0x7ff;
         return ((b & 0xfffffffffffffLL) | 0x10000000000000LL) << (e - e0 + 2);
     }
-    __device__ __forceinline__ double to(long long v) const {
+    __host__ __device__ __forceinline__ double to(long long v) const {
         const int up = first_bit(v) - 22;        // the binade above e0
         const long long b = ((long long)(e0 + up) << 52) | ((v >> (up + 2)) & 0xfffffffffffffLL);
-        return __longlong_as_double(b | (long long)((unsigned long long)sign << 32));
+        const unsigned long long bits = (unsigned long long)b | ((unsigned long long)sign << 32);
+        double v64;
+        memcpy(&v64, &bits, 8);
+        return v64;
     }
     // some result is not the FP64 one
-    __device__ __forceinline__ bool failed() const { return (wide >> 24) != 0; }
-    __device__ __forceinline__ long long sum(long long a, long long b) const {
+    __host__ __device__ __forceinline__ bool failed() const { return (wide >> 24) != 0; }
+    __host__ __device__ __forceinline__ long long sum(long long a, long long b) const {
         return leading_53(a + b);
     }
-    __device__ __forceinline__ long long next(long long c, long long pe, long long pw) {
+    __host__ __device__ __forceinline__ long long next(long long c, long long pe, long long pw) {
         const long long K = (sum(pe, pw) >> 2) - c;
         wide = max(wide, (unsigned)(K >> 32) + (1u << 23));
         const unsigned long long Kb = (unsigned long long)(K + (1LL << 61));   // 2^61 R 2^-64 = R / 8

@@ -41,7 +41,6 @@
 
 #include <climits>
 
-#include "exact64.cuh"
 #include "ops.cuh"
 
 namespace swept {
@@ -797,7 +796,7 @@ __global__ void __launch_bounds__(256) naive_heat_kernel(HeatOp op, Geom G, cons
         high = __reduce_max_sync(0xffffffffu, high);
         low = __reduce_min_sync(0xffffffffu, low);
         FixedHeat f;
-        done = f.fits(op.r, high, low);
+        done = f.fits(op.R, high, low);
         if (done) {
             long long c = f.from(u[1]);
             long long pp = f.sum(__shfl_down_sync(0xffffffffu, f.from(u[0]), 1), c);

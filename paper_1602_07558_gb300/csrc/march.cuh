@@ -394,7 +394,7 @@ struct HeatMarch {
                 low = min(low, sm.low[w]);
             }
             FixedCell fixed;
-            if (fixed.f.fits(op.r, high, low)) {
+            if (fixed.f.fits(op.R, high, low)) {
                 L2 v[R], none[1];
 #pragma unroll
                 for (int j = 0; j < R; ++j) v[j] = two(fixed.f.from(u[j].l), fixed.f.from(u[j].h));

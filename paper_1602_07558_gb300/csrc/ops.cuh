@@ -28,6 +28,8 @@
 #include <cstdint>
 #include <cstring>
 
+#include "exact64.cuh"
+
 typedef unsigned long long u64;
 
 namespace swept {
@@ -42,7 +44,8 @@ struct HeatOp {
     static constexpr bool INPLACE = false;
     static constexpr bool INPLACE_AFTER_AUX = true;
     double r;
-    __host__ __device__ explicit HeatOp(const double *c) : r(c[0]) {}
+    u64 R;                   // r on the integer units
+    __host__ __device__ explicit HeatOp(const double *c) : r(c[0]), R(heat_ratio(c[0])) {}
     template <class A>
     __device__ __forceinline__ void operator()(int, u64, const A &a, S *out) const {
         const double c = a(0, 0, 0);
