@@ -10,10 +10,10 @@
 //    leading bits (the position of the first bit gives the rounding's);
 //  - K = s / 4 - c is a multiple of 4, and d = 4 K is exact while |K| < 2^55, twice
 //    the lowest value of binade e0: always, if the values differ by less;
-//  - r d = 4 r K = R K 2^-64 with a 64-bit integer R for r in [1/8, 1/4), a
-//    128-bit product whose lower half only tells whether something lies below
-//    the unit; the unit's two bits below a last place are enough for the same
-//    rounding of c + r d.
+//  - r d = 4 r K = R K 2^-64 with a 64-bit integer R, a multiple of 8, for r in
+//    [2^-11, 1/4), a 128-bit product whose lower half only tells whether something
+//    lies below the unit; the unit's two bits below a last place are enough for the
+//    same rounding of c + r d.
 // A new value is a rounded mean of old ones with weights 1 - 4r and r, so it
 // stays within the block's extremes, hence in the six binades. A K that is too
 // large is recorded, and the caller repeats the block's steps by the FP64
@@ -29,12 +29,13 @@
 
 namespace swept {
 
-// 4 r as R 2^-64, or 0 when r is not in [1/8, 1/4).
+// 4 r as R 2^-64, R a multiple of 8; 0 when r is not in [2^-11, 1/4).
 __host__ __device__ inline unsigned long long heat_ratio(double r) {
-    if (!(r >= 0.125 && r < 0.25)) return 0;
+    if (!(r >= 0.00048828125 && r < 0.25)) return 0;
     unsigned long long bits;
     memcpy(&bits, &r, 8);
-    return ((bits & 0xfffffffffffffULL) | 0x10000000000000ULL) << 11;
+    const int below = 1020 - (int)(bits >> 52);          // binades below [1/8, 1/4): 0 .. 8
+    return ((bits & 0xfffffffffffffULL) | 0x10000000000000ULL) << (11 - below);
 }
 
 constexpr int kFixedBinades = 6;

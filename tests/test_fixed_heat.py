@@ -9,7 +9,7 @@ import pytest
 from paper_1602_07558_gb300 import build
 
 HERE = os.path.dirname(os.path.abspath(__file__))
-RS = [0.2499999999, 0.2, 0.1875, 0.125]
+RS = [0.2499999999, 0.2, 0.1875, 0.125, 0.1, 0.0625, 0.05, 0.01, 2.0 ** -11 * 1.3, 2.0 ** -11]
 
 
 @pytest.fixture(scope="module")
@@ -41,7 +41,7 @@ def test_a_block_of_one_binade_never_fails(program, kind):
     assert program(0.2, kind, 2000)[1] == 0
 
 
-@pytest.mark.parametrize("r", [0.25, 0.2500001, 0.1249999, 0.0, -0.1, float("inf"),
+@pytest.mark.parametrize("r", [0.25, 0.2500001, 2.0 ** -11 * 0.9999999, 0.0, -0.1, float("inf"),
                                float("nan")])
 def test_other_diffusion_numbers_are_left_to_the_fp64_operations(program, r):
     assert program(r, "smooth", 5)[0] == 0

@@ -342,3 +342,18 @@ def test_short_advances_take_naive_launches_with_the_same_bits(op, dtype, nx, ny
                     assert s.query("launches") - launches == 8 * s.nstages
                 results.append(s.get_state())
     assert all(np.array_equal(results[0], r) for r in results)
+
+
+@pytest.mark.parametrize("r", [0.0625, 0.05, 0.01, 2.0 ** -11 * 1.3, 2.0 ** -11, 2.0 ** -11 * 0.99])
+@pytest.mark.parametrize("kind", ["one_binade", "binades", "negative", "crossing", "noise",
+                                  "mixed_sign_noise", "ties", "few_bits", "powers", "constant",
+                                  "zeros", "tiny", "smallest_normal", "huge"])
+def test_small_diffusion_numbers_are_bitwise_in_either_mode(oracle_lib, kind, r):
+    u0 = field(kind, 96, 64)
+    with np.errstate(all="ignore"):
+        ref = oracle_lib.heat(u0, r, 21)
+    with Swept2D(96, 64, op="heat", tile=32, params=(r,)) as s:
+        for mode in ("swept", "naive"):
+            s.set_state(u0[None])
+            s.advance(21, mode=mode)
+            assert np.array_equal(s.get_state()[0], ref, equal_nan=True)
