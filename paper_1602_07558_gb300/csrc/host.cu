@@ -495,7 +495,7 @@ int swept2d_create(swept2d_t **out, int nx, int ny, int nvars, int nstages, int 
     }
     if (h->mt) {
         h->mgrid = h->mt->cut(h->mshape, nx, ny);
-        if ((e = cudaMalloc(&h->msched, ((size_t)h->mgrid.bx * h->mgrid.by + 1) * sizeof(int))) !=
+        if ((e = cudaMalloc(&h->msched, (size_t)h->mt->words(h->mshape, nx, ny) * sizeof(int))) !=
             cudaSuccess) {
             cuda_fail(h, e, "schedule allocation");
             return bail(e == cudaErrorMemoryAllocation ? SWEPT2D_ENOMEM : SWEPT2D_ECUDA);

@@ -102,12 +102,14 @@ __device__ __forceinline__ bool march_wait(const MarchTile &m, const int *done, 
     return __syncthreads_or(bad) == 0;
 }
 
-template <class Body, class Op, class Loc>
+// AFTER: launched without a gap to the launch before (launch_after).
+template <class Body, class Op, class Loc, bool AFTER>
 __global__ void __launch_bounds__(Body::kThreads, Body::kMinBlocks)
 march_kernel(Op op, Loc at, MarchRun<typename Op::S> run) {
     typedef typename Op::S S;
     __shared__ typename Body::Smem sm;
     __shared__ int s_item;
+    if constexpr (AFTER) after_previous_launch();
     const int nitems = run.NT * run.phases;
     for (;;) {
         if (threadIdx.x == 0) {
@@ -437,6 +439,70 @@ struct HeatMarch {
     }
 };
 
+// FP64 heat by the FP64 operations, a step a phase, for fields that the integer
+// units cannot take: with no ring of K the pipe, which bounds it, does 1.03 times the
+// work of the points kept (HeatMarch 1.31 and more), as much as the swept kernels. A
+// warp walks down 64 columns, two a lane, of which the outermost only supply
+// neighbours, with the rows above and at the current one in registers; its walks share
+// nothing. 4096², mixed-sign noise, 100 steps, ms: 13.4 (swept 13.5, HeatMarch 17.5);
+// 2048²: 3.44 (3.89, 4.46); 1024 x 512: 0.66 (0.60, 0.75).
+struct HeatWalkOp : HeatOp {
+    __host__ __device__ explicit HeatWalkOp(const double *c) : HeatOp(c) {}
+};
+template <int HR_, int WY_, int MINB_>
+struct HeatWalk {
+    typedef double S;
+    static constexpr int HR = HR_, WY = WY_, K = 1;
+    static constexpr int kThreads = 32 * WY, kMinBlocks = MINB_;
+    static constexpr bool kInPlace = false;
+    static constexpr int kTileCols = 62, kTileRows = HR * WY;
+    struct Smem {};
+    // `steps` is 1, or 0 for a copy (a phase that only moves the state to the other buffer).
+    __device__ static __forceinline__ void run(const HeatOp &op, const MarchTile &m, const S *src,
+                                               S *dst, int, int steps, int, Smem &) {
+        const HeatCell<HeatOp> cell(op);
+        const int wy = threadIdx.x >> 5, c = 2 * (int)(threadIdx.x & 31) - 1;
+        const int y = wy * m.h / WY, n = (wy + 1) * m.h / WY - y;
+        if (n == 0) return;
+        const int gx = wrap_index(m.x0 + c, m.g.nx), ny = m.g.ny;
+        const ptrdiff_t east = gx + 1 == m.g.nx ? 1 - m.g.nx : 1;
+        const bool one = c >= 0 && c < m.w, both = c + 1 < m.w;
+        const size_t nx = m.g.nx, plane = nx * ny;
+        int gy = m.y0 + y == 0 ? ny - 1 : m.y0 + y - 1;      // the row that is read next
+        const S *p = src + (size_t)gy * nx + gx;
+        const auto fetch = [&] {
+            const D2 v = two(p[0], p[east]);
+            const bool last = ++gy == ny;
+            gy = last ? 0 : gy;
+            p += last ? nx - plane : nx;
+            return v;
+        };
+        S *o = dst + (size_t)(m.y0 + y) * nx + gx;
+        const D2 up = fetch();
+        if (steps == 0) {
+            for (int i = 0; i < n; ++i, o += nx) {
+                const D2 u = fetch();
+                if (one) o[0] = u.l;
+                if (both) o[east] = u.h;
+            }
+            return;
+        }
+        D2 at = fetch(), ahead = fetch(), none;
+        D2 pp = cell.pair(east_of(up), at);
+        for (int i = 0; i < n; ++i, o += nx) {
+            const D2 dn = ahead;
+            if (i + 1 < n) ahead = fetch();
+            const D2 pe = cell.pair(east_of(at), dn);
+            D2 u = at;
+            cell.next(u, none, pe, moved_right(pp));
+            if (one) o[0] = u.l;
+            if (both) o[east] = u.h;
+            pp = pe;
+            at = dn;
+        }
+    }
+};
+
 // ------------------------------------------------------------------- Euler
 // Packed arithmetic on two columns, in the update's arithmetic type.
 __device__ __forceinline__ D2 add2(D2 a, D2 b) { return two(__dadd_rn(a.l, b.l), __dadd_rn(a.h, b.h)); }
@@ -659,6 +725,10 @@ struct EulerMarch {
 //   binary32, 2048², 2000 steps (all additions packed): (16, 4, 4, 8) 8.2, (8, 8, 4, 6) 8.9,
 //     (16, 8, 2, 12) 8.7; 1,024 grids of {32..512}²: 25.7, 27.6, 28.0
 //
+// FP64 heat's walks: rows a walk, warps, blocks an SM; ms for 100 steps of mixed-sign noise:
+//   4096² 13.3, 13.6, 14.3, 18.5; 2048² 3.72, 3.44, 3.53, 4.35; 1280² 2.31, 1.77, 1.40,
+//   1.64; 1024² 1.80, 1.50, 1.08, 1.10; 768² 1.37, 1.14, 0.95, 0.68
+//
 // Euler: lanes and rows a walk, warps, blocks an SM. More rows form fewer fluxes
 // twice; more blocks hide the loads' latency, as far as the three rows of values
 // stay in registers (binary64, at the FP64 pipe's rate, needs few); fewer lanes
@@ -682,6 +752,15 @@ struct MarchShapes<HeatOp> {
         std::conditional_t<I == 1, HeatMarch<HeatOp, 4, 8, 4, 4>,
                            std::conditional_t<I == 2, HeatMarch<HeatOp, 2, 8, 4, 3>,
                                               HeatMarch<HeatOp, 1, 8, 4, 2>>>>;
+};
+template <>
+struct MarchShapes<HeatWalkOp> {
+    static constexpr int kCount = 4;
+    template <int I>
+    using Body = std::conditional_t<
+        I == 0, HeatWalk<16, 4, 8>,
+        std::conditional_t<I == 1, HeatWalk<8, 4, 8>,
+                           std::conditional_t<I == 2, HeatWalk<4, 4, 8>, HeatWalk<2, 4, 8>>>>;
 };
 template <>
 struct MarchShapes<EulerOp> {
@@ -968,7 +1047,7 @@ inline int naive_shape(int nx, int ny) {
 // launches than as one launch in the marching form, whose ring and first phase it
 // then has alone (a batch's naive launches take a thread a point: it marches). Measured on the GB300, us by the stream, naive launches / marching:
 //   heat binary64: 256 x 256, 2 steps 10.9 / 12.9, 4: 19.1 / 19.0; 768 x 768, 2: 22 / 27,
-//     4: 43 / 40; 2048 x 2048, 2: 46 / 74, 6: 140 / 157 (mixed signs 251 / 290), 16: 370 /
+//     4: 43 / 40 (with the survey 47, mixed signs 45 / 46); 2048 x 2048, 2: 46 / 74, 6: 140 / 157 (mixed signs 251 / 290), 16: 370 /
 //     371; 4096 x 4096, 6: 510 / 514 (mixed signs 836 / 1090)
 //   heat binary32: 256 x 256, 1 step 5.4 / 10.3, 2: 9.8 / 9.9, 3: 14.4 / 9.8; 2048 x 2048, 1:
 //     15.9 / 33, 2: 28 / 33, 3: 41 / 33
@@ -979,7 +1058,8 @@ inline int naive_shape(int nx, int ny) {
 template <class Op>
 inline bool march_short(int shape, int nx, int ny, int tile, long long substeps) {
     if constexpr (std::is_same<Op, HeatOp>::value) {
-        return substeps <= 3 || (substeps <= 6 && (double)nx * ny >= 2e6);
+        const double points = (double)nx * ny;
+        return substeps <= 3 || (substeps <= 5 && points >= 5e5) || (substeps <= 6 && points >= 2e6);
     } else if constexpr (std::is_same<Op, EulerOp>::value) {
         if (substeps >= tile / 2) return false;
         const int s = naive_shape<Op>(nx, ny);
@@ -992,9 +1072,28 @@ inline bool march_short(int shape, int nx, int ny, int tile, long long substeps)
     }
 }
 
+// One launch of a run whose counters are set.
+template <class B, bool AFTER, class Op, class Loc>
+inline cudaError_t march_launch(const Op &op, const Loc &at, const MarchRun<typename Op::S> &run,
+                                cudaStream_t st) {
+    const auto kern = march_kernel<B, Op, Loc, AFTER>;
+    int per_sm = 0, dev = 0, nsm = 0;
+    const cudaError_t e =
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, B::kThreads, 0);
+    if (e != cudaSuccess) return e;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    long long grid = (long long)(per_sm > 0 ? per_sm : 1) * nsm;
+    if (grid > 2LL * run.NT) grid = 2LL * run.NT;
+    if (grid > (long long)run.NT * run.phases) grid = (long long)run.NT * run.phases;
+    if constexpr (AFTER) return launch_after(kern, dim3((unsigned)grid), B::kThreads, 0, st, op, at, run);
+    kern<<<(int)grid, B::kThreads, 0, st>>>(op, at, run);
+    return cudaGetLastError();
+}
+
 // Queues `steps` steps over NT tiles: reads `src`, writes b0, b1, b0, ... phase
 // by phase (src may be b1). sched: NT counters and the item counter; without `err`
-// the word after them is the error word and is cleared with them. `launches` is
+// the word before them is the error word and is cleared with them. `launches` is
 // raised by the launches made, `*out` set to the buffer with the result.
 template <class Op, class Loc>
 inline cudaError_t march_advance(int shape, const Op &op, const Loc &at, int NT, const void *src,
@@ -1005,18 +1104,12 @@ inline cudaError_t march_advance(int shape, const Op &op, const Loc &at, int NT,
     return with_march_shape<Op>(shape, [&](auto *body) {
         typedef typename std::remove_pointer<decltype(body)>::type B;
         constexpr int K = B::K;
-        const auto kern = march_kernel<B, Op, Loc>;
         if (B::kInPlace) b0 = b1 = const_cast<void *>(src);
-        int per_sm = 0, dev = 0, nsm = 0;
-        cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, B::kThreads, 0);
-        if (e != cudaSuccess) return e;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
         // items of one launch count in an int
         // (an even number of phases: the stages of Euler alternate)
         const long long most = (((1LL << 30) - 1) / NT + 2) & ~1LL;
-        size_t words = (size_t)NT + (err ? 1 : 2);
-        if (!err) err = sched + NT + 1;
+        int *clear = sched;
+        if (!err) err = sched++;
         while (steps > 0) {
             const long long left = (steps + K - 1) / K;
             MarchRun<S> run;
@@ -1032,13 +1125,10 @@ inline cudaError_t march_advance(int shape, const Op &op, const Loc &at, int NT,
             run.last = run.phases < left ? K : (int)(steps - (left - 1) * K);
             run.first = first;
             run.spin_limit = spin_limit;
-            if ((e = cudaMemsetAsync(sched, 0, words * sizeof(int), st)) != cudaSuccess) return e;
-            words = (size_t)NT + 1;
-            long long grid = (long long)(per_sm > 0 ? per_sm : 1) * nsm;
-            if (grid > 2LL * NT) grid = 2LL * NT;
-            if (grid > (long long)NT * run.phases) grid = (long long)NT * run.phases;
-            kern<<<(int)grid, B::kThreads, 0, st>>>(op, at, run);
-            if ((e = cudaGetLastError()) != cudaSuccess) return e;
+            cudaError_t e = cudaMemsetAsync(clear, 0, (sched + NT + 1 - clear) * sizeof(int), st);
+            if (e != cudaSuccess) return e;
+            clear = sched;
+            if ((e = march_launch<B, false>(op, at, run, st)) != cudaSuccess) return e;
             *launches += 1;
             steps -= (long long)(run.phases - 1) * K + run.last;
             *out = run.buf[(run.phases - 1) & 1];
@@ -1050,6 +1140,158 @@ inline cudaError_t march_advance(int shape, const Op &op, const Loc &at, int NT,
         }
         return cudaSuccess;
     });
+}
+
+// ----------------------------------------------------- FP64 heat by its field
+// Whether large FP64 heat grids march on the integer units or by the walks of the
+// FP64 operations depends on the field, which only the device has: a survey of up to
+// 304 tiles counts those that the integer units could not take, and leaves the item
+// counter of the form that does not run behind its last item; both are launched. A
+// tile of which more than 60% are unfit is quicker by the walks (2048², us a step,
+// integer / FP64 tiles / walks: 20.6 / 44.6 / 34.7). Measured on the GB300, the survey
+// and the launch that finds nothing to do: 5 to 8 us an advance.
+constexpr int kEitherSteps = 264;        // steps a survey decides on: whole phase pairs of K = 2, 3, 4
+
+template <class Op>
+__global__ void __launch_bounds__(256) heat_survey_kernel(Op op, MarchGrid g, const double *u,
+                                                          bool soon, unsigned *count, int *march_queue,
+                                                          int march_items, int *walk_queue,
+                                                          int walk_items) {
+    __shared__ int extreme[4][8];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const MarchTile m = OneMarch{g}((int)((long long)blockIdx.x * (g.bx * g.by) / gridDim.x));
+    // 32 rows of the tile (the last repeated), 8 values a thread
+    int high = INT_MIN, low = INT_MAX;
+    double sum = 0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const size_t y = m.y0 + min(4 * warp + j, m.h - 1);
+            const double v = u[y * g.nx + m.x0 + min(2 * lane + i, m.w - 1)];
+            high = max(high, __double2hiint(v));
+            low = min(low, __double2hiint(v));
+            sum += v;
+        }
+    // sums of 8 x 4 points: what some ten steps leave of a field that is only rough
+    sum += __shfl_xor_sync(0xffffffffu, sum, 1);
+    sum += __shfl_xor_sync(0xffffffffu, sum, 2);
+    const int s = __double2hiint(sum);
+    high = __reduce_max_sync(0xffffffffu, high);
+    low = __reduce_min_sync(0xffffffffu, low);
+    const int shigh = __reduce_max_sync(0xffffffffu, s), slow = __reduce_min_sync(0xffffffffu, s);
+    if (lane == 0) {
+        extreme[0][warp] = high;
+        extreme[1][warp] = low;
+        extreme[2][warp] = shigh;
+        extreme[3][warp] = slow;
+    }
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    int e[4] = {extreme[0][0], extreme[1][0], extreme[2][0], extreme[3][0]};
+    for (int w = 1; w < 8; ++w) {
+        e[0] = max(e[0], extreme[0][w]);
+        e[1] = min(e[1], extreme[1][w]);
+        e[2] = max(e[2], extreme[2][w]);
+        e[3] = min(e[3], extreme[3][w]);
+    }
+    FixedHeat f;
+    const unsigned unfit = !f.fits(op.R, e[0], e[1]) && !(soon && f.fits(op.R, e[2], e[3]));
+    // (blocks that have counted in the lower half, unfit tiles in the upper)
+    const unsigned before = atomicAdd(count, (unfit << 16) + 1);
+    if ((before & 0xffff) + 1 < gridDim.x) return;
+    if (5 * ((before >> 16) + unfit) > 3 * gridDim.x)
+        *march_queue = march_items;
+    else
+        *walk_queue = walk_items;
+}
+
+// The walks' shape: the most rows that still give every resident block a tile.
+inline int heat_walk_shape(int nx, int ny) {
+    int shape = 0;
+    while (march_tiles<HeatWalkOp>(shape, &nx, &ny, 1) < 8 * 152 &&
+           shape + 1 < MarchShapes<HeatWalkOp>::kCount)
+        ++shape;
+    return shape;
+}
+
+// Counters of the two forms, with the survey's and the error word's.
+template <class Op>
+inline long long march_words(int shape, int nx, int ny) {
+    long long words = march_tiles<Op>(shape, &nx, &ny, 1) + 2;
+    if constexpr (std::is_same<Op, HeatOp>::value)
+        words += march_tiles<HeatWalkOp>(heat_walk_shape(nx, ny), &nx, &ny, 1) + 2;
+    return words;
+}
+
+// Whether a grid takes either: where the walks are the quicker ones on a field that
+// the integer units cannot take (us a step of mixed-sign noise, HeatMarch / walks:
+// 640 x 640 6.17 / 6.49, 1024 x 512 7.46 / 6.57, 768 x 768 8.17 / 6.77).
+template <class Op>
+inline bool march_either(const double *c, int nx, int ny) {
+    if constexpr (std::is_same<Op, HeatOp>::value)
+        return heat_ratio(c[0]) != 0 && (double)nx * ny >= 5e5 &&
+               march_tiles<HeatWalkOp>(heat_walk_shape(nx, ny), &nx, &ny, 1) *
+                       (kEitherSteps + 1LL) < (1LL << 30);
+    return false;
+}
+
+// As march_advance for one grid.
+inline cudaError_t heat_either_advance(int shape, const MarchGrid &g, const HeatOp &op,
+                                       const HeatWalkOp &walk, const void *src, void *b0, void *b1,
+                                       int *sched, long long steps, int *err,
+                                       long long spin_limit, void **out, long long *launches,
+                                       cudaStream_t st) {
+    const int ws = heat_walk_shape(g.nx, g.ny);
+    const MarchGrid wg = march_cut<HeatWalkOp>(ws, g.nx, g.ny);
+    const int NT = g.bx * g.by, WT = wg.bx * wg.by, K = march_steps<HeatOp>(shape);
+    int *clear = sched;
+    if (!err) err = sched++;
+    int *const walk_sched = sched + NT + 1, *const count = walk_sched + WT + 1;
+    while (steps > 0) {
+        const int n = steps < kEitherSteps ? (int)steps : kEitherSteps;
+        MarchRun<double> run;
+        run.src = (const double *)src;
+        run.buf[0] = (double *)b0;
+        run.buf[1] = (double *)b1;
+        run.err = err;
+        run.first = 0;
+        run.spin_limit = spin_limit;
+        run.done = sched;
+        run.queue = sched + NT;
+        run.NT = NT;
+        run.K = K;
+        run.phases = (n + K - 1) / K;
+        run.last = n - (run.phases - 1) * K;
+        MarchRun<double> walked = run;
+        walked.done = walk_sched;
+        walked.queue = walk_sched + WT;
+        walked.NT = WT;
+        walked.K = 1;
+        walked.phases = n + ((n ^ run.phases) & 1);     // (both end in the same buffer)
+        walked.last = n + 1 - walked.phases;
+        cudaError_t e = cudaMemsetAsync(clear, 0, (count + 1 - clear) * sizeof(int), st);
+        if (e != cudaSuccess) return e;
+        clear = sched;
+        heat_survey_kernel<HeatOp><<<NT < 304 ? NT : 304, 256, 0, st>>>(
+            op, g, run.src, n >= 8, (unsigned *)count, run.queue, NT * run.phases, walked.queue,
+            WT * walked.phases);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        e = with_march_shape<HeatOp>(shape, [&](auto *body) {
+            return march_launch<typename std::remove_pointer<decltype(body)>::type, true>(
+                op, OneMarch{g}, run, st);
+        });
+        if (e != cudaSuccess) return e;
+        e = with_march_shape<HeatWalkOp>(ws, [&](auto *body) {
+            return march_launch<typename std::remove_pointer<decltype(body)>::type, true>(
+                walk, OneMarch{wg}, walked, st);
+        });
+        if (e != cudaSuccess) return e;
+        *launches += 3;
+        steps -= n;
+        src = *out = run.buf[(run.phases - 1) & 1];
+    }
+    return cudaSuccess;
 }
 
 // One phase over NT tiles of an update computed in place.
@@ -1080,6 +1322,10 @@ struct March {
                            void *b0, void *b1, int *sched, long long steps, int *err, int first,
                            long long spin_limit, void **out, long long *launches,
                            cudaStream_t st) {
+        if constexpr (std::is_same<Op, HeatOp>::value)
+            if (first == 0 && march_either<Op>(c, g.nx, g.ny))
+                return heat_either_advance(shape, g, Op(c), HeatWalkOp(c), src, b0, b1, sched,
+                                           steps, err, spin_limit, out, launches, st);
         return march_advance(shape, Op(c), OneMarch{g}, g.bx * g.by, src, b0, b1, sched, steps,
                              err, first, spin_limit, out, launches, st);
     }
@@ -1092,6 +1338,7 @@ struct March {
     }
     static const MarchTable *table() {
         static const MarchTable t = {&march_shape<Op>, &march_steps<Op>, &march_cut<Op>,
+                                     &march_words<Op>,
                                      &march_short<Op>, &naive_shape<Op>, &one, &many,
                                      &phase_one, &phase_many};
         return &t;

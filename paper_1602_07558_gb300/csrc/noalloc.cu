@@ -125,8 +125,8 @@ int advance_static(const double *u_in, double *u_out, int nx, int ny, int tile, 
         if (e != cudaSuccess) set_err(err, errlen, cudaGetErrorString(e));
         return e == cudaSuccess ? SWEPT2D_OK : SWEPT2D_ECUDA;
     }
-    // the scratch holds the second state buffer, the marching form's counters and
-    // an error word; two panel sets hold more than four times the state, so they
+    // the scratch holds the second state buffer, an error word and the marching
+    // form's counters; two panel sets hold more than four times the state, so they
     // fit wherever the check above passed
     const swept::MarchTable *mt = swept::marchtable_heat();
     const int shape = mt->shape(&nx, &ny, nullptr, 1, false);
@@ -156,7 +156,7 @@ int advance_static(const double *u_in, double *u_out, int nx, int ny, int tile, 
     e = mt->one(shape, cut, consts, u_in, b0, b1, sched, nsteps, nullptr,
                             skip ? tiles : 0, spin_limit, &out, &made, st);
     if (e == cudaSuccess)
-        e = swept::launch_after(spoil_if_failed, dim3(152), 256, 0, st, sched + tiles + 1, u_out,
+        e = swept::launch_after(spoil_if_failed, dim3(152), 256, 0, st, sched, u_out,
                                 (size_t)nx * ny);
     if (e != cudaSuccess) {
         char msg[200];

@@ -357,3 +357,41 @@ def test_small_diffusion_numbers_are_bitwise_in_either_mode(oracle_lib, kind, r)
             s.set_state(u0[None])
             s.advance(21, mode=mode)
             assert np.array_equal(s.get_state()[0], ref, equal_nan=True)
+
+
+@pytest.mark.parametrize("kind", ["signed", "crossing", "uniform", "half", "zeros", "nan"])
+@pytest.mark.parametrize("nx,ny,tile,nsteps", [
+    (1024, 512, 32, 7), (768, 768, 32, 8), (768, 768, 32, 9), (1010, 1010, 10, 10),
+    (1022, 504, 14, 11), (712, 720, 8, 264), (1280, 400, 40, 264 + 13)])
+def test_large_fp64_heat_grids_of_every_kind_of_field(oracle_lib, kind, nx, ny, tile, nsteps):
+    """Grids whose form the field decides (integer units or the FP64 walks): step
+    counts of either parity, with a phase that only copies, and over two decisions;
+    in the modes, as a graph, and by the call without a handle."""
+    from paper_1602_07558_gb300.swept2d import SweptError, heat_advance_static
+    rng = np.random.default_rng(nx)
+    u0 = {"signed": lambda: 2 * rng.random((ny, nx)) - 1, "zeros": lambda: np.zeros((ny, nx)),
+          "crossing": lambda: inputs.smooth_field(nx, ny, seed=2),
+          "half": lambda: 1.5 + rng.random((ny, nx)), "uniform": lambda: rng.random((ny, nx)),
+          "nan": lambda: 1.0 + rng.random((ny, nx))}[kind]()
+    if kind == "half":
+        u0[:, :nx // 2] -= 2.0
+    if kind == "nan":
+        u0[5, 6], u0[300, 400] = np.nan, np.inf
+    with np.errstate(all="ignore"):
+        ref = oracle_lib.heat(u0, 0.2, nsteps)
+    with Swept2D(nx, ny, op="heat", tile=tile, params=(0.2,), stream=torch.cuda.Stream()) as s:
+        for mode, graph in (("swept", False), ("swept", True), ("persistent", False)):
+            s.set_state(u0[None])
+            s.advance(nsteps, mode=mode, graph=graph)
+            assert np.array_equal(s.get_state()[0], ref, equal_nan=True)
+    d_in = torch.from_numpy(u0).to("cuda")
+    d_out = torch.zeros_like(d_in)
+    stream = torch.cuda.current_stream()
+    try:
+        heat_advance_static(d_in, d_out, nx, ny, 16 if nx % 16 == 0 and ny % 16 == 0 else tile,
+                            0.2, nsteps, stream=stream)
+    except SweptError as e:                     # (more panels than the scratch holds)
+        assert "scratch" in str(e)
+        return
+    stream.synchronize()
+    assert np.array_equal(d_out.cpu().numpy(), ref, equal_nan=True)
