@@ -415,7 +415,7 @@ int swept2d_batch_create(swept2d_batch_t **out, int count, const int *nx, const 
         b->dt.assign(count, 0.0);
     }
     b->mt = batch_march(op, dtype);
-    if (b->mt) b->mshape = b->mt->shape(nx, ny, tile, count, false);
+    if (b->mt) b->mshape = b->mt->shape(nx, ny, tile, count, false, b->consts);
     if (b->mshape < 0) b->mt = nullptr;
     // grids, classes (by tile side), pooled offsets
     long long soff = 0, poff = 0;

@@ -59,7 +59,7 @@ struct swept2d {
     int mshape = 0;
     swept::MarchGrid mgrid{};
     int *msched = nullptr;
-    // the naive path's launches by its walks (Euler): the grid's shape and cut
+    // the naive path's launches by walks (nullptr: not): the grid's shape and cut
     const swept::MarchTable *nt = nullptr;
     int nshape = 0;
     swept::MarchGrid ngrid{};
@@ -224,20 +224,14 @@ void free_all(swept2d *h) {
 int naive_substeps(swept2d *h, long long count) {
     for (long long s = 0; s < count; ++s) {
         const u64 g = (u64)h->substeps;
-        if (h->nt) {                     // in place
-            int rc = launch(h, SWEPT2D_K_NAIVE, "naive kernel", [&] {
-                return h->nt->phase_one(h->nshape, h->ngrid, h->consts, h->state, (int)(g & 1),
-                                        h->stream);
-            });
-            if (rc) return rc;
-            h->substeps += 1;
-            continue;
-        }
+        const bool in_place = h->nt && h->nst == 2;          // (Euler's walks)
         int rc = launch(h, SWEPT2D_K_NAIVE, "naive kernel", [&] {
-            return h->ops->naive(h->G, h->consts, h->state, h->state2, g, h->stream);
+            return h->nt ? h->nt->phase_one(h->nshape, h->ngrid, h->consts, h->state,
+                                            in_place ? h->state : h->state2, (int)(g & 1), h->stream)
+                         : h->ops->naive(h->G, h->consts, h->state, h->state2, g, h->stream);
         });
         if (rc) return rc;
-        std::swap(h->state, h->state2);
+        if (!in_place) std::swap(h->state, h->state2);
         h->substeps += 1;
     }
     return SWEPT2D_OK;
@@ -482,15 +476,15 @@ int swept2d_create(swept2d_t **out, int nx, int ny, int nvars, int nstages, int 
     }
     h->nt = march_for(op, dtype);
     if (h->nt) {
-        h->nshape = h->nt->naive_shape(nx, ny);
+        h->nshape = h->nt->naive_shape(nx, ny, h->consts);
         if (h->nshape < 0) h->nt = nullptr;
-        else h->ngrid = h->nt->cut(h->nshape, nx, ny);
+        else h->ngrid = h->nt->naive_cut(h->nshape, nx, ny);
     }
     h->mt = tile ? march_for(op, dtype) : nullptr;
     if (h->mt) {
-        h->mshape = h->mt->shape(&nx, &ny, nullptr, 1, false);
+        h->mshape = h->mt->shape(&nx, &ny, nullptr, 1, false, h->consts);
         for (int p = 0; p < 2; ++p)
-            h->marches[p] = h->mt->shape(&nx, &ny, &tile, 1, p != 0) >= 0;
+            h->marches[p] = h->mt->shape(&nx, &ny, &tile, 1, p != 0, h->consts) >= 0;
         if (!h->marches[0] && !h->marches[1] && op != SWEPT2D_OP_EULER_RK2) h->mt = nullptr;
     }
     if (h->mt) {

@@ -131,16 +131,16 @@ march_kernel(Op op, Loc at, MarchRun<typename Op::S> run) {
     }
 }
 
-// One phase of an update computed in place, one tile a block: the naive path's
-// launch per sub-step.
+// One phase, one tile a block: the naive path's launch per sub-step (Euler in place,
+// dst == src).
 template <class Body, class Op, class Loc>
 __global__ void __launch_bounds__(Body::kThreads, Body::kMinBlocks)
-march_phase_kernel(Op op, Loc at, typename Op::S *state, int phase) {
+march_phase_kernel(Op op, Loc at, const typename Op::S *src, typename Op::S *dst, int phase) {
     __shared__ typename Body::Smem sm;
     const MarchTile m = at(blockIdx.x);
     const Op own = m.c ? Op(m.c) : op;
     after_previous_launch();
-    Body::run(own, m, state + m.soff, state + m.soff, Body::K, Body::K, phase, sm);
+    Body::run(own, m, src + m.soff, dst + m.soff, Body::K, Body::K, phase, sm);
 }
 
 // ------------------------------------------------------------------- heat
@@ -933,13 +933,16 @@ inline double euler_swept_cost(const int *nx, const int *ny, const int *tile, in
 //    with the swept kernels when its tiles fill less than 0.78 of their 64 columns
 //    and the grid is too large to be bound by latency (fields with a zero crossing in
 //    every tile, 96 steps, us, swept / marching: 64 x 2048 292 / 437, 192 x 384 241 /
-//    281, but 48 x 512 221 / 181, 256 x 256 241 / 232, 1024 x 1024 1469 / 706).
+//    281, but 48 x 512 221 / 181, 256 x 256 241 / 232, 1024 x 1024 1469 / 706), and so
+//    it does where r keeps it off the integer units altogether (r = 1/4, 100 steps, us:
+//    256² 306 / 290, 512² 413 / 492, 1024² 1122 / 1370, 4096² 13505 / 17470).
 //  - Binary64 Euler, bound by the FP64 pipe in either form: the least of the costs
 //    above (us a step, swept at the tile given / marching: 64 x 2048, 32, 54 / 61;
 //    384 x 384, 32, 54 / 68; 48 x 512, 16, 22 / 27; 128 x 512, 32, 47 / 43; 256 grids
 //    of 32..96 460 / 385, by the largest shape that fills the SMs 450).
 template <class Op>
-inline int march_shape(const int *nx, const int *ny, const int *tile, int count, bool persistent) {
+inline int march_shape(const int *nx, const int *ny, const int *tile, int count, bool persistent,
+                       const double *c) {
     if constexpr (std::is_same<Op, EulerOp>::value) {
         int best = 0;
         double least = 0;
@@ -961,8 +964,17 @@ inline int march_shape(const int *nx, const int *ny, const int *tile, int count,
             points += (double)nx[i] * ny[i];
             columns += 64.0 * march_cut<Op>(shape, nx[i], ny[i]).bx * ny[i];
         }
-        if (points > 28000 && points < 0.78 * columns) return -1;
+        if (points > 28000 && (points < 0.78 * columns || heat_ratio(c[0]) == 0)) return -1;
     }
+    return shape;
+}
+
+// The shape of FP64 heat's walks: the most rows that still give every resident block a tile.
+inline int heat_walk_shape(int nx, int ny) {
+    int shape = 0;
+    while (march_tiles<HeatWalkOp>(shape, &nx, &ny, 1) < 8 * 152 &&
+           shape + 1 < MarchShapes<HeatWalkOp>::kCount)
+        ++shape;
     return shape;
 }
 
@@ -1027,7 +1039,11 @@ inline const WaveCost *naive_costs<EulerKahanOp<__nv_bfloat16>>() {
 }
 
 template <class Op>
-inline int naive_shape(int nx, int ny) {
+inline int naive_shape(int nx, int ny, const double *c) {
+    // FP64 heat: its walks where no warp could take the integer units (r) and the pipe
+    // is the bound (us a step, naive_heat_kernel / walks: 4096² 147 / 136)
+    if constexpr (std::is_same<Op, HeatOp>::value)
+        return heat_ratio(c[0]) == 0 && (double)nx * ny >= 5e5 ? heat_walk_shape(nx, ny) : -1;
     const WaveCost *cost = naive_costs<Op>();
     if (!cost) return -1;
     int best = -1;
@@ -1062,7 +1078,7 @@ inline bool march_short(int shape, int nx, int ny, int tile, long long substeps)
         return substeps <= 3 || (substeps <= 5 && points >= 5e5) || (substeps <= 6 && points >= 2e6);
     } else if constexpr (std::is_same<Op, EulerOp>::value) {
         if (substeps >= tile / 2) return false;
-        const int s = naive_shape<Op>(nx, ny);
+        const int s = naive_shape<Op>(nx, ny, nullptr);
         const WaveCost cost = naive_costs<Op>()[s < 0 ? MarchShapes<Op>::kCount : s];
         const double naive = cost(s < 0 ? ((nx + 31LL) / 32) * ((ny + 7) / 8)
                                         : march_tiles<Op>(s, &nx, &ny, 1));
@@ -1206,15 +1222,6 @@ __global__ void __launch_bounds__(256) heat_survey_kernel(Op op, MarchGrid g, co
         *walk_queue = walk_items;
 }
 
-// The walks' shape: the most rows that still give every resident block a tile.
-inline int heat_walk_shape(int nx, int ny) {
-    int shape = 0;
-    while (march_tiles<HeatWalkOp>(shape, &nx, &ny, 1) < 8 * 152 &&
-           shape + 1 < MarchShapes<HeatWalkOp>::kCount)
-        ++shape;
-    return shape;
-}
-
 // Counters of the two forms, with the survey's and the error word's.
 template <class Op>
 inline long long march_words(int shape, int nx, int ny) {
@@ -1294,15 +1301,16 @@ inline cudaError_t heat_either_advance(int shape, const MarchGrid &g, const Heat
     return cudaSuccess;
 }
 
-// One phase over NT tiles of an update computed in place.
+// One phase of one step over NT tiles.
 template <class Op, class Loc>
-inline cudaError_t march_phase(int shape, const Op &op, const Loc &at, int NT, void *state,
-                               int phase, cudaStream_t st) {
+inline cudaError_t march_phase(int shape, const Op &op, const Loc &at, int NT, const void *src,
+                               void *dst, int phase, cudaStream_t st) {
+    typedef typename Op::S S;
     return with_march_shape<Op>(shape, [&](auto *body) {
         typedef typename std::remove_pointer<decltype(body)>::type B;
-        if constexpr (B::kInPlace)
+        if constexpr (B::K == 1)
             return launch_after(march_phase_kernel<B, Op, Loc>, dim3(NT), B::kThreads, 0, st, op, at,
-                                (typename Op::S *)state, phase);
+                                (const S *)src, (S *)dst, phase);
         else
             return cudaErrorInvalidValue;
     });
@@ -1310,13 +1318,22 @@ inline cudaError_t march_phase(int shape, const Op &op, const Loc &at, int NT, v
 
 template <class Op>
 struct March {
-    static cudaError_t phase_one(int shape, const MarchGrid &g, const double *c, void *state,
-                                 int phase, cudaStream_t st) {
-        return march_phase(shape, Op(c), OneMarch{g}, g.bx * g.by, state, phase, st);
+    static MarchGrid naive_cut(int shape, int nx, int ny) {
+        if constexpr (std::is_same<Op, HeatOp>::value)
+            return march_cut<HeatWalkOp>(shape, nx, ny);
+        else
+            return march_cut<Op>(shape, nx, ny);
+    }
+    static cudaError_t phase_one(int shape, const MarchGrid &g, const double *c, const void *src,
+                                 void *dst, int phase, cudaStream_t st) {
+        if constexpr (std::is_same<Op, HeatOp>::value)      // (by its walks)
+            return march_phase(shape, HeatWalkOp(c), OneMarch{g}, g.bx * g.by, src, dst, phase, st);
+        else
+            return march_phase(shape, Op(c), OneMarch{g}, g.bx * g.by, src, dst, phase, st);
     }
     static cudaError_t phase_many(int shape, const GridDesc *grids, const int2 *tiles, int NT,
                                   const double *c, void *state, int phase, cudaStream_t st) {
-        return march_phase(shape, Op(c), ManyMarch{grids, tiles}, NT, state, phase, st);
+        return march_phase(shape, Op(c), ManyMarch{grids, tiles}, NT, state, state, phase, st);
     }
     static cudaError_t one(int shape, const MarchGrid &g, const double *c, const void *src,
                            void *b0, void *b1, int *sched, long long steps, int *err, int first,
@@ -1340,7 +1357,7 @@ struct March {
         static const MarchTable t = {&march_shape<Op>, &march_steps<Op>, &march_cut<Op>,
                                      &march_words<Op>,
                                      &march_short<Op>, &naive_shape<Op>, &one, &many,
-                                     &phase_one, &phase_many};
+                                     &naive_cut, &phase_one, &phase_many};
         return &t;
     }
 };

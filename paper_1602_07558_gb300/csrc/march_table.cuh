@@ -8,8 +8,9 @@ namespace swept {
 struct MarchTable {
     // the shape for these grids; -1 where the swept kernels with these tile sides, in
     // the launch-per-phase or the persistent form, do better (without tile sides, a
-    // shape in any case)
-    int (*shape)(const int *nx, const int *ny, const int *tile, int count, bool persistent);
+    // shape in any case); c: the update's constants (heat's r)
+    int (*shape)(const int *nx, const int *ny, const int *tile, int count, bool persistent,
+                 const double *c);
     int (*steps)(int shape);     // steps a phase
     MarchGrid (*cut)(int shape, int nx, int ny);
     // ints of the counters that `one` needs, its own error word included
@@ -18,7 +19,7 @@ struct MarchTable {
     bool (*is_short)(int shape, int nx, int ny, int tile, long long substeps);
     // the shape whose walks (phase_one) are the quickest for the naive sub-steps of
     // one grid, -1 for a thread a point
-    int (*naive_shape)(int nx, int ny);
+    int (*naive_shape)(int nx, int ny, const double *c);
     // one grid (`g` its cut), or the tiles of a batch's table; without `err`, the
     // error word is the first of the counters' words
     cudaError_t (*one)(int shape, const MarchGrid &g, const double *c, const void *src, void *b0,
@@ -27,9 +28,11 @@ struct MarchTable {
     cudaError_t (*many)(int shape, const GridDesc *grids, const int2 *tiles, int NT,
                         const double *c, const void *src, void *b0, void *b1, int *sched,
                         long long steps, int *err, void **out, long long *launches, cudaStream_t);
-    // one sub-step in place (Euler), as one launch: the naive path
-    cudaError_t (*phase_one)(int shape, const MarchGrid &g, const double *c, void *state, int phase,
-                             cudaStream_t);
+    // one sub-step by walks as one launch, the naive path: `g` the grid's naive_cut;
+    // Euler in place (dst == src)
+    MarchGrid (*naive_cut)(int shape, int nx, int ny);
+    cudaError_t (*phase_one)(int shape, const MarchGrid &g, const double *c, const void *src,
+                             void *dst, int phase, cudaStream_t);
     cudaError_t (*phase_many)(int shape, const GridDesc *grids, const int2 *tiles, int NT,
                               const double *c, void *state, int phase, cudaStream_t);
 };

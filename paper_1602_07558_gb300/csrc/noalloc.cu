@@ -9,11 +9,13 @@
 // other device memory this path touches is the file-scope array below, which
 // the CUDA runtime sets up when it loads this library's device code.
 //
-// The marching form of swept2d_advance (march.cuh) on the caller's buffers, so
-// the result is bit for bit that of a handle created with op SWEPT2D_OP_HEAT and
+// The marching form of swept2d_advance (march.cuh) on the caller's buffers, or, where
+// the diffusion number keeps that off the integer units, the swept kernels (Up, then
+// per half cycle the x/y Bridge launch and the Octahedron, a final Down, naive tail),
+// so the result is bit for bit that of a handle created with op SWEPT2D_OP_HEAT and
 // advanced with SWEPT2D_SWEPT from the same input. The call has returned before a
-// wait of that form could give up, and its caller has no handle to ask: a last
-// kernel then overwrites u_out with NaN.
+// wait of the marching form could give up, and its caller has no handle to ask: a
+// last kernel then overwrites u_out with NaN.
 #include <cuda_runtime.h>
 
 #include <cstdio>
@@ -28,7 +30,8 @@ namespace {
 constexpr size_t kScratchBytes = SWEPT2D_STATIC_SCRATCH_BYTES;
 
 // Shared by every call on a device and kept until the process exits. Holds the
-// second state buffer and the counters of the marching form. Nothing in it has
+// second state buffer and the counters of the marching form, or the swept kernels'
+// panels. Nothing in it has
 // to start at zero: every element a call reads was written earlier in that same
 // call.
 static __device__ __align__(256) unsigned char g_scratch[kScratchBytes];
@@ -66,6 +69,38 @@ __global__ void __launch_bounds__(256) spoil_if_failed(const int *err, double *u
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n;
          i += (size_t)gridDim.x * blockDim.x)
         u[i] = __longlong_as_double(0x7ff8000000000000LL);
+}
+
+// The swept schedule on the caller's buffers and two panel sets, then the tail, whose
+// last sub-step lands in u_out (`tmp`: one state copy, where there is a tail).
+cudaError_t advance_swept(const swept::Geom &G, const double *consts, const double *u_in,
+                          double *u_out, void *up, void *br, double *tmp, long long nsteps,
+                          cudaStream_t st) {
+    const swept::OpTable *t = swept::optable_heat();
+    const swept::Tuning tn;   // 256 threads, per-level prefetch (the handle path's heat default)
+    const int half = G.n / 2;
+    const long long H = nsteps / half, rem = nsteps - H * half;
+    const double *src = u_in;
+    cudaError_t e = cudaSuccess;
+    if (H > 0) {
+        double *to = rem % 2 == 1 ? tmp : u_out;
+        e = t->up(G, consts, u_in, up, 0, 0, st);
+        for (long long j = 0; j < H && e == cudaSuccess; ++j) {
+            const u64 g0 = (u64)j * half;
+            const int o = (j & 1) ? half : 0;
+            e = t->bridge(G, consts, up, br, g0, nullptr, tn, st);
+            if (e == cudaSuccess)
+                e = j + 1 < H ? t->octahedron(G, consts, br, up, o, g0, nullptr, tn, st)
+                              : t->down(G, consts, br, to, o, g0, nullptr, tn, st);
+        }
+        src = to;
+    }
+    for (long long i = 0; i < rem && e == cudaSuccess; ++i) {
+        double *to = (rem - 1 - i) % 2 == 0 ? u_out : tmp;
+        e = t->naive(G, consts, src, to, (u64)(H * half + i), st);
+        src = to;
+    }
+    return e;
 }
 
 // The advance; `skip` (the wait-timeout self-test): its first phase is skipped.
@@ -129,12 +164,20 @@ int advance_static(const double *u_in, double *u_out, int nx, int ny, int tile, 
     // form's counters; two panel sets hold more than four times the state, so they
     // fit wherever the check above passed
     const swept::MarchTable *mt = swept::marchtable_heat();
-    const int shape = mt->shape(&nx, &ny, nullptr, 1, false);
+    const double consts[8] = {r, 0, 0, 0, 0, 0, 0, 0};
+    const int shape = mt->shape(&nx, &ny, nullptr, 1, false, consts);
     const swept::MarchGrid cut = mt->cut(shape, nx, ny);
     const int tiles = cut.bx * cut.by;
     void *tmp = base;
-    const double consts[8] = {r, 0, 0, 0, 0, 0, 0, 0};
     cudaError_t e = cudaSuccess;
+    if (!skip && swept::heat_ratio(r) == 0 &&
+        mt->shape(&nx, &ny, &tile, 1, false, consts) < 0) {
+        char *const sb = (char *)base;
+        e = advance_swept(G, consts, u_in, u_out, sb, sb + align256(panel_bytes),
+                          (double *)(sb + 2 * align256(panel_bytes)), nsteps, st);
+        if (e != cudaSuccess) set_err(err, errlen, cudaGetErrorString(e));
+        return e == cudaSuccess ? SWEPT2D_OK : SWEPT2D_ECUDA;
+    }
     if (!skip && mt->is_short(shape, nx, ny, tile, nsteps)) {
         // naive launches, the last of which lands in u_out
         const void *src = u_in;
@@ -154,7 +197,7 @@ int advance_static(const double *u_in, double *u_out, int nx, int ny, int tile, 
     void *out = nullptr;
     long long made = 0;
     e = mt->one(shape, cut, consts, u_in, b0, b1, sched, nsteps, nullptr,
-                            skip ? tiles : 0, spin_limit, &out, &made, st);
+                skip ? tiles : 0, spin_limit, &out, &made, st);
     if (e == cudaSuccess)
         e = swept::launch_after(spoil_if_failed, dim3(152), 256, 0, st, sched, u_out,
                                 (size_t)nx * ny);

@@ -395,3 +395,45 @@ def test_large_fp64_heat_grids_of_every_kind_of_field(oracle_lib, kind, nx, ny, 
         return
     stream.synchronize()
     assert np.array_equal(d_out.cpu().numpy(), ref, equal_nan=True)
+
+
+@pytest.mark.parametrize("r", [0.25, 0.3, -0.05, 2.0 ** -12])
+@pytest.mark.parametrize("nx,ny,tile,nsteps", [
+    (64, 48, 16, 21), (192, 384, 32, 37), (192, 384, 32, 16), (512, 512, 32, 34), (512, 512, 32, 33),
+    (704, 720, 16, 19), (1000, 760, 40, 45)])
+def test_diffusion_numbers_the_integer_units_cannot_take(oracle_lib, r, nx, ny, tile, nsteps):
+    """The swept kernels (marching on small grids) and the naive walks, with tails of
+    either parity, in every mode and by the call without a handle."""
+    from paper_1602_07558_gb300.swept2d import heat_advance_static
+    u0 = 2 * np.random.default_rng(nx).random((ny, nx)) - 1
+    with np.errstate(all="ignore"):
+        ref = oracle_lib.heat(u0, r, nsteps)
+    with Swept2D(nx, ny, op="heat", tile=tile, params=(r,), stream=torch.cuda.Stream()) as s:
+        for mode, graph in (("swept", False), ("swept", True), ("persistent", False),
+                            ("naive", False), ("naive", True)):
+            s.set_state(u0[None])
+            s.advance(nsteps, mode=mode, graph=graph)
+            assert np.array_equal(s.get_state()[0], ref)
+    d_in = torch.from_numpy(u0).to("cuda")
+    d_out = torch.zeros_like(d_in)
+    heat_advance_static(d_in, d_out, nx, ny, tile, r, nsteps, stream=torch.cuda.current_stream())
+    torch.cuda.synchronize()
+    assert np.array_equal(d_out.cpu().numpy(), ref) and np.array_equal(d_in.cpu().numpy(), u0)
+
+
+@pytest.mark.parametrize("nx,ny,tile,nsteps", [(64, 2048, 32, 37), (64, 2048, 16, 20), (192, 384, 32, 53),
+                                               (192, 384, 16, 25)])
+@pytest.mark.parametrize("mode,graph", [("swept", False), ("swept", True), ("persistent", False)])
+def test_fp64_heat_grids_that_keep_the_swept_kernels(oracle_lib, nx, ny, tile, nsteps, mode, graph):
+    """Grids too narrow for the marching form's columns: the Up, Bridge, Octahedron and
+    Down launches without a gap between them, with odd tails, twice in a row."""
+    u0 = inputs.smooth_field(nx, ny, seed=3)
+    ref = oracle_lib.heat(u0, 0.2, 2 * nsteps)
+    with Swept2D(nx, ny, op="heat", tile=tile, params=(0.2,), stream=torch.cuda.Stream()) as s:
+        s.set_timing(not graph)
+        s.set_state(u0[None])
+        s.advance(nsteps, mode=mode, graph=graph)
+        s.advance(nsteps, mode=mode, graph=graph)
+        assert np.array_equal(s.get_state()[0], ref)
+        if not graph:
+            assert s.kernel_stats("octahedron")[0] > 0 and s.kernel_stats("march")[0] == 0
