@@ -16,7 +16,8 @@ struct Tuning {
     bool stage = false;
 };
 
-// Function table of one point update (filled in by an instantiation unit).
+// Function table of one point update (filled in by an instantiation unit). The
+// launches per phase are null for an update whose swept mode always marches.
 struct OpTable {
     int nv, nst, esize;
     size_t (*smem_bytes)(int n);   // largest dynamic shared memory of a swept block, tile n
@@ -241,6 +242,15 @@ struct Launch {
         static const OpTable t = {Op::NV,      Op::NST,     (int)sizeof(S), &swept_smem_bytes<Op>,
                                   &naive,      &up,         &bridge,        &octahedron,
                                   &down,       Op::STAGE,   &swept_smem_for<Op>, &persistent,
+                                  SweptBounds<Op>::kThreads, kMaxPersistentThreads};
+        return &t;
+    }
+    // an update whose swept mode always marches (march.cuh): the naive launches, and
+    // the persistent form for its trace
+    static const OpTable *marching_table() {
+        static const OpTable t = {Op::NV,      Op::NST,     (int)sizeof(S), &swept_smem_bytes<Op>,
+                                  &naive,      nullptr,     nullptr,        nullptr,
+                                  nullptr,     Op::STAGE,   &swept_smem_for<Op>, &persistent,
                                   SweptBounds<Op>::kThreads, kMaxPersistentThreads};
         return &t;
     }

@@ -437,3 +437,34 @@ def test_fp64_heat_grids_that_keep_the_swept_kernels(oracle_lib, nx, ny, tile, n
         assert np.array_equal(s.get_state()[0], ref)
         if not graph:
             assert s.kernel_stats("octahedron")[0] > 0 and s.kernel_stats("march")[0] == 0
+
+
+@pytest.mark.parametrize("threads,stage", [(256, False), (128, True)])
+@pytest.mark.parametrize("op,dtype,tile", [("heat_kahan", "f32", 16), ("heat_kahan", "bf16", 32),
+                                           ("euler_kahan", "f32", 16), ("euler_kahan", "bf16", 8)])
+def test_traced_persistent_advance_of_the_updates_that_march(oracle_lib, op, dtype, tile, threads, stage):
+    """A trace records the persistent swept kernel's items, which nothing else runs for
+    these updates: same bits as the marching advance, every item timed."""
+    nx, ny, steps = 96, 64, 21
+    if op == "heat_kahan":
+        u, params, nst = 1.0 + np.random.default_rng(2).random((1, ny, nx)), (0.2,), 1
+        u0 = np.concatenate([u, np.zeros_like(u)]).astype(np.float32)
+    else:
+        U, params, nst = inputs.euler_pulse(nx, ny, 4, gamma=1.4), (1.4, 0.3, 0.5), 2
+        u0 = np.concatenate([U, U, np.zeros_like(U)]).astype(np.float32)
+    if dtype == "bf16":
+        u0 = torch.from_numpy(u0).to(torch.bfloat16).view(torch.int16).numpy().view(np.uint16)
+    tiles, halves = (nx // tile) * (ny // tile), steps * nst // (tile // 2)
+    buf = torch.zeros(2 * tiles * (1 + 3 * halves), dtype=torch.int32, device="cuda")
+    with Swept2D(nx, ny, op=op, tile=tile, params=params, dtype=dtype,
+                 stream=torch.cuda.Stream()) as s:
+        s.set_state(u0)
+        s.advance(steps, mode="persistent")
+        want = s.get_state()
+        s.set_tuning(threads, stage)
+        s.set_trace(buf)
+        for graph in (False, True):
+            s.set_state(u0)
+            s.advance(steps, mode="persistent", graph=graph)
+            assert np.array_equal(s.get_state(), want)
+    assert (buf.cpu().numpy().view(np.uint32).reshape(-1, 2)[:, 1] > 0).all()
