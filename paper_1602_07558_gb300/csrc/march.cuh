@@ -102,14 +102,12 @@ __device__ __forceinline__ bool march_wait(const MarchTile &m, const int *done, 
     return __syncthreads_or(bad) == 0;
 }
 
-// AFTER: launched without a gap to the launch before (launch_after).
-template <class Body, class Op, class Loc, bool AFTER>
-__global__ void __launch_bounds__(Body::kThreads, Body::kMinBlocks)
-march_kernel(Op op, Loc at, MarchRun<typename Op::S> run) {
+// The items of a run, taken until none is left (or a wait gave up).
+template <class Body, class Op, class Loc>
+__device__ __forceinline__ void march_items(const Op &op, const Loc &at,
+                                            const MarchRun<typename Op::S> &run,
+                                            typename Body::Smem &sm, int &s_item) {
     typedef typename Op::S S;
-    __shared__ typename Body::Smem sm;
-    __shared__ int s_item;
-    if constexpr (AFTER) after_previous_launch();
     const int nitems = run.NT * run.phases;
     for (;;) {
         if (threadIdx.x == 0) {
@@ -129,6 +127,36 @@ march_kernel(Op op, Loc at, MarchRun<typename Op::S> run) {
         __syncthreads();
         if (threadIdx.x == 0) add_release(run.done + t, 1);
     }
+}
+
+// AFTER: launched without a gap to the launch before (launch_after).
+template <class Body, class Op, class Loc, bool AFTER>
+__global__ void __launch_bounds__(Body::kThreads, Body::kMinBlocks)
+march_kernel(Op op, Loc at, MarchRun<typename Op::S> run) {
+    __shared__ typename Body::Smem sm;
+    __shared__ int s_item;
+    if constexpr (AFTER) after_previous_launch();
+    march_items<Body>(op, at, run, sm, s_item);
+}
+
+// The same for a caller that cannot ask for the error word: the block that leaves
+// last overwrites the result, `points` values, with NaN if a wait gave up.
+template <class Body, class Op, class Loc, bool AFTER>
+__global__ void __launch_bounds__(Body::kThreads, Body::kMinBlocks)
+march_or_spoil_kernel(Op op, Loc at, MarchRun<double> run, unsigned *left, size_t points) {
+    __shared__ typename Body::Smem sm;
+    __shared__ int s_item;
+    if constexpr (AFTER) after_previous_launch();
+    march_items<Body>(op, at, run, sm, s_item);
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0)
+        s_item = atomicAdd(left, 1u) + 1 == gridDim.x && ld_acquire(run.err) != 0;
+    __syncthreads();
+    if (!s_item) return;
+    double *u = run.buf[(run.phases - 1) & 1];
+    for (size_t i = threadIdx.x; i < points; i += Body::kThreads)
+        u[i] = __longlong_as_double(0x7ff8000000000000LL);
 }
 
 // One phase, one tile a block: the naive path's launch per sub-step (Euler in place,
@@ -396,7 +424,10 @@ struct HeatMarch {
                 low = min(low, sm.low[w]);
             }
             FixedCell fixed;
-            if (fixed.f.fits(op.R, high, low)) {
+            // (with one row a thread, which latency bounds, the ratio formed here is 2-5%
+            // quicker than the kernel's parameter: 1770 x 30 3.42 / 3.58 ms; otherwise 1-5%
+            // slower: 768² 576 / 623 us)
+            if (fixed.f.fits(R == 1 ? heat_ratio(op.r) : op.R, high, low)) {
                 L2 v[R], none[1];
 #pragma unroll
                 for (int j = 0; j < R; ++j) v[j] = two(fixed.f.from(u[j].l), fixed.f.from(u[j].h));
@@ -1088,34 +1119,42 @@ inline bool march_short(int shape, int nx, int ny, int tile, long long substeps)
     }
 }
 
-// One launch of a run whose counters are set.
+// One launch of a run whose counters are set; with `left` (a zero), the result is
+// spoiled where a wait gives up.
 template <class B, bool AFTER, class Op, class Loc>
 inline cudaError_t march_launch(const Op &op, const Loc &at, const MarchRun<typename Op::S> &run,
-                                cudaStream_t st) {
-    const auto kern = march_kernel<B, Op, Loc, AFTER>;
-    int per_sm = 0, dev = 0, nsm = 0;
-    const cudaError_t e =
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, B::kThreads, 0);
-    if (e != cudaSuccess) return e;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    long long grid = (long long)(per_sm > 0 ? per_sm : 1) * nsm;
-    if (grid > 2LL * run.NT) grid = 2LL * run.NT;
-    if (grid > (long long)run.NT * run.phases) grid = (long long)run.NT * run.phases;
-    if constexpr (AFTER) return launch_after(kern, dim3((unsigned)grid), B::kThreads, 0, st, op, at, run);
-    kern<<<(int)grid, B::kThreads, 0, st>>>(op, at, run);
-    return cudaGetLastError();
+                                unsigned *left, size_t points, cudaStream_t st) {
+    const auto launch = [&](auto *kern, auto... more) {
+        int per_sm = 0, dev = 0, nsm = 0;
+        const cudaError_t e =
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, B::kThreads, 0);
+        if (e != cudaSuccess) return e;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+        long long grid = (long long)(per_sm > 0 ? per_sm : 1) * nsm;
+        if (grid > 2LL * run.NT) grid = 2LL * run.NT;
+        if (grid > (long long)run.NT * run.phases) grid = (long long)run.NT * run.phases;
+        if constexpr (AFTER)
+            return launch_after(kern, dim3((unsigned)grid), B::kThreads, 0, st, op, at, run, more...);
+        kern<<<(int)grid, B::kThreads, 0, st>>>(op, at, run, more...);
+        return cudaGetLastError();
+    };
+    if constexpr (std::is_base_of<HeatOp, Op>::value && std::is_same<Loc, OneMarch>::value)
+        if (left) return launch(&march_or_spoil_kernel<B, Op, Loc, AFTER>, left, points);
+    return launch(&march_kernel<B, Op, Loc, AFTER>);
 }
 
 // Queues `steps` steps over NT tiles: reads `src`, writes b0, b1, b0, ... phase
 // by phase (src may be b1). sched: NT counters and the item counter; without `err`
-// the word before them is the error word and is cleared with them. `launches` is
-// raised by the launches made, `*out` set to the buffer with the result.
+// (one heat grid) two words more precede them, the error word and a count, both
+// cleared with them, and a result of `points` values becomes NaN where a wait gives
+// up. `launches` is raised by the launches made, `*out` set to the buffer with the
+// result.
 template <class Op, class Loc>
 inline cudaError_t march_advance(int shape, const Op &op, const Loc &at, int NT, const void *src,
                                  void *b0, void *b1, int *sched, long long steps, int *err,
                                  int first, long long spin_limit, void **out, long long *launches,
-                                 cudaStream_t st) {
+                                 cudaStream_t st, size_t points = 0) {
     typedef typename Op::S S;
     return with_march_shape<Op>(shape, [&](auto *body) {
         typedef typename std::remove_pointer<decltype(body)>::type B;
@@ -1125,7 +1164,12 @@ inline cudaError_t march_advance(int shape, const Op &op, const Loc &at, int NT,
         // (an even number of phases: the stages of Euler alternate)
         const long long most = (((1LL << 30) - 1) / NT + 2) & ~1LL;
         int *clear = sched;
-        if (!err) err = sched++;
+        unsigned *blocks_left = nullptr;
+        if (!err) {
+            err = sched;
+            blocks_left = (unsigned *)sched + 1;
+            sched += 2;
+        }
         while (steps > 0) {
             const long long left = (steps + K - 1) / K;
             MarchRun<S> run;
@@ -1143,8 +1187,9 @@ inline cudaError_t march_advance(int shape, const Op &op, const Loc &at, int NT,
             run.spin_limit = spin_limit;
             cudaError_t e = cudaMemsetAsync(clear, 0, (sched + NT + 1 - clear) * sizeof(int), st);
             if (e != cudaSuccess) return e;
-            clear = sched;
-            if ((e = march_launch<B, false>(op, at, run, st)) != cudaSuccess) return e;
+            clear = blocks_left ? sched - 1 : sched;
+            if ((e = march_launch<B, false>(op, at, run, blocks_left, points, st)) != cudaSuccess)
+                return e;
             *launches += 1;
             steps -= (long long)(run.phases - 1) * K + run.last;
             *out = run.buf[(run.phases - 1) & 1];
@@ -1225,7 +1270,7 @@ __global__ void __launch_bounds__(256) heat_survey_kernel(Op op, MarchGrid g, co
 // Counters of the two forms, with the survey's and the error word's.
 template <class Op>
 inline long long march_words(int shape, int nx, int ny) {
-    long long words = march_tiles<Op>(shape, &nx, &ny, 1) + 2;
+    long long words = march_tiles<Op>(shape, &nx, &ny, 1) + 3;
     if constexpr (std::is_same<Op, HeatOp>::value)
         words += march_tiles<HeatWalkOp>(heat_walk_shape(nx, ny), &nx, &ny, 1) + 2;
     return words;
@@ -1253,7 +1298,12 @@ inline cudaError_t heat_either_advance(int shape, const MarchGrid &g, const Heat
     const MarchGrid wg = march_cut<HeatWalkOp>(ws, g.nx, g.ny);
     const int NT = g.bx * g.by, WT = wg.bx * wg.by, K = march_steps<HeatOp>(shape);
     int *clear = sched;
-    if (!err) err = sched++;
+    unsigned *blocks_left = nullptr;
+    if (!err) {
+        err = sched;
+        blocks_left = (unsigned *)sched + 1;
+        sched += 2;
+    }
     int *const walk_sched = sched + NT + 1, *const count = walk_sched + WT + 1;
     while (steps > 0) {
         const int n = steps < kEitherSteps ? (int)steps : kEitherSteps;
@@ -1279,19 +1329,19 @@ inline cudaError_t heat_either_advance(int shape, const MarchGrid &g, const Heat
         walked.last = n + 1 - walked.phases;
         cudaError_t e = cudaMemsetAsync(clear, 0, (count + 1 - clear) * sizeof(int), st);
         if (e != cudaSuccess) return e;
-        clear = sched;
+        clear = blocks_left ? sched - 1 : sched;
         heat_survey_kernel<HeatOp><<<NT < 304 ? NT : 304, 256, 0, st>>>(
             op, g, run.src, n >= 8, (unsigned *)count, run.queue, NT * run.phases, walked.queue,
             WT * walked.phases);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         e = with_march_shape<HeatOp>(shape, [&](auto *body) {
             return march_launch<typename std::remove_pointer<decltype(body)>::type, true>(
-                op, OneMarch{g}, run, st);
+                op, OneMarch{g}, run, nullptr, 0, st);
         });
         if (e != cudaSuccess) return e;
         e = with_march_shape<HeatWalkOp>(ws, [&](auto *body) {
             return march_launch<typename std::remove_pointer<decltype(body)>::type, true>(
-                walk, OneMarch{wg}, walked, st);
+                walk, OneMarch{wg}, walked, blocks_left, (size_t)g.nx * g.ny, st);
         });
         if (e != cudaSuccess) return e;
         *launches += 3;
@@ -1344,7 +1394,7 @@ struct March {
                 return heat_either_advance(shape, g, Op(c), HeatWalkOp(c), src, b0, b1, sched,
                                            steps, err, spin_limit, out, launches, st);
         return march_advance(shape, Op(c), OneMarch{g}, g.bx * g.by, src, b0, b1, sched, steps,
-                             err, first, spin_limit, out, launches, st);
+                             err, first, spin_limit, out, launches, st, (size_t)g.nx * g.ny);
     }
     static cudaError_t many(int shape, const GridDesc *grids, const int2 *tiles, int NT,
                             const double *c, const void *src, void *b0, void *b1, int *sched,

@@ -13,15 +13,15 @@ struct MarchTable {
                  const double *c);
     int (*steps)(int shape);     // steps a phase
     MarchGrid (*cut)(int shape, int nx, int ny);
-    // ints of the counters that `one` needs, its own error word included
+    // ints of the counters that `one` needs, its own error words included
     long long (*words)(int shape, int nx, int ny);
     // whether an advance of so few sub-steps of one grid is quicker by naive launches
     bool (*is_short)(int shape, int nx, int ny, int tile, long long substeps);
     // the shape whose walks (phase_one) are the quickest for the naive sub-steps of
     // one grid, -1 for a thread a point
     int (*naive_shape)(int nx, int ny, const double *c);
-    // one grid (`g` its cut), or the tiles of a batch's table; without `err`, the
-    // error word is the first of the counters' words
+    // one grid (`g` its cut), or the tiles of a batch's table; without `err` (heat
+    // alone) the result becomes NaN where a wait gives up
     cudaError_t (*one)(int shape, const MarchGrid &g, const double *c, const void *src, void *b0,
                        void *b1, int *sched, long long steps, int *err, int first,
                        long long spin_limit, void **out, long long *launches, cudaStream_t);

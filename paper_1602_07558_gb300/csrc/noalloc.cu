@@ -14,8 +14,8 @@
 // per half cycle the x/y Bridge launch and the Octahedron, a final Down, naive tail),
 // so the result is bit for bit that of a handle created with op SWEPT2D_OP_HEAT and
 // advanced with SWEPT2D_SWEPT from the same input. The call has returned before a
-// wait of the marching form could give up, and its caller has no handle to ask: a
-// last kernel then overwrites u_out with NaN.
+// wait of the marching form could give up, and its caller has no handle to ask: the
+// last block to leave then overwrites u_out with NaN.
 #include <cuda_runtime.h>
 
 #include <cstdio>
@@ -60,15 +60,6 @@ int scratch_address(void **out, char *err, int errlen) {
     }
     *out = p;
     return SWEPT2D_OK;
-}
-
-// u = NaN everywhere if the launch before this one recorded a failure.
-__global__ void __launch_bounds__(256) spoil_if_failed(const int *err, double *u, size_t n) {
-    swept::after_previous_launch();
-    if (*err == 0) return;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n;
-         i += (size_t)gridDim.x * blockDim.x)
-        u[i] = __longlong_as_double(0x7ff8000000000000LL);
 }
 
 // The swept schedule on the caller's buffers and two panel sets, then the tail, whose
@@ -198,9 +189,6 @@ int advance_static(const double *u_in, double *u_out, int nx, int ny, int tile, 
     long long made = 0;
     e = mt->one(shape, cut, consts, u_in, b0, b1, sched, nsteps, nullptr,
                 skip ? tiles : 0, spin_limit, &out, &made, st);
-    if (e == cudaSuccess)
-        e = swept::launch_after(spoil_if_failed, dim3(152), 256, 0, st, sched, u_out,
-                                (size_t)nx * ny);
     if (e != cudaSuccess) {
         char msg[200];
         snprintf(msg, sizeof msg, "marching kernel: %s", cudaGetErrorString(e));
