@@ -1098,7 +1098,9 @@ inline int naive_shape(int nx, int ny, const double *c) {
 //     371; 4096 x 4096, 6: 510 / 514 (mixed signs 836 / 1090)
 //   heat binary32: 256 x 256, 1 step 5.4 / 10.3, 2: 9.8 / 9.9, 3: 14.4 / 9.8; 2048 x 2048, 1:
 //     15.9 / 33, 2: 28 / 33, 3: 41 / 33
-//   Euler binary32: 256 x 256, 1 step 11.9 / 15.8, 2: 20.3 / 22.2, 3: 28.6 / 28.8
+//   Euler binary32: 256 x 256, 1 step 11.9 / 15.8, 2: 20.3 / 22.2, 3: 28.6 / 28.8; in a
+//     graph every step of what fills no half cycle: 512 x 512 8.1 / 9.9, 128 x 2048 9.8 /
+//     12.5, 1024 x 1024 19.6 / 20.8, 2048 x 2048 98.2 / 96.2
 //   Euler binary64 (by both forms' costs; never more than the caller's half cycle, which
 //     the swept form would not fill either): 80 x 320, 3 steps 76 / 104; 384 x 192, 3: 126 /
 //     147; 64 x 64, 1: 24 / 21
@@ -1114,8 +1116,10 @@ inline bool march_short(int shape, int nx, int ny, int tile, long long substeps)
         const double naive = cost(s < 0 ? ((nx + 31LL) / 32) * ((ny + 7) / 8)
                                         : march_tiles<Op>(s, &nx, &ny, 1));
         return 0.5 * (double)substeps * (naive - euler_march_cost(shape, &nx, &ny, 1)) < 6;
+    } else if constexpr (Op::NST == 2) {
+        return substeps <= 4 || substeps < tile / 2;
     } else {
-        return substeps <= 2 * Op::NST;
+        return substeps <= 2;
     }
 }
 

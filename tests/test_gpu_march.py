@@ -315,7 +315,8 @@ def test_binary64_euler_gives_the_same_bits_in_either_form(oracle_lib, nx, ny, t
 @pytest.mark.parametrize("op,dtype,nx,ny,tile", [
     ("heat", "f64", 64, 48, 16), ("heat", "f64", 2048, 1024, 64), ("heat_kahan", "f32", 64, 48, 16),
     ("heat_kahan", "bf16", 64, 48, 16), ("euler_rk2", "f64", 80, 320, 40),
-    ("euler_kahan", "f32", 64, 48, 16), ("euler_kahan", "bf16", 64, 48, 16)])
+    ("euler_kahan", "f32", 64, 48, 16), ("euler_kahan", "bf16", 64, 48, 16),
+    ("euler_kahan", "bf16", 64, 1664, 32)])
 def test_short_advances_take_naive_launches_with_the_same_bits(op, dtype, nx, ny, tile):
     """Up to a few sub-steps an advance in a swept mode is one naive launch each; every
     split of eight steps, by stream and by graph, ends in the same state."""
