@@ -19,6 +19,9 @@ alone depends on n, so the model favours large tiles and the measured table
 Steps per stage are n/2 for tile n (the swept rule advances each tile n/2
 sub-steps between exchanges), so choosing the tile chooses them.
 All candidates give bitwise the same result, so the choice is purely about speed.
+Where an advance takes the marching form, which ignores tile and launch shape, there
+is nothing to time but its one form: a tile that marches is timed once, with the
+default launch shape, and among tiles that all march the largest is taken.
 """
 from __future__ import annotations
 
@@ -61,16 +64,22 @@ def _time_advance(s, state, steps, stream):
     ms = None
     for rep in range(2):
         with torch.cuda.stream(stream):
-            if state is not None:
-                s.set_state(state)
-            else:
-                s.set_state(torch.zeros(s.shape, device="cuda", dtype=_torch_dtype(s.np_dtype)))
+            s.set_state(state)
             ev0.record(stream)
             s.advance(steps)
             ev1.record(stream)
         ev1.synchronize()
         ms = ev0.elapsed_time(ev1)
     return ms
+
+
+def _marches(s, steps):
+    """Whether the handle's swept mode takes the marching form for `steps` steps."""
+    s.set_timing(True)
+    s.advance(steps)
+    marched = s.kernel_stats("march")[0] > 0
+    s.set_timing(False)
+    return marched
 
 
 def autotune(nx, ny, op, params, dtype=None, state=None, stream=None, probe_steps=None,
@@ -107,6 +116,8 @@ def autotune(nx, ny, op, params, dtype=None, state=None, stream=None, probe_step
             h = handle(n)
             if h is None:
                 continue
+            if state is None:
+                state = _probe_state(h, op, [nx], [ny]).reshape(h.shape)
             ms = _time_advance(h, state, probe_steps, stream)
             probes.append((n, ms * 1e-3 / substeps))
         if not probes:
@@ -120,29 +131,39 @@ def autotune(nx, ny, op, params, dtype=None, state=None, stream=None, probe_step
             h = handle(n)
             if h is None:
                 continue
-            for t in threads:
-                for st in stages:
-                    try:
-                        h.set_tuning(t, st)
-                    except SweptError:
-                        continue
-                    ms = _time_advance(h, state, probe_steps, stream)
-                    table.append({"tile": n, "threads": t, "stage": bool(st), "ms": ms,
-                                  "gcell_per_s": N2 * probe_steps / (ms * 1e-3) / 1e9,
-                                  "predicted_ms": pred[n]})
+            _time_advance(h, state, probe_steps, stream)
+            march = _marches(h, probe_steps)
+            shapes = [(int(h.query("threads")), h.query("stage") != 0)] if march else \
+                [(t, st) for t in threads for st in stages]
+            for t, st in shapes:
+                try:
+                    h.set_tuning(t, st)
+                except SweptError:
+                    continue
+                ms = _time_advance(h, state, probe_steps, stream)
+                table.append({"tile": n, "threads": t, "stage": bool(st), "march": march, "ms": ms,
+                              "gcell_per_s": N2 * probe_steps / (ms * 1e-3) / 1e9,
+                              "predicted_ms": pred[n]})
     finally:
         for h in handles.values():
             if h is not None:
                 h.close()
     if not table:
         raise RuntimeError("no candidate could run")
-    best = min(table, key=lambda r: r["ms"])
+    best = _best(table)
     table.append({"model": "t(n) = N^2 s + 4 tau / n per sub-step (Section 4, eq. (cost))",
                   "s_ns_per_point_update": s_pt * 1e9, "tau_us": tau * 1e6,
                   "probes": [{"tile": n, "us_per_substep": t * 1e6} for n, t in probes],
                   "ranking": ranked, "timed_tiles": ranked[:top],
                   "predicted_ms": {str(n): pred[n] for n in valid}})
     return (best["tile"], best["threads"], best["stage"]), table
+
+
+def _best(rows):
+    """The fastest row; among tiles that all march, the largest tile's."""
+    if all(r["march"] for r in rows):
+        return max(rows, key=lambda r: r["tile"])
+    return min(rows, key=lambda r: r["ms"])
 
 
 def _torch_dtype(np_dtype):
@@ -157,25 +178,29 @@ def size_class(nx, ny, tiles=(16, 32, 64)):
     return tuple(n for n in tiles if nx % n == 0 and ny % n == 0)
 
 
-def _probe_state(b, op):
-    """A valid state for timing probes: zeros, or for the Euler updates a gas at
-    rest (rho = 1, E = 2.5) in every grid (zeros would divide by zero)."""
+def _probe_state(b, op, nx, ny):
+    """A valid state for timing probes, grids one after the other: values in [1, 2) in
+    every plane (binary64 heat of one sign can take the integer units, zeros cannot),
+    or for the Euler updates a gas at rest (rho = 1, E = 2.5)."""
     import numpy as np
     import torch
     dt = _torch_dtype(b.np_dtype)
-    if op not in ("euler_rk2", "euler_kahan"):
-        return torch.zeros(b.total, device="cuda", dtype=dt)
     parts = []
-    for a, c in zip(b.nx, b.ny):
-        U = np.zeros((b.nvars, c, a), np.float32)
-        U[0] = U[4] = 1.0
-        U[3] = U[7] = 2.5
+    for i, (a, c) in enumerate(zip(nx, ny)):
+        if op in ("euler_rk2", "euler_kahan"):
+            U = np.zeros((b.nvars, c, a), np.float32)
+            U[0] = U[4] = 1.0
+            U[3] = U[7] = 2.5
+        else:
+            U = 1.0 + np.random.default_rng(i).random((b.nvars, c, a))
+            if op == "heat_kahan":
+                U[1] = 0.0
         parts.append(U.reshape(-1))
     host = torch.from_numpy(np.concatenate(parts))
     if dt == torch.int16:                      # bfloat16 bits
         host = host.to(torch.bfloat16).view(torch.int16)
-    elif dt == torch.float64:
-        host = host.double()
+    else:
+        host = host.to(dt)
     return host.to("cuda")
 
 
@@ -232,13 +257,13 @@ def autotune_batch(nx, ny, op, params, dtype=None, state=None, stream=None, prob
                     batches[n] = None
             return batches[n]
 
-        best = None
+        best, rows = None, []
         try:
             probes = []
             for n in sorted({min(cand), max(cand)}):
                 b = batch(n)
                 if b is not None:
-                    probes.append((n, timed(b, _probe_state(b, op)) * 1e-3 / substeps))
+                    probes.append((n, timed(b, _probe_state(b, op, sub_nx, sub_ny)) * 1e-3 / substeps))
             if not probes:
                 continue
             s_pt, tau = fit_cost_model(cells, probes if len(probes) == 2 else probes * 2)
@@ -248,21 +273,24 @@ def autotune_batch(nx, ny, op, params, dtype=None, state=None, stream=None, prob
                 b = batch(n)
                 if b is None:
                     continue
-                zeros = _probe_state(b, op)
-                for t in threads:
-                    for st in stages:
-                        try:
-                            b.set_tuning(t, st)
-                        except SweptError:
-                            continue
-                        ms = timed(b, zeros)
-                        row = {"class": list(cand), "grids": len(members), "tile": n,
-                               "threads": t, "stage": st, "ms": ms,
-                               "gcell_per_s": cells * probe_steps / (ms * 1e-3) / 1e9,
-                               "predicted_ms": pred[n]}
-                        table.append(row)
-                        if best is None or ms < best["ms"]:
-                            best = row
+                probe = _probe_state(b, op, sub_nx, sub_ny)
+                b.set_state(probe)
+                launches = b.query("launches")
+                b.advance(probe_steps)
+                march = b.query("launches") - launches == 1      # (several in any other form)
+                for t, st in [(256, False)] if march else \
+                        [(t, st) for t in threads for st in stages]:
+                    try:
+                        b.set_tuning(t, st)
+                    except SweptError:
+                        continue
+                    ms = timed(b, probe)
+                    rows.append({"class": list(cand), "grids": len(members), "tile": n,
+                                 "threads": t, "stage": st, "march": march, "ms": ms,
+                                 "gcell_per_s": cells * probe_steps / (ms * 1e-3) / 1e9,
+                                 "predicted_ms": pred[n]})
+            table += rows
+            best = _best(rows) if rows else None
             table.append({"class": list(cand), "model": "t(n) = N^2 s + 4 tau / n per sub-step",
                           "s_ns_per_point_update": s_pt * 1e9, "tau_us": tau * 1e6,
                           "ranking": ranked, "predicted_ms": {str(n): pred[n] for n in cand}})

@@ -469,3 +469,21 @@ def test_traced_persistent_advance_of_the_updates_that_march(oracle_lib, op, dty
             s.advance(steps, mode="persistent", graph=graph)
             assert np.array_equal(s.get_state(), want)
     assert (buf.cpu().numpy().view(np.uint32).reshape(-1, 2)[:, 1] > 0).all()
+
+
+@pytest.mark.parametrize("op,dtype,params,march", [
+    ("heat", "f64", (0.2,), True), ("heat", "f64", (0.25,), False), ("heat_kahan", "bf16", (0.2,), True),
+    ("wave", "f64", (0.3,), False)])
+def test_autotune_times_one_launch_shape_of_a_form_that_ignores_it(op, dtype, params, march):
+    from paper_1602_07558_gb300.autotune import autotune, autotune_batch
+    (tile, threads, _), table = autotune(256, 256, op, params, dtype=dtype, tiles=(16, 32), threads=(128, 256))
+    rows = [r for r in table if "tile" in r]
+    assert all(r["march"] == march for r in rows)
+    assert len(rows) == 2 if march else len(rows) > 2
+    assert (tile, threads) == (32, 256) if march else tile in (16, 32)
+    if op != "wave":
+        tiles, tuning, table = autotune_batch([64] * 3, [64] * 3, op, params, dtype=dtype, tiles=(16, 32),
+                                              threads=(128, 256), probe_steps=16,
+                                              stream=torch.cuda.Stream())
+        assert [r["march"] for r in table if "tile" in r] == [True, True]   # (12,288 points)
+        assert tiles == [32] * 3 and list(tuning) == [32]
