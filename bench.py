@@ -415,6 +415,13 @@ WORK = {
 }
 
 
+# Marching FP64 heat (integer arithmetic): lane instructions of the ALU pipe for one
+# update, from the pipe's busy share and the duration of profiles/march_heat_2048.md
+# (0.686 of 152 SMs x 64 lanes x 2.07 GHz for 241 us and 50.3 M updates), and its peak.
+ALU_PEAK = 152 * 64 * 2.07e9
+ALU_PER_UPDATE = 0.686 * ALU_PEAK * 241e-6 / 50.3e6
+
+
 def hbm_peak():
     """(GB/s, source): MEASURED_PEAKS.json's copy rate, else the fallback."""
     try:
@@ -453,10 +460,10 @@ def bounds(w, esize, upd, hbm_bytes, seconds, peaks):
 
 def roofline(w, kern, peaks, esize, nvars):
     """Roofline of the dominant kernel (the octahedron, or the marching form's one
-    kernel, whose FP64 heat runs on the integer units and may pass the FP64
-    pipe's bound): its algorithmic
-    work per launch over its CUDA-event launch time against the slowest of the
-    HBM, FP64, FP32 and shared-memory bounds; the bridge's beside it."""
+    kernel): its algorithmic work per launch over its CUDA-event launch time
+    against the slowest of the HBM, FP64, FP32 and shared-memory bounds; the
+    bridge's beside it. Marching FP64 heat runs on the integer units instead of
+    the FP64 pipe: its bound is their ALU rate."""
     n, N = w.tile, w.grid
     launches, ms = kern.get("march", (0, 0.0))
     if launches:                       # the marching form: every step in one launch
@@ -466,6 +473,13 @@ def roofline(w, kern, peaks, esize, nvars):
         out = {"kernel": "march", "avg_launch_ms": ms / launches, "updates_per_launch": upd,
                "hbm_bytes_per_launch": hbm_bytes, "traffic": None, "traffic_source": None}
         out.update(bounds(w, esize, upd, hbm_bytes, ms / launches * 1e-3, peaks))
+        if (w.op, w.dtype) == ("heat", "f64"):
+            seconds = ms / launches * 1e-3
+            out.update({"bound": "int_alu", "achieved": ALU_PER_UPDATE * upd / seconds / 1e9,
+                        "peak": ALU_PEAK / 1e9, "unit": "Gop/s (integer ALU)",
+                        "frac": ALU_PER_UPDATE * upd / seconds / ALU_PEAK,
+                        "peak_source": "152 SMs x 64 lanes x 2.07 GHz; lane instructions an "
+                                       "update from ncu, redundant points included"})
         return out
     tiles = (N // n) ** 2
     launches, ms = kern["octahedron"]
@@ -837,8 +851,9 @@ def accuracy_report(w, sw, state_host, state_dev, out_sw, stream, Swept2D, full=
 
 
 def persistent_trace(sw, w, state_dev, stream, sm_mhz):
-    """One persistent advance with the per-item trace on: the mean SM cycles
-    (and microseconds at the sampled SM clock) a block waited for an item's
+    """One persistent advance of the swept kernels with the per-item trace on (an
+    update that marches takes them for a trace alone, so this is then not the timed
+    form): the mean SM cycles (and microseconds at the sampled SM clock) a block waited for an item's
     3 x 3 neighbourhood and spent on the item, per kind of item."""
     import torch
     n, N = w.tile, w.grid
@@ -861,7 +876,7 @@ def persistent_trace(sw, w, state_dev, stream, sm_mhz):
     last = NT + (H - 1) * 3 * NT + 2 * NT
     kind[last:] = "final_down"
     mhz = sm_mhz or 2070.0
-    out = {"sm_mhz_used": mhz, "items": int(items), "half_cycles": int(H)}
+    out = {"form": "persistent swept kernel", "sm_mhz_used": mhz, "items": int(items), "half_cycles": int(H)}
     for k in ("first_up", "bridge", "octahedron", "final_down"):
         sel = kind == k
         if sel.any():
