@@ -16,7 +16,8 @@
  * advance in the marching form where it is faster: one launch in which blocks
  * take tiles of their own choice through several steps in registers, computing a
  * ring around them redundantly (the same bits; the caller's tile side, threads
- * and staging then only decide what is accepted). A plain one-kernel-per-sub-step path (mode
+ * and staging then only decide what is accepted, and, for the updates in binary64,
+ * which form is the faster). Advances of a few sub-steps take naive launches. A plain one-kernel-per-sub-step path (mode
  * SWEPT2D_NAIVE) uses the same point-update code and gives bitwise identical
  * results. Many independent grids of uneven sizes share launches through the
  * swept2d_batch_* calls.
@@ -132,13 +133,15 @@ typedef struct swept2d swept2d_t;
 /* Batches only, OR-ed with SWEPT2D_SWEPT | SWEPT2D_PERSISTENT: one persistent
  * launch covers the half cycles of every tile class, instead of one persistent
  * launch per class. Its blocks (256 threads, shared memory for the largest
- * class) take the classes in order; the tile-16 and tile-32 classes run in
- * teams of warps (one small tile per team), larger ones one tile per block;
+ * class) take the classes in order; classes of tile sides up to 16 run in
+ * teams of two warps (one tile per team), larger ones one tile per block;
  * each class keeps its own tile side, half-cycle count, counters and item
  * counter. Staging follows swept2d_batch_set_tuning and is dropped if the
  * staged blocks do not fit; the thread count of that tuning is not used. Naive
  * tails (steps that do not fill a half cycle of a class) follow as before.
- * Same bits. EINVAL without SWEPT2D_PERSISTENT, for a single-grid handle, with
+ * Same bits. (A batch that takes the marching form has no classes to order: its
+ * one launch runs every step in any of these modes; what they refuse, they refuse.)
+ * EINVAL without SWEPT2D_PERSISTENT, for a single-grid handle, with
  * more than 16 classes, or if even unstaged blocks do not fit. */
 #define SWEPT2D_ONE_LAUNCH 0x400
 
@@ -153,7 +156,8 @@ typedef struct swept2d swept2d_t;
  *   params op parameters (see above); nparams their count.
  *   stream a cudaStream_t (NULL = legacy default stream).
  * Allocates the device state and, if tile > 0, two panel buffers of
- * 4 (n^2/2 + n) nvars elements per tile each. Errors: EINVAL (bad sizes, op
+ * 4 (n^2/2 + n) nvars elements per tile each (where both swept modes take the
+ * marching form, only once a traced persistent advance needs them). Errors: EINVAL (bad sizes, op
  * mismatch), ENOMEM, ECUDA. On error *out is NULL.
  */
 int swept2d_create(swept2d_t **out, int nx, int ny, int nvars, int nstages, int tile,
@@ -183,8 +187,9 @@ int swept2d_get_state(swept2d_t *h, void *dst, int dst_is_device);
 /*
  * Self-test of the persistent form's bounded waits (no counterpart in the
  * paper; Section 4's exchanges are the dependencies being waited for): runs the
- * persistent kernel for one half cycle with its first phase skipped, so the
- * phase counters those waits read are never released. Every block's wait gives
+ * kernel of the handle's persistent mode (the persistent kernel for one half cycle,
+ * or the marching one for two phases a stage) with its first phase skipped, so the
+ * counters those waits read are never released. Every block's wait gives
  * up after spin_limit polls (>= 1; each poll is a load plus a ~64 ns pause, so
  * a few thousand take milliseconds), records the timeout in the handle's error
  * word and returns. No work item runs, so the state is unchanged; the error
@@ -209,7 +214,8 @@ const char *swept2d_last_error(const swept2d_t *h);
 #define SWEPT2D_Q_SUBSTEPS      2   /* sub-steps advanced since set_state */
 #define SWEPT2D_Q_LAUNCHES      3   /* kernels launched by this handle since create */
 #define SWEPT2D_Q_STATE_BYTES   4   /* bytes of one state copy */
-#define SWEPT2D_Q_PANEL_BYTES   5   /* bytes of one panel buffer (0 if naive-only) */
+#define SWEPT2D_Q_PANEL_BYTES   5   /* bytes of one panel buffer (0 if naive-only), allocated
+                                       or not: a batch that marches never does */
 #define SWEPT2D_Q_SMEM_BYTES    6   /* dynamic shared memory per swept block */
 #define SWEPT2D_Q_CELLS         7   /* points of the grid (of all grids, for a batch) */
 #define SWEPT2D_Q_THREADS       8   /* swept threads per block (swept2d_set_tuning) */

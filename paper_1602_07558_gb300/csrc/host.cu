@@ -221,6 +221,16 @@ void free_all(swept2d *h) {
     h->sched = h->msched = nullptr;
 }
 
+cudaError_t allocate_panels(swept2d *h) {
+    if (h->up) return cudaSuccess;
+    cudaError_t e = cudaMalloc(&h->up, h->panel_bytes);
+    if (e == cudaSuccess && (e = cudaMalloc(&h->br, h->panel_bytes)) != cudaSuccess) {
+        cudaFree(h->up);
+        h->up = nullptr;
+    }
+    return e;
+}
+
 int naive_substeps(swept2d *h, long long count) {
     for (long long s = 0; s < count; ++s) {
         const u64 g = (u64)h->substeps;
@@ -466,14 +476,7 @@ int swept2d_create(swept2d_t **out, int nx, int ny, int nvars, int nstages, int 
         cuda_fail(h, e, "state allocation");
         return bail(e == cudaErrorMemoryAllocation ? SWEPT2D_ENOMEM : SWEPT2D_ECUDA);
     }
-    if (tile) {
-        h->panel_bytes = (size_t)h->G.T * h->G.Q * 4 * nvars * h->G.PS * t->esize;
-        if ((e = cudaMalloc(&h->up, h->panel_bytes)) != cudaSuccess ||
-            (e = cudaMalloc(&h->br, h->panel_bytes)) != cudaSuccess) {
-            cuda_fail(h, e, "panel allocation");
-            return bail(e == cudaErrorMemoryAllocation ? SWEPT2D_ENOMEM : SWEPT2D_ECUDA);
-        }
-    }
+    if (tile) h->panel_bytes = (size_t)h->G.T * h->G.Q * 4 * nvars * h->G.PS * t->esize;
     h->nt = march_for(op, dtype);
     if (h->nt) {
         h->nshape = h->nt->naive_shape(nx, ny, h->consts);
@@ -494,6 +497,11 @@ int swept2d_create(swept2d_t **out, int nx, int ny, int nvars, int nstages, int 
             cuda_fail(h, e, "schedule allocation");
             return bail(e == cudaErrorMemoryAllocation ? SWEPT2D_ENOMEM : SWEPT2D_ECUDA);
         }
+    }
+    // (a handle that marches in both swept modes has no use for panels but a trace's)
+    if (tile && !(h->marches[0] && h->marches[1]) && (e = allocate_panels(h)) != cudaSuccess) {
+        cuda_fail(h, e, "panel allocation");
+        return bail(e == cudaErrorMemoryAllocation ? SWEPT2D_ENOMEM : SWEPT2D_ECUDA);
     }
     if ((e = cudaMalloc(&h->scratch8, sizeof(unsigned long long))) != cudaSuccess ||
         (e = cudaMalloc(&h->errword, sizeof(int))) != cudaSuccess ||
@@ -546,7 +554,8 @@ int swept2d_set_state(swept2d_t *h, const void *src, int src_is_device) {
 
 // Checks and scratch of the persistent form for H half cycles: the staged
 // shared-memory plan must fit, the work items must fit an int, and the phase
-// counters (T*Q + 1 ints) are allocated on first use.
+// counters (T*Q + 1 ints), with the panels where a handle that marches is traced,
+// are allocated on first use.
 static int persistent_prepare(swept2d *h, long long H) {
     int dev = 0, optin = 0;
     cudaGetDevice(&dev);
@@ -559,6 +568,10 @@ static int persistent_prepare(swept2d *h, long long H) {
     if (!h->sched) {
         cudaError_t e = cudaMalloc(&h->sched, ((size_t)h->G.T * h->G.Q + 1) * sizeof(int));
         if (e != cudaSuccess) return cuda_fail(h, e, "persistent schedule allocation");
+    }
+    if (h->trace || !h->marches[1]) {
+        const cudaError_t e = allocate_panels(h);
+        if (e != cudaSuccess) return cuda_fail(h, e, "panel allocation");
     }
     return SWEPT2D_OK;
 }

@@ -54,7 +54,8 @@ struct Geom {
 };
 
 // How the marching form (march.cuh) cuts a grid: bx x by tiles, tile i of a
-// side of n points covering [i n / b, (i + 1) n / b).
+// side of n points covering [i n / b, (i + 1) n / b), along x from the even column
+// at or before it on.
 struct MarchGrid {
     int nx, ny, bx, by;
 };
