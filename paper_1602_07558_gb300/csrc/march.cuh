@@ -911,9 +911,9 @@ inline double euler_march_cost(int shape, const int *nx, const int *ny, int coun
         return cudaSuccess;
     });
     static const double alone[] = {169.6, 88.6, 28.5, 17.4}, each[] = {1.05, 0.537, 0.1585, 0.047},
-                        spread[] = {75, 75, 75, 306};
-    double crowd = 1.0 + (tiles - 76) / spread[shape];
-    crowd = crowd < 1.0 ? 1.0 : crowd > 2.7 ? 2.7 : crowd;
+                        shared[] = {1.42, 1.42, 1.42, 1}, spread[] = {150, 150, 150, 306};
+    double crowd = tiles <= 76 ? 1.0 : shared[shape] + (tiles - 76) / spread[shape];
+    if (crowd > 2.7) crowd = 2.7;
     const double one = alone[shape] * crowd, all = each[shape] * full;
     return one > all ? one : all;
 }
@@ -928,7 +928,7 @@ inline double euler_swept_cost(int n, double tiles, bool persistent) {
     double t = 17.3 + 0.00442 * std::pow((double)n, 2.6);
     const double wave = n >= 20 ? 0.6 + 0.01 * n : 0.38 + 0.0225 * n;   // of each after the first
     if (persistent && tiles > 200)                // (13 µs a wave at n = 8, 17.5, 47.5 at n = 32)
-        return (t - 5.3) * (n >= 20 ? std::ceil(tiles / 152) : tiles / 152 + 0.2);
+        return (t - 5.3) * (n >= 20 ? std::ceil(tiles / 152) - 0.15 : tiles / 152 + 0.2);
     const double more = (double)(((long long)tiles - 1) / 152);
     if (n >= 20)
         t *= tiles <= 100 ? 0.88 : 1.0 + wave * (more == 1 ? 0.93 : more);
