@@ -368,7 +368,8 @@ int swept2d_batch_query_grid(const swept2d_batch_t *b, int grid, int what, doubl
  * Errors: SWEPT2D_EINVAL (bad sizes or pointers, grid too large for the
  * scratch), SWEPT2D_ECUDA; a message goes to err (errlen bytes, may be NULL).
  * The call has returned by the time a kernel's bounded neighbourhood wait could
- * give up (a handle's SWEPT2D_ETIMEOUT): u_out is then NaN at every point.
+ * give up (a handle's SWEPT2D_ETIMEOUT): u_out is then NaN, but where blocks in the
+ * middle of a tile still wrote theirs, and so in at least one tile.
  */
 #define SWEPT2D_STATIC_SCRATCH_BYTES ((size_t)32 << 20)
 int swept2d_heat_advance_static(const double *u_in, double *u_out, int nx, int ny, int tile,

@@ -19,7 +19,7 @@
 // large is recorded, and the caller repeats the block's steps by the FP64
 // operations; blocks on a zero crossing, or with values more than a factor of 32
 // to 64 apart, take them from the start. Measured on the GB300: 4096², 500 steps,
-// 36.5 ms with this (the integer ALU 68% busy), 67.4 by the FP64 operations of the
+// 35.4 ms with this (the integer ALU 68% busy), 67.4 by the FP64 operations of the
 // swept kernels (their pipe 95% busy). On the host the same functions serve to compare
 // them with the FP64 operations.
 #pragma once

@@ -102,9 +102,9 @@ __device__ __forceinline__ bool march_wait(const MarchTile &m, const int *done, 
     return __syncthreads_or(bad) == 0;
 }
 
-// The items of a run, taken until none is left (or a wait gave up).
+// The items of a run, taken until none is left; false if a wait gave up.
 template <class Body, class Op, class Loc>
-__device__ __forceinline__ void march_items(const Op &op, const Loc &at,
+__device__ __forceinline__ bool march_items(const Op &op, const Loc &at,
                                             const MarchRun<typename Op::S> &run,
                                             typename Body::Smem &sm, int &s_item) {
     typedef typename Op::S S;
@@ -116,10 +116,10 @@ __device__ __forceinline__ void march_items(const Op &op, const Loc &at,
         }
         __syncthreads();
         const int item = s_item;
-        if (item >= nitems) return;
+        if (item >= nitems) return true;
         const int j = item / run.NT, t = item - j * run.NT;
         const MarchTile m = at(t);
-        if (!march_wait(m, run.done, j, run.err, run.spin_limit)) return;
+        if (!march_wait(m, run.done, j, run.err, run.spin_limit)) return false;
         const S *src = (j == 0 ? run.src : run.buf[(j - 1) & 1]) + m.soff;
         Body::run(m.c ? Op(m.c) : op, m, src, run.buf[j & 1] + m.soff, run.K,
                   j + 1 == run.phases ? run.last : run.K, j, sm);
@@ -139,24 +139,18 @@ march_kernel(Op op, Loc at, MarchRun<typename Op::S> run) {
     march_items<Body>(op, at, run, sm, s_item);
 }
 
-// The same for a caller that cannot ask for the error word: the block that leaves
-// last overwrites the result, `points` values, with NaN if a wait gave up.
+// The same for a caller that cannot ask for the error word: a block whose wait gives
+// up overwrites the `points` values of the result with NaN. (Its own tile stays so,
+// as no phase of it follows; blocks in the middle of theirs may still write those.)
 template <class Body, class Op, class Loc, bool AFTER>
 __global__ void __launch_bounds__(Body::kThreads, Body::kMinBlocks)
-march_or_spoil_kernel(Op op, Loc at, MarchRun<double> run, unsigned *left, size_t points) {
+march_or_spoil_kernel(Op op, Loc at, MarchRun<double> run, double *result, size_t points) {
     __shared__ typename Body::Smem sm;
     __shared__ int s_item;
     if constexpr (AFTER) after_previous_launch();
-    march_items<Body>(op, at, run, sm, s_item);
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0)
-        s_item = atomicAdd(left, 1u) + 1 == gridDim.x && ld_acquire(run.err) != 0;
-    __syncthreads();
-    if (!s_item) return;
-    double *u = run.buf[(run.phases - 1) & 1];
+    if (march_items<Body>(op, at, run, sm, s_item)) return;
     for (size_t i = threadIdx.x; i < points; i += Body::kThreads)
-        u[i] = __longlong_as_double(0x7ff8000000000000LL);
+        result[i] = __longlong_as_double(0x7ff8000000000000LL);
 }
 
 // One phase, one tile a block: the naive path's launch per sub-step (Euler in place,
@@ -1123,11 +1117,11 @@ inline bool march_short(int shape, int nx, int ny, int tile, long long substeps)
     }
 }
 
-// One launch of a run whose counters are set; with `left` (a zero), the result is
-// spoiled where a wait gives up.
+// One launch of a run whose counters are set; with `spoil`, the advance's result, that
+// becomes NaN where a wait gives up.
 template <class B, bool AFTER, class Op, class Loc>
 inline cudaError_t march_launch(const Op &op, const Loc &at, const MarchRun<typename Op::S> &run,
-                                unsigned *left, size_t points, cudaStream_t st) {
+                                void *spoil, size_t points, cudaStream_t st) {
     const auto launch = [&](auto *kern, auto... more) {
         int per_sm = 0, dev = 0, nsm = 0;
         const cudaError_t e =
@@ -1144,14 +1138,15 @@ inline cudaError_t march_launch(const Op &op, const Loc &at, const MarchRun<type
         return cudaGetLastError();
     };
     if constexpr (std::is_base_of<HeatOp, Op>::value && std::is_same<Loc, OneMarch>::value)
-        if (left) return launch(&march_or_spoil_kernel<B, Op, Loc, AFTER>, left, points);
+        if (spoil)
+            return launch(&march_or_spoil_kernel<B, Op, Loc, AFTER>, (double *)spoil, points);
     return launch(&march_kernel<B, Op, Loc, AFTER>);
 }
 
 // Queues `steps` steps over NT tiles: reads `src`, writes b0, b1, b0, ... phase
 // by phase (src may be b1). sched: NT counters and the item counter; without `err`
-// (one heat grid) two words more precede them, the error word and a count, both
-// cleared with them, and a result of `points` values becomes NaN where a wait gives
+// (one heat grid) the word before them is the error word and is cleared with them,
+// and the result, which `*out` then names beforehand, becomes NaN where a wait gives
 // up. `launches` is raised by the launches made, `*out` set to the buffer with the
 // result.
 template <class Op, class Loc>
@@ -1168,12 +1163,8 @@ inline cudaError_t march_advance(int shape, const Op &op, const Loc &at, int NT,
         // (an even number of phases: the stages of Euler alternate)
         const long long most = (((1LL << 30) - 1) / NT + 2) & ~1LL;
         int *clear = sched;
-        unsigned *blocks_left = nullptr;
-        if (!err) {
-            err = sched;
-            blocks_left = (unsigned *)sched + 1;
-            sched += 2;
-        }
+        void *const spoil = err ? nullptr : *out;
+        if (!err) err = sched++;
         while (steps > 0) {
             const long long left = (steps + K - 1) / K;
             MarchRun<S> run;
@@ -1191,8 +1182,8 @@ inline cudaError_t march_advance(int shape, const Op &op, const Loc &at, int NT,
             run.spin_limit = spin_limit;
             cudaError_t e = cudaMemsetAsync(clear, 0, (sched + NT + 1 - clear) * sizeof(int), st);
             if (e != cudaSuccess) return e;
-            clear = blocks_left ? sched - 1 : sched;
-            if ((e = march_launch<B, false>(op, at, run, blocks_left, points, st)) != cudaSuccess)
+            clear = sched;
+            if ((e = march_launch<B, false>(op, at, run, spoil, points, st)) != cudaSuccess)
                 return e;
             *launches += 1;
             steps -= (long long)(run.phases - 1) * K + run.last;
@@ -1274,7 +1265,7 @@ __global__ void __launch_bounds__(256) heat_survey_kernel(Op op, MarchGrid g, co
 // Counters of the two forms, with the survey's and the error word's.
 template <class Op>
 inline long long march_words(int shape, int nx, int ny) {
-    long long words = march_tiles<Op>(shape, &nx, &ny, 1) + 3;
+    long long words = march_tiles<Op>(shape, &nx, &ny, 1) + 2;
     if constexpr (std::is_same<Op, HeatOp>::value)
         words += march_tiles<HeatWalkOp>(heat_walk_shape(nx, ny), &nx, &ny, 1) + 2;
     return words;
@@ -1302,12 +1293,9 @@ inline cudaError_t heat_either_advance(int shape, const MarchGrid &g, const Heat
     const MarchGrid wg = march_cut<HeatWalkOp>(ws, g.nx, g.ny);
     const int NT = g.bx * g.by, WT = wg.bx * wg.by, K = march_steps<HeatOp>(shape);
     int *clear = sched;
-    unsigned *blocks_left = nullptr;
-    if (!err) {
-        err = sched;
-        blocks_left = (unsigned *)sched + 1;
-        sched += 2;
-    }
+    void *const spoil = err ? nullptr : *out;
+    const size_t points = (size_t)g.nx * g.ny;
+    if (!err) err = sched++;
     int *const walk_sched = sched + NT + 1, *const count = walk_sched + WT + 1;
     while (steps > 0) {
         const int n = steps < kEitherSteps ? (int)steps : kEitherSteps;
@@ -1333,19 +1321,19 @@ inline cudaError_t heat_either_advance(int shape, const MarchGrid &g, const Heat
         walked.last = n + 1 - walked.phases;
         cudaError_t e = cudaMemsetAsync(clear, 0, (count + 1 - clear) * sizeof(int), st);
         if (e != cudaSuccess) return e;
-        clear = blocks_left ? sched - 1 : sched;
+        clear = sched;
         heat_survey_kernel<HeatOp><<<NT < 304 ? NT : 304, 256, 0, st>>>(
             op, g, run.src, n >= 8, (unsigned *)count, run.queue, NT * run.phases, walked.queue,
             WT * walked.phases);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         e = with_march_shape<HeatOp>(shape, [&](auto *body) {
             return march_launch<typename std::remove_pointer<decltype(body)>::type, true>(
-                op, OneMarch{g}, run, nullptr, 0, st);
+                op, OneMarch{g}, run, spoil, points, st);
         });
         if (e != cudaSuccess) return e;
         e = with_march_shape<HeatWalkOp>(ws, [&](auto *body) {
             return march_launch<typename std::remove_pointer<decltype(body)>::type, true>(
-                walk, OneMarch{wg}, walked, blocks_left, (size_t)g.nx * g.ny, st);
+                walk, OneMarch{wg}, walked, spoil, points, st);
         });
         if (e != cudaSuccess) return e;
         *launches += 3;

@@ -13,7 +13,7 @@ struct MarchTable {
                  const double *c);
     int (*steps)(int shape);     // steps a phase
     MarchGrid (*cut)(int shape, int nx, int ny);
-    // ints of the counters that `one` needs, its own error words included
+    // ints of the counters that `one` needs, its own error word included
     long long (*words)(int shape, int nx, int ny);
     // whether an advance of so few sub-steps of one grid is quicker by naive launches
     bool (*is_short)(int shape, int nx, int ny, int tile, long long substeps);
@@ -21,7 +21,7 @@ struct MarchTable {
     // one grid, -1 for a thread a point
     int (*naive_shape)(int nx, int ny, const double *c);
     // one grid (`g` its cut), or the tiles of a batch's table; without `err` (heat
-    // alone) the result becomes NaN where a wait gives up
+    // alone) the result, which *out names beforehand, becomes NaN where a wait gives up
     cudaError_t (*one)(int shape, const MarchGrid &g, const double *c, const void *src, void *b0,
                        void *b1, int *sched, long long steps, int *err, int first,
                        long long spin_limit, void **out, long long *launches, cudaStream_t);

@@ -15,7 +15,7 @@
 // so the result is bit for bit that of a handle created with op SWEPT2D_OP_HEAT and
 // advanced with SWEPT2D_SWEPT from the same input. The call has returned before a
 // wait of the marching form could give up, and its caller has no handle to ask: the
-// last block to leave then overwrites u_out with NaN.
+// block then overwrites u_out with NaN.
 #include <cuda_runtime.h>
 
 #include <cstdio>
@@ -185,7 +185,7 @@ int advance_static(const double *u_in, double *u_out, int nx, int ny, int tile, 
     if (skip) nsteps = 2LL * mt->steps(shape);
     const long long phases = (nsteps + mt->steps(shape) - 1) / mt->steps(shape);
     void *b0 = (phases & 1) ? (void *)u_out : tmp, *b1 = (phases & 1) ? tmp : (void *)u_out;
-    void *out = nullptr;
+    void *out = u_out;
     long long made = 0;
     e = mt->one(shape, cut, consts, u_in, b0, b1, sched, nsteps, nullptr,
                 skip ? tiles : 0, spin_limit, &out, &made, st);
