@@ -80,6 +80,7 @@ struct swept2d {
     long long launches = 0;
     bool has_state = false;
     bool timing = false;
+    bool capturing = false;                      // the advance is being captured as a graph
     std::vector<TimedLaunch> timed;
     std::vector<cudaEvent_t> event_pool;
     std::vector<GraphEntry> graphs;
@@ -274,7 +275,7 @@ int swept_substeps(swept2d *h, long long total, bool persistent) {
         // launches to choose from, whichever form the longer advances take)
         const bool any = h->op == SWEPT2D_OP_EULER_RK2 && total < half;
         if ((any || h->marches[persistent]) &&
-            h->mt->is_short(h->mshape, h->nx, h->ny, h->n, total))
+            h->mt->is_short(h->mshape, h->nx, h->ny, h->n, total, h->capturing))
             return naive_substeps(h, total);
         if (any || h->marches[persistent])
             return march_substeps(h, total, 0, swept::kPersistSpinLimit);
@@ -358,7 +359,9 @@ int graph_advance(swept2d *h, long long nsteps, int mode) {
         h->timing = timing;
         return cuda_fail(h, e, "graph capture begin");
     }
+    h->capturing = true;
     int rc = run_advance(h, nsteps * h->nst, mode);
+    h->capturing = false;
     cudaGraph_t graph = nullptr;
     e = cudaStreamEndCapture(h->stream, &graph);
     h->timing = timing;

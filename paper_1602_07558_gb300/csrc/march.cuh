@@ -1089,7 +1089,8 @@ inline int naive_shape(int nx, int ny, const double *c) {
 // then has alone (a batch's naive launches take a thread a point: it marches). Measured on the GB300, us by the stream, naive launches / marching:
 //   heat binary64: 256 x 256, 2 steps 10.9 / 12.9, 4: 19.1 / 19.0; 768 x 768, 2: 22 / 27,
 //     4: 43 / 40 (with the survey 47, mixed signs 45 / 46); 2048 x 2048, 2: 46 / 74, 6: 140 / 157 (mixed signs 251 / 290), 16: 370 /
-//     371; 4096 x 4096, 6: 510 / 514 (mixed signs 836 / 1090)
+//     371; 4096 x 4096, 6: 510 / 514 (mixed signs 836 / 1090); in a graph (uniform noise) 64 x
+//     384, 7: 59 / 65 with the state's copies
 //   heat binary32: 256 x 256, 1 step 5.4 / 10.3, 2: 9.8 / 9.9, 3: 14.4 / 9.8; 2048 x 2048, 1:
 //     15.9 / 33, 2: 28 / 33, 3: 41 / 33
 //   Euler binary32: 256 x 256, 1 step 11.9 / 15.8, 2: 20.3 / 22.2, 3: 28.6 / 28.8; in a
@@ -1099,9 +1100,10 @@ inline int naive_shape(int nx, int ny, const double *c) {
 //     the swept form would not fill either): 80 x 320, 3 steps 76 / 104; 384 x 192, 3: 126 /
 //     147; 64 x 64, 1: 24 / 21
 template <class Op>
-inline bool march_short(int shape, int nx, int ny, int tile, long long substeps) {
+inline bool march_short(int shape, int nx, int ny, int tile, long long substeps, bool graph) {
     if constexpr (std::is_same<Op, HeatOp>::value) {
         const double points = (double)nx * ny;
+        if (graph && substeps <= 12 && substeps < tile / 2 && points < 1e6) return true;
         return substeps <= 3 || (substeps <= 5 && points >= 5e5) || (substeps <= 6 && points >= 2e6);
     } else if constexpr (std::is_same<Op, EulerOp>::value) {
         if (substeps >= tile / 2) return false;

@@ -16,7 +16,8 @@ struct MarchTable {
     // ints of the counters that `one` needs, its own error word included
     long long (*words)(int shape, int nx, int ny);
     // whether an advance of so few sub-steps of one grid is quicker by naive launches
-    bool (*is_short)(int shape, int nx, int ny, int tile, long long substeps);
+    // (made one by one or from a graph)
+    bool (*is_short)(int shape, int nx, int ny, int tile, long long substeps, bool graph);
     // the shape whose walks (phase_one) are the quickest for the naive sub-steps of
     // one grid, -1 for a thread a point
     int (*naive_shape)(int nx, int ny, const double *c);

@@ -169,7 +169,7 @@ int advance_static(const double *u_in, double *u_out, int nx, int ny, int tile, 
         if (e != cudaSuccess) set_err(err, errlen, cudaGetErrorString(e));
         return e == cudaSuccess ? SWEPT2D_OK : SWEPT2D_ECUDA;
     }
-    if (!skip && mt->is_short(shape, nx, ny, tile, nsteps)) {
+    if (!skip && mt->is_short(shape, nx, ny, tile, nsteps, false)) {
         // naive launches, the last of which lands in u_out
         const void *src = u_in;
         for (long long i = 0; i < nsteps && e == cudaSuccess; ++i) {
