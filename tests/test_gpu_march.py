@@ -487,3 +487,30 @@ def test_autotune_times_one_launch_shape_of_a_form_that_ignores_it(op, dtype, pa
                                               stream=torch.cuda.Stream())
         assert [r["march"] for r in table if "tile" in r] == [True, True]   # (12,288 points)
         assert tiles == [32] * 3 and list(tuning) == [32]
+
+
+@pytest.mark.parametrize("nx,ny", [(1, 500_001), (2, 300_001), (3, 200_001), (61, 9_001), (62, 9_000),
+                                   (63, 8_999), (125, 4_001), (9_001, 61)])
+def test_fp64_walks_on_narrow_and_odd_grids(oracle_lib, nx, ny):
+    """The naive walks of an r off the integer units: fewer columns than lanes, tiles
+    of the most and the fewest columns, odd sides."""
+    u0 = 2 * np.random.default_rng(nx).random((ny, nx)) - 1
+    with Swept2D(nx, ny, op="heat", tile=0, params=(0.25,), stream=torch.cuda.Stream()) as s:
+        for graph in (False, True):
+            s.set_state(u0[None])
+            s.advance(5, mode="naive", graph=graph)
+            assert np.array_equal(s.get_state()[0], oracle_lib.heat(u0, 0.25, 5))
+
+
+@pytest.mark.parametrize("kind", ["signed", "uniform", "one_sign"])
+@pytest.mark.parametrize("nx,ny,tile,nsteps", [(8, 65_536, 8, 8), (65_536, 8, 8, 13), (56, 9_184, 8, 9)])
+def test_static_advance_of_large_narrow_grids(oracle_lib, kind, nx, ny, tile, nsteps):
+    """Whose form the field decides, with fewer columns or rows than a tile has."""
+    from paper_1602_07558_gb300.swept2d import heat_advance_static
+    u0 = np.random.default_rng(ny).random((ny, nx))
+    u0 = {"signed": 2 * u0 - 1, "uniform": u0, "one_sign": -1 - u0}[kind]
+    d_in = torch.from_numpy(u0).to("cuda")
+    d_out = torch.zeros_like(d_in)
+    heat_advance_static(d_in, d_out, nx, ny, tile, 0.2, nsteps, stream=torch.cuda.current_stream())
+    torch.cuda.synchronize()
+    assert np.array_equal(d_out.cpu().numpy(), oracle_lib.heat(u0, 0.2, nsteps))
